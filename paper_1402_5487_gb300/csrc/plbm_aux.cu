@@ -591,31 +591,6 @@ __global__ void k_set_pop(const __grid_constant__ LatticeParams P, const double*
         default: return cudaErrorInvalidValue;                           \
     }
 
-// Initial fields are checked on the device before the state is built from them:
-// a non-finite value sets PLBM_STATUS_NONFINITE, rho <= 0 PLBM_STATUS_RHO_NONPOS,
-// theta <= 0 PLBM_STATUS_THETA_NONPOS.  One atomic per warp that found any.
-__global__ void k_check_fields(FieldSet F, long long n, unsigned* __restrict__ status) {
-    unsigned bits = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        for (int k = 0; k < F.count; ++k) {
-            const double v = F.field[k][i];
-            if (!isfinite(v)) bits |= PLBM_STATUS_NONFINITE;
-            else if (k == F.rho && !(v > 0.0)) bits |= PLBM_STATUS_RHO_NONPOS;
-            else if (k == F.theta && !(v > 0.0)) bits |= PLBM_STATUS_THETA_NONPOS;
-        }
-    }
-    bits = __reduce_or_sync(0xffffffffu, bits);
-    if ((threadIdx.x & 31) == 0 && bits) atomicOr(status, bits);
-}
-
-cudaError_t launch_check_fields(const FieldSet& F, long long n, unsigned* status, cudaStream_t stream) {
-    if (n <= 0 || F.count <= 0) return cudaSuccess;
-    const long long blocks = (n + 255) / 256;
-    k_check_fields<<<(int)(blocks < 4096 ? blocks : 4096), 256, 0, stream>>>(F, n, status);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_init(int prec, const LatticeParams& P, const double* rho, const double* ux,
                         const double* uy, const double* theta, void* f, cudaStream_t stream, int y0, int y1) {
     if (y1 < 0) y1 = P.ny;

@@ -577,19 +577,6 @@ plbm_status plbm_destroy(plbm_handle hh) {
     return PLBM_OK;
 }
 
-static plbm::FieldSet field_set(const double* const* d, int nd) {
-    plbm::FieldSet F{};
-    F.rho = -1;
-    F.theta = -1;
-    for (int k = 0; k < nd; ++k) {
-        if (!d[k]) continue;
-        if (k == 0) F.rho = F.count;
-        if (k == nd - 1) F.theta = F.count;
-        F.field[F.count++] = d[k];
-    }
-    return F;
-}
-
 // After a synchronous (host-pointer) init: PLBM_E_ARG if the field check set a
 // status bit; the handle is then left uninitialised.
 static plbm_status init_fields_verdict(Handle* h) {
@@ -844,9 +831,9 @@ plbm_status plbm_init3(plbm_handle hh, const double* rho, const double* ux, cons
         }
     }
     h->cur = 0;
-    CK(plbm::launch_init3(h->prec, h->P, d[0], d[1], d[2], d[3], d[4], h->f[0], h->stream));
+    // as in plbm_init: the initialisation kernel sets the status bits as it reads the fields
     CK(cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream));
-    CK(plbm::launch_check_fields(field_set(d, 5), (long long)n, h->status, h->stream));
+    CK(plbm::launch_init3(h->prec, h->P, d[0], d[1], d[2], d[3], d[4], h->f[0], h->stream));
     h->steps = 0;
     h->initialised = true;
     return on_device ? PLBM_OK : init_fields_verdict(h);

@@ -242,14 +242,6 @@ cudaError_t launch_init(int prec, const LatticeParams& P, const double* rho, con
 cudaError_t launch_moments(int prec, const LatticeParams& P, const void* f, double* rho,
                            double* ux, double* uy, double* theta, cudaStream_t stream, int y0 = 0,
                            int y1 = -1);
-// Up to five FP64 field arrays of n values; rho and theta index the fields that
-// must be positive (-1: none).  Null pointers are not allowed in field[0..count).
-struct FieldSet {
-    const double* field[5];
-    int count, rho, theta;
-};
-// Sets PLBM_STATUS_* bits in *status for non-finite values, rho <= 0, theta <= 0.
-cudaError_t launch_check_fields(const FieldSet& F, long long n, unsigned* status, cudaStream_t stream);
 // Three-dimensional lattices (plbm_step3.cu): storage [q][nz][ny][pitch].
 long long reduce3_blocks(const LatticeParams& P);
 cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void* dst, cudaStream_t s);

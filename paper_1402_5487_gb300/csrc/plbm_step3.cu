@@ -35,8 +35,8 @@
 // nodes as the lanes of packed FP32x2 instructions.  Pull across the z wrap:
 // node z = r reads z - v_z; when r - v_z leaves [0, nz/2) the source pair row is
 // r - v_z -+ nz/2 and holds the two nodes in swapped lane order.
-// k_stream_collide3_f64: FP64 storage of f, any q1 <= 5, thermal or isothermal,
-// the plain formulas (an ALU-bound path).
+// k_stream_collide3_f64q<Q1>: FP64 storage of f, q1 = 3, 4 or 5, thermal or
+// isothermal, the plain formulas (an ALU-bound path).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -483,20 +483,7 @@ __global__ void __launch_bounds__(kZpairBlock) k_stream_collide3_zpair(const __g
         zpair_update<S, false>(P, s32, d32, x, y, r);
 }
 
-// FP64: any q1 <= 5; fin[p] pulled, moments, f^eq from C and the Gaussian moments.
-__device__ void rule_f64(const LatticeParams& P, double u, double th, double* r) {
-    double mu[kMaxQ1];
-    const int q1 = P.q1;
-    mu[0] = 1.0;
-    mu[1] = u;
-    for (int n = 1; n + 1 < q1; ++n) mu[n + 1] = u * mu[n] + (double)n * th * mu[n - 1];
-    for (int i = 0; i < q1; ++i) {
-        double s = 0.0;
-        for (int n = 0; n < q1; ++n) s += P.C[i * q1 + n] * mu[n];
-        r[i] = s;
-    }
-}
-
+// FP64, any q1 <= 5: moments of a node from its populations.
 __device__ void moments3_f64(const LatticeParams& P, const double* f, double* m) {
     const int q1 = P.q1;
     double m0 = 0.0, mx = 0.0, my = 0.0, mz = 0.0, en = 0.0;
@@ -522,53 +509,17 @@ __device__ void moments3_f64(const LatticeParams& P, const double* f, double* m)
     m[8] = en;
 }
 
-__device__ void feq3_f64(const LatticeParams& P, double rho, double ux, double uy, double uz, double th,
-                         double* out) {
-    double ra[kMaxQ1], rb[kMaxQ1], rc[kMaxQ1];
-    rule_f64(P, ux, th, ra);
-    rule_f64(P, uy, th, rb);
-    rule_f64(P, uz, th, rc);
-    const int q1 = P.q1;
-    for (int a = 0; a < q1; ++a)
-        for (int b = 0; b < q1; ++b)
-            for (int c = 0; c < q1; ++c) out[(a * q1 + b) * q1 + c] = rho * ra[a] * rb[b] * rc[c];
-}
-
 __device__ __forceinline__ double w0_3(const LatticeParams& P, int p) {
     const int q1 = P.q1;
     const int a = p / (q1 * q1), b = (p / q1) % q1, c = p % q1;
     return P.w1[a] * P.w1[b] * P.w1[c];
 }
 
-__global__ void __launch_bounds__(kB3) k_stream_collide3_f64(const __grid_constant__ LatticeParams P,
-                                                             const double* __restrict__ src,
-                                                             double* __restrict__ dst) {
-    const int x = blockIdx.x * kB3 + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
-    if (x >= P.nx) return;
-    const int q1 = P.q1;
-    double fin[kQ3], fe[kQ3], m[9];
-    for (int a = 0; a < q1; ++a)
-        for (int b = 0; b < q1; ++b)
-            for (int c = 0; c < q1; ++c) {
-                const int p = (a * q1 + b) * q1 + c;
-                const long long row = ((long long)wrap_add(z, P.vzm[c], P.nz) * P.ny + wrap_add(y, P.vym[b], P.ny)) *
-                                      P.pitch;
-                fin[p] = src[(long long)p * P.plane + row + wrap_add(x, P.vxm[a], P.nx)];
-            }
-    moments3_f64(P, fin, m);
-    flag_status<double>(P, m[0], m[4]);
-    feq3_f64(P, m[0], m[1], m[2], m[3], P.isothermal ? P.theta0 : m[4], fe);
-    const long long here = ((long long)z * P.ny + y) * P.pitch + x;
-    const double om = P.omega;
-    for (int p = 0; p < q1 * q1 * q1; ++p) dst[(long long)p * P.plane + here] = (1.0 - om) * fin[p] + om * fe[p];
-}
-
-// FP64, compile-time q1 (3 or 5), in two passes over the pulled values so that
+// FP64, compile-time q1 (3 to 5), in two passes over the pulled values so that
 // no thread holds all q1^3 of them: the first forms the row sums
 // R_ab = sum_c f, S_a, T_b, U_c; the second loads them again (L1/L2 hits) and
-// writes f' = (1 - omega) f + (omega rho r^x_a r^y_b) r^z_c.  The same formulas
-// as k_stream_collide3_f64 (moments, C mu rule), with the sums factorised.
+// writes f' = (1 - omega) f + (omega rho r^x_a r^y_b) r^z_c (moments and the
+// C mu rule of Eq. eq:rdr, with the sums factorised).
 __device__ __forceinline__ double ldg_again(const double* p) {
     double v;
     asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
@@ -662,37 +613,425 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
         }
 }
 
-template <typename S>
-__global__ void k_init3(const __grid_constant__ LatticeParams P, const double* __restrict__ rho,
-                        const double* __restrict__ ux, const double* __restrict__ uy, const double* __restrict__ uz,
-                        const double* __restrict__ theta, S* __restrict__ f) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
-    if (x >= P.nx) return;
-    const long long n = ((long long)z * P.ny + y) * P.nx + x;
-    const double th = (P.isothermal || theta == nullptr) ? P.theta0 : theta[n];
-    double fe[kQ3];
-    feq3_f64(P, rho[n], ux ? ux[n] : 0.0, uy ? uy[n] : 0.0, uz ? uz[n] : 0.0, th, fe);
-    const long long here = node3(P, x, y, z);
-    for (int p = 0; p < P.q; ++p) f[(long long)p * P.plane + here] = Storage<S>::from_f64(fe[p], w0_3(P, p));
+// ---------------------------------------------------------------------------
+// Initial state and output fields.
+//
+// 16/32-bit storage (symmetric five-velocity thermal sets): FP64-grade results on
+// the FP32 pipe.  GB300 retires two FP64 operations per SM and cycle, so FP64
+// arithmetic over 125 populations per node (held in local memory) took 2,509 us
+// (initial state) and 5,152 us (fields) for 128^3 FP32 nodes and 9,989 / 20,554 us
+// for 256 x 256 x 128 FP16 nodes.  Float-float pairs hi + lo (error-free sums and
+// products, ~2^-47 relative) on the deviations from the rest state, whose magnitude
+// is a hundredth of f's (so the absolute error stays at FP64's on f), take 404 / 241 us
+// and 1,234 / 812 us, bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
+// the z-paired layout a thread takes both nodes of a pair (V = float2: packed FP32x2
+// arithmetic, one aligned 4-byte access for the two); otherwise one node (V = float).
+// ---------------------------------------------------------------------------
+template <class V>
+struct FFV {
+    V hi, lo;
+};
+__device__ __forceinline__ float ffsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float2 ffsub(float2 a, float2 b) { return fma2(b, f2s(-1.0f), a); }   // exact product
+template <class V>
+__device__ __forceinline__ V two_sum_err(V a, V b, V s) {   // a + b - s for s = fl(a + b)
+    const V t = ffsub(s, a);
+    return add2(ffsub(a, ffsub(s, t)), ffsub(b, t));
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ff_norm(V s, V e) {       // |e| below an ulp or so of s
+    const V h = add2(s, e);
+    return {h, ffsub(e, ffsub(h, s))};
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_acc(FFV<V> a, V b) {   // accumulate one value (not normalised)
+    const V s = add2(a.hi, b);
+    return {s, add2(a.lo, two_sum_err(a.hi, b, s))};
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_acc(FFV<V> a, FFV<V> b) {
+    const V s = add2(a.hi, b.hi);
+    return {s, add2(add2(a.lo, b.lo), two_sum_err(a.hi, b.hi, s))};
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_add(FFV<V> a, FFV<V> b) {
+    const FFV<V> r = ffv_acc(a, b);
+    return ff_norm(r.hi, r.lo);
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_neg(FFV<V> a) { return {neg2(a.hi), neg2(a.lo)}; }
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_prod(FFV<V> a, FFV<V> b) {   // not normalised
+    const V p = mul2(a.hi, b.hi);
+    const V e = fma2(a.hi, b.lo, fma2(a.lo, b.hi, fma2(a.hi, b.hi, neg2(p))));
+    return {p, e};
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_mul(FFV<V> a, FFV<V> b) {
+    const FFV<V> r = ffv_prod(a, b);
+    return ff_norm(r.hi, r.lo);
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_small(FFV<V> a, float c) {   // times a small integer or a power of two
+    const V p = mul2(a.hi, splat<V>(c));
+    return ff_norm(p, fma2(a.lo, splat<V>(c), fma2(a.hi, splat<V>(c), neg2(p))));
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_const(float2 c) { return {splat<V>(c.x), splat<V>(c.y)}; }
+
+// Constants of the rule as float-float pairs (x = hi, y = lo).
+struct Rule5FF {
+    float2 w[kQ1], w2[kQ1 * kQ1];   // rest weights w_i and w_i w_j
+    float2 th0, kOa, kOb, kEa, kEb;
+};
+float2 split_ff(double v) {
+    const float hi = (float)v;
+    return make_float2(hi, (float)(v - (double)hi));
+}
+Rule5FF rule5_ff(const LatticeParams& P) {
+    Rule5FF R;
+    for (int i = 0; i < kQ1; ++i) {
+        R.w[i] = split_ff(P.w1[i]);
+        for (int j = 0; j < kQ1; ++j) R.w2[i * kQ1 + j] = split_ff(P.w1[i] * P.w1[j]);
+    }
+    const double a = P.v[1], b = P.v[3];
+    R.th0 = split_ff(P.theta0);
+    R.kOa = split_ff(1.0 / (2.0 * a));
+    R.kOb = split_ff(1.0 / (2.0 * b * (b * b - a * a)));
+    R.kEa = split_ff(1.0 / (2.0 * a * a));
+    R.kEb = split_ff(1.0 / (2.0 * b * b * (b * b - a * a)));
+    return R;
 }
 
+// dr_i = r_i(u, theta) - w_i of one axis (constraint form, see the file header).
+template <class V>
+__device__ __forceinline__ void axis_ff(const LatticeParams& P, const Rule5FF& R, FFV<V> u, FFV<V> dth,
+                                        FFV<V> (&dr)[kQ1]) {
+    const FFV<V> th0 = ffv_const<V>(R.th0);
+    const FFV<V> th = ffv_add(th0, dth);
+    const FFV<V> u2 = ffv_mul(u, u);
+    const FFV<V> d2 = ffv_add(u2, dth);
+    const FFV<V> d3 = ffv_mul(u, ffv_add(u2, ffv_small(th, 3.0f)));
+    const FFV<V> d4 = ffv_add(ffv_mul(u2, ffv_add(u2, ffv_small(th, 6.0f))),
+                              ffv_small(ffv_mul(dth, ffv_add(th, th0)), 3.0f));
+    const FFV<V> Ob = ffv_mul(ffv_add(d3, ffv_small(u, -P.sa2)), ffv_const<V>(R.kOb));
+    const FFV<V> Oa = ffv_mul(ffv_add(u, ffv_small(Ob, -2.0f * P.sb)), ffv_const<V>(R.kOa));
+    const FFV<V> Eb = ffv_mul(ffv_add(d4, ffv_small(d2, -P.sa2)), ffv_const<V>(R.kEb));
+    const FFV<V> Ea = ffv_mul(ffv_add(d2, ffv_small(Eb, -2.0f * P.sb2)), ffv_const<V>(R.kEa));
+    dr[0] = ffv_small(ffv_add(Ea, Eb), -2.0f);
+    dr[1] = ffv_add(Ea, Oa);
+    dr[2] = ffv_add(Ea, ffv_neg(Oa));
+    dr[3] = ffv_add(Eb, Ob);
+    dr[4] = ffv_add(Eb, ffv_neg(Ob));
+}
+
+// hi + lo rounded to the storage type S (for 16 bits: an FP32 value that rounds on
+// to S as hi + lo would).  near: whether a value within d of hi + lo could round
+// otherwise.  Every 16-bit tie is an FP32 number whose twelve low bits are zero, so
+// only such a value is moved off the tie towards hi + lo.
 template <typename S>
-__global__ void k_moments3(const __grid_constant__ LatticeParams P, const S* __restrict__ f, double* rho,
-                           double* ux, double* uy, double* uz, double* theta) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ float round_ff(float hi, float lo, float d, bool& near) {
+    const float r = __fadd_rn(hi, lo);
+    if constexpr (sizeof(S) == 4) {
+        near = __fadd_rn(hi, __fadd_rn(lo, d)) != __fadd_rn(hi, __fsub_rn(lo, d));
+        return r;
+    } else {
+        near = false;
+        if (__float_as_int(r) & 0xfff) return r;
+        const float e = two_sum_err(hi, lo, r);
+        near = fabsf(e) <= d;
+        int b = __float_as_int(r);
+        if (e != 0.0f && isfinite(r)) b += ((e > 0.0f) == (b >= 0)) ? 1 : -1;
+        return __int_as_float(b);
+    }
+}
+
+// The populations of one node whose rounding the float-float arithmetic left open
+// (bit 5 b + c of open[a * stride]): f^eq_abc = rho r^x_a r^y_b r^z_c by the C mu rule in FP64.
+template <typename S>
+__device__ __noinline__ void init3_open(const LatticeParams& P, const unsigned* open, int stride, double rho, double ux,
+                                        double uy, double uz, double th, S* at) {
+    double ra[kQ1], rb[kQ1], rc[kQ1];
+    rule_q<kQ1>(P, ux, th, ra);
+    rule_q<kQ1>(P, uy, th, rb);
+    rule_q<kQ1>(P, uz, th, rc);
+#pragma unroll
+    for (int a = 0; a < kQ1; ++a) {
+        const unsigned m = open[a * stride];
+        if (!m) continue;
+        const double ra1 = rho * ra[a];
+#pragma unroll
+        for (int b = 0; b < kQ1; ++b) {
+            const double X = ra1 * rb[b];
+#pragma unroll
+            for (int c = 0; c < kQ1; ++c)
+                if ((m >> (kQ1 * b + c)) & 1u) {
+                    const int p = (a * kQ1 + b) * kQ1 + c;
+                    at[(long long)p * P.plane] = Storage<S>::from_f64(__dmul_rn(X, rc[c]), w0_3(P, p));   // f^eq rounded before the difference
+                }
+        }
+    }
+}
+
+// The checks of plbm_init3, made as the fields are read: the bits of a value that
+// is not finite, or of a rho or theta that is not positive.
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool positive64(double v) { return __double_as_longlong(v) > 0; }
+__device__ __forceinline__ void check_init3(const LatticeParams& P, double r, double a, double b, double c, double t) {
+    const bool fr = finite64(r), ft = finite64(t);
+    if (fr && ft && finite64(a) && finite64(b) && finite64(c) && positive64(r) && positive64(t)) return;
+    unsigned bits = 0u;
+    if (!(fr && ft && finite64(a) && finite64(b) && finite64(c))) bits |= PLBM_STATUS_NONFINITE;
+    if (fr && !positive64(r)) bits |= PLBM_STATUS_RHO_NONPOS;
+    if (ft && !positive64(t)) bits |= PLBM_STATUS_THETA_NONPOS;
+    atomicOr(P.status, bits);
+}
+
+__device__ __forceinline__ void set_lane(FFV<float>& v, int, double d) {
+    v.hi = (float)d;
+    v.lo = (float)(d - (double)v.hi);
+}
+__device__ __forceinline__ void set_lane(FFV<float2>& v, int lane, double d) {
+    const float hi = (float)d, lo = (float)(d - (double)hi);
+    if (lane) {
+        v.hi.y = hi;
+        v.lo.y = lo;
+    } else {
+        v.hi.x = hi;
+        v.lo.x = lo;
+    }
+}
+
+// g_abc = A_ab r^z_c + w_a w_b dr^z_c with A_ab = X_a r^y_b + w_a dr^y_b and
+// X_a = rho r^x_a - w_a = (rho - 1) w_a + rho dr^x_a.  Values nearer to a rounding
+// boundary of S than 2^-45 of the two products and 2^-50 of w_a w_b (more than the
+// error of this arithmetic and of the FP64 rule; some 1e-5 of all in a flow) are formed
+// again by the FP64 rule, so the stored state is the FP64 rule's, rounded.  The
+// loops over a and b stay loops, their factors in shared memory: unrolled, the
+// 125 roundings overflow the instruction cache.
+template <typename S, class V>
+__global__ void __launch_bounds__(kB3) k_init3_dev(const __grid_constant__ LatticeParams P,
+                                                   const __grid_constant__ Rule5FF R, const double* __restrict__ rho,
+                                                   const double* __restrict__ ux, const double* __restrict__ uy,
+                                                   const double* __restrict__ uz, const double* __restrict__ theta,
+                                                   S* __restrict__ f) {
+    constexpr int kLanes = sizeof(V) / sizeof(float);
+    __shared__ FFV<V> sX[kQ1][kB3], sRy[kQ1][kB3], sDy[kQ1][kB3];
+    __shared__ unsigned sOpen[kLanes][kQ1][kB3];
+    const int x = blockIdx.x * kB3 + threadIdx.x, t = threadIdx.x;
+    const int y = blockIdx.y, z = blockIdx.z;
+    if (x >= P.nx) return;   // no barrier below: a thread reads only its own column of the shared arrays
+    FFV<V> drho, dth, u[3];
+#pragma unroll
+    for (int l = 0; l < kLanes; ++l) {
+        const long long n = ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x;
+        const double r = rho[n], a = ux[n], b = uy[n], c = uz[n], th = theta[n];
+        check_init3(P, r, a, b, c, th);
+        set_lane(drho, l, r - 1.0);
+        set_lane(u[0], l, a);
+        set_lane(u[1], l, b);
+        set_lane(u[2], l, c);
+        set_lane(dth, l, th - P.theta0);
+    }
+    FFV<V> dr[kQ1], rz[kQ1];
+    {
+        const FFV<V> rh = ffv_add(FFV<V>{splat<V>(1.0f), splat<V>(0.0f)}, drho);
+        axis_ff(P, R, u[0], dth, dr);
+#pragma unroll
+        for (int a = 0; a < kQ1; ++a)
+            sX[a][t] = ffv_add(ffv_mul(drho, ffv_const<V>(R.w[a])), ffv_mul(rh, dr[a]));
+        axis_ff(P, R, u[1], dth, dr);
+#pragma unroll
+        for (int b = 0; b < kQ1; ++b) {
+            sDy[b][t] = dr[b];
+            sRy[b][t] = ffv_add(ffv_const<V>(R.w[b]), dr[b]);
+        }
+    }
+    axis_ff(P, R, u[2], dth, dr);
+#pragma unroll
+    for (int c = 0; c < kQ1; ++c) rz[c] = ffv_add(ffv_const<V>(R.w[c]), dr[c]);
+    S* out = f + node3(P, x, y, z);
+    unsigned any[2] = {0u, 0u};
+#pragma unroll 1
+    for (int a = 0; a < kQ1; ++a) {
+        const FFV<V> wa = ffv_const<V>(R.w[a]), X = sX[a][t];
+        unsigned open[2] = {0u, 0u};
+#pragma unroll 1
+        for (int b = 0; b < kQ1; ++b) {
+            const FFV<V> A = ffv_add(ffv_mul(X, sRy[b][t]), ffv_mul(wa, sDy[b][t]));
+            const FFV<V> W = ffv_const<V>(R.w2[a * kQ1 + b]);
+            const float dw = fabsf(R.w2[a * kQ1 + b].x) * 0x1p-50f;
+#pragma unroll
+            for (int c = 0; c < kQ1; ++c, out += P.plane) {
+                const FFV<V> q = ffv_prod(A, rz[c]), w = ffv_prod(W, dr[c]);
+                const FFV<V> g = ffv_acc(q, w);
+                bool near;
+                if constexpr (kLanes == 2) {
+                    const float v0 = round_ff<S>(g.hi.x, g.lo.x, fmaf(fabsf(q.hi.x) + fabsf(w.hi.x), 0x1p-45f, dw), near);
+                    open[0] = 2u * open[0] + near;
+                    const float v1 = round_ff<S>(g.hi.y, g.lo.y, fmaf(fabsf(q.hi.y) + fabsf(w.hi.y), 0x1p-45f, dw), near);
+                    open[1] = 2u * open[1] + near;
+                    *reinterpret_cast<unsigned*>(out) = Pack2<S>::pack(f2(v0, v1));
+                } else {
+                    Storage<S>::store(out, round_ff<S>(g.hi, g.lo, fmaf(fabsf(q.hi) + fabsf(w.hi), 0x1p-45f, dw), near));
+                    open[0] = 2u * open[0] + near;
+                }
+            }
+        }
+#pragma unroll
+        for (int l = 0; l < kLanes; ++l) {
+            open[l] = __brev(open[l]) >> 7;   // bit 5 b + c
+            sOpen[l][a][t] = open[l];
+            any[l] |= open[l];
+        }
+    }
+#pragma unroll 1
+    for (int l = 0; l < kLanes; ++l) {
+        if (!(l ? any[1] : any[0])) continue;
+        const long long n = ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x;
+        init3_open<S>(P, &sOpen[l][0][t], kB3, rho[n], ux[n], uy[n], uz[n], theta[n], f + node3(P, x, y, z) + l);
+    }
+}
+
+// FP64 value of a float-float sum; hi alone when it overflowed (lo is NaN then).
+__device__ __forceinline__ double ffv_f64(float hi, float lo) { return (double)hi + (lo == lo ? (double)lo : 0.0); }
+__device__ __forceinline__ double lane_f64(FFV<float> v, int) { return ffv_f64(v.hi, v.lo); }
+__device__ __forceinline__ double lane_f64(FFV<float2> v, int l) {
+    return l ? ffv_f64(v.hi.y, v.lo.y) : ffv_f64(v.hi.x, v.lo.x);
+}
+
+// Row sums R_ab = sum_c g, S_a, T_b, U_c of the stored deviations, then
+// rho - 1 = sum S, j = sum v S (per axis), E - 3 theta0 = sum v^2 (S + T + U); the
+// fields of each node in FP64.
+template <typename S, class V>
+__global__ void __launch_bounds__(kB3) k_moments3_dev(const __grid_constant__ LatticeParams P, const S* __restrict__ f,
+                                                      double* rho, double* ux, double* uy, double* uz, double* theta) {
+    constexpr int kLanes = sizeof(V) / sizeof(float);
+    const int x = blockIdx.x * kB3 + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= P.nx) return;
     const long long here = node3(P, x, y, z);
-    double fn[kQ3], m[9];
-    for (int p = 0; p < P.q; ++p) fn[p] = Storage<S>::to_f64(f[(long long)p * P.plane + here], w0_3(P, p));
-    moments3_f64(P, fn, m);
+    const FFV<V> zero{splat<V>(0.0f), splat<V>(0.0f)};
+    FFV<V> Sa[kQ1], Tb[kQ1], Uc[kQ1];
+#pragma unroll
+    for (int i = 0; i < kQ1; ++i) Sa[i] = Tb[i] = Uc[i] = zero;
+#pragma unroll
+    for (int a = 0; a < kQ1; ++a)
+#pragma unroll
+        for (int b = 0; b < kQ1; ++b) {
+            FFV<V> Rab = zero;
+#pragma unroll
+            for (int c = 0; c < kQ1; ++c) {
+                const S* at = f + (long long)((a * kQ1 + b) * kQ1 + c) * P.plane + here;
+                V g;
+                if constexpr (kLanes == 2)
+                    g = Pack2<S>::unpack(__ldg(reinterpret_cast<const unsigned*>(at)));
+                else
+                    g = Storage<S>::load(at);
+                if (c == 0)
+                    Rab.hi = g;
+                else
+                    Rab = ffv_acc(Rab, g);
+                Uc[c] = ffv_acc(Uc[c], g);
+            }
+            Sa[a] = ffv_acc(Sa[a], Rab);
+            Tb[b] = ffv_acc(Tb[b], Rab);
+        }
+    FFV<V> dm = zero, jx = zero, jy = zero, jz = zero, de = zero;
+#pragma unroll
+    for (int i = 0; i < kQ1; ++i) {
+        const float vi = (float)P.v[i];
+        dm = ffv_acc(dm, Sa[i]);
+        jx = ffv_acc(jx, ffv_small(Sa[i], vi));
+        jy = ffv_acc(jy, ffv_small(Tb[i], vi));
+        jz = ffv_acc(jz, ffv_small(Uc[i], vi));
+        de = ffv_acc(de, ffv_small(ffv_acc(ffv_acc(Sa[i], Tb[i]), Uc[i]), vi * vi));
+    }
+#pragma unroll
+    for (int l = 0; l < kLanes; ++l) {
+        const double m = 1.0 + lane_f64(dm, l);
+        const double im = 1.0 / m;
+        const double a = lane_f64(jx, l) * im, b = lane_f64(jy, l) * im, c = lane_f64(jz, l) * im;
+        const long long n = ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x;
+        if (rho) rho[n] = m;
+        if (ux) ux[n] = a;
+        if (uy) uy[n] = b;
+        if (uz) uz[n] = c;
+        if (theta) theta[n] = ((3.0 * P.theta0 + lane_f64(de, l)) * im - (a * a + b * b + c * c)) * (1.0 / 3.0);
+    }
+}
+
+// FP64 storage (q1 = 3 to 5 at compile time: nothing in local memory).
+template <int Q1>
+__global__ void __launch_bounds__(kB3) k_init3_q(const __grid_constant__ LatticeParams P,
+                                                 const double* __restrict__ rho, const double* __restrict__ ux,
+                                                 const double* __restrict__ uy, const double* __restrict__ uz,
+                                                 const double* __restrict__ theta, double* __restrict__ f) {
+    const int x = blockIdx.x * kB3 + threadIdx.x;
+    const int y = blockIdx.y, z = blockIdx.z;
+    if (x >= P.nx) return;
     const long long n = ((long long)z * P.ny + y) * P.nx + x;
-    if (rho) rho[n] = m[0];
-    if (ux) ux[n] = m[1];
-    if (uy) uy[n] = m[2];
-    if (uz) uz[n] = m[3];
-    if (theta) theta[n] = m[4];
+    const double t = theta ? theta[n] : 1.0;
+    check_init3(P, rho[n], ux[n], uy[n], uz[n], t);
+    const double th = (P.isothermal || theta == nullptr) ? P.theta0 : t;
+    double ra[Q1], rb[Q1], rc[Q1];
+    rule_q<Q1>(P, ux[n], th, ra);
+    rule_q<Q1>(P, uy[n], th, rb);
+    rule_q<Q1>(P, uz[n], th, rc);
+    const long long here = node3(P, x, y, z);
+    const double r = rho[n];
+#pragma unroll
+    for (int a = 0; a < Q1; ++a)
+#pragma unroll
+        for (int b = 0; b < Q1; ++b) {
+            const double X = r * ra[a] * rb[b];
+#pragma unroll
+            for (int c = 0; c < Q1; ++c) f[(long long)((a * Q1 + b) * Q1 + c) * P.plane + here] = X * rc[c];
+        }
+}
+
+template <int Q1>
+__global__ void __launch_bounds__(kB3) k_moments3_q(const __grid_constant__ LatticeParams P,
+                                                    const double* __restrict__ f, double* rho, double* ux, double* uy,
+                                                    double* uz, double* theta) {
+    const int x = blockIdx.x * kB3 + threadIdx.x;
+    const int y = blockIdx.y, z = blockIdx.z;
+    if (x >= P.nx) return;
+    const long long here = node3(P, x, y, z);
+    double Sa[Q1], Tb[Q1], Uc[Q1];
+#pragma unroll
+    for (int i = 0; i < Q1; ++i) Sa[i] = Tb[i] = Uc[i] = 0.0;
+#pragma unroll
+    for (int a = 0; a < Q1; ++a)
+#pragma unroll
+        for (int b = 0; b < Q1; ++b) {
+            double Rab = 0.0;
+#pragma unroll
+            for (int c = 0; c < Q1; ++c) {
+                const double v = __ldg(f + (long long)((a * Q1 + b) * Q1 + c) * P.plane + here);
+                Rab += v;
+                Uc[c] += v;
+            }
+            Sa[a] += Rab;
+            Tb[b] += Rab;
+        }
+    double m = 0.0, mx = 0.0, my = 0.0, mz = 0.0, en = 0.0;
+#pragma unroll
+    for (int i = 0; i < Q1; ++i) {
+        const double vi = (double)P.v[i];
+        m += Sa[i];
+        mx += vi * Sa[i];
+        my += vi * Tb[i];
+        mz += vi * Uc[i];
+        en += vi * vi * (Sa[i] + Tb[i] + Uc[i]);
+    }
+    const double a = mx / m, b = my / m, c = mz / m;
+    const long long n = ((long long)z * P.ny + y) * P.nx + x;
+    if (rho) rho[n] = m;
+    if (ux) ux[n] = a;
+    if (uy) uy[n] = b;
+    if (uz) uz[n] = c;
+    if (theta) theta[n] = (en / m - (a * a + b * b + c * c)) / 3.0;
 }
 
 // Per-block FP64 record: mass, j_x, j_y, energy, min rho, min theta, j_z.
@@ -881,6 +1220,29 @@ dim3 grid3(const LatticeParams& P) { return dim3((P.nx + kB3 - 1) / kB3, P.ny, P
         default: return cudaErrorInvalidValue;                           \
     }
 
+// A kernel <S, V> of the 16/32-bit precisions: both nodes of a pair per thread on
+// the z-paired layout (16-bit storage only), one node otherwise.
+#define PLBM_LAUNCH3_DEV(KERNEL, ARGS)                                                           \
+    {                                                                                            \
+        const dim3 grid((P.nx + kB3 - 1) / kB3, P.ny, P.zpaired ? P.half_nz : P.nz);             \
+        switch (prec) {                                                                          \
+            case kF32: { using S = float; KERNEL<S, float><<<grid, kB3, 0, s>>> ARGS; break; }   \
+            case kF16Dev: {                                                                      \
+                using S = __half;                                                                \
+                if (P.zpaired) KERNEL<S, float2><<<grid, kB3, 0, s>>> ARGS;                      \
+                else KERNEL<S, float><<<grid, kB3, 0, s>>> ARGS;                                 \
+                break;                                                                           \
+            }                                                                                    \
+            case kBF16Dev: {                                                                     \
+                using S = __nv_bfloat16;                                                         \
+                if (P.zpaired) KERNEL<S, float2><<<grid, kB3, 0, s>>> ARGS;                      \
+                else KERNEL<S, float><<<grid, kB3, 0, s>>> ARGS;                                 \
+                break;                                                                           \
+            }                                                                                    \
+            default: return cudaErrorInvalidValue;                                               \
+        }                                                                                        \
+    }
+
 }  // namespace
 
 long long reduce3_blocks(const LatticeParams& P) {
@@ -893,10 +1255,10 @@ cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void
         double* b = static_cast<double*>(dst);
         if (P.q1 == 5)
             k_stream_collide3_f64q<5><<<grid3(P), kB3, 0, s>>>(P, a, b);
-        else if (P.q1 == 3)
-            k_stream_collide3_f64q<3><<<grid3(P), kB3, 0, s>>>(P, a, b);
+        else if (P.q1 == 4)
+            k_stream_collide3_f64q<4><<<grid3(P), kB3, 0, s>>>(P, a, b);
         else
-            k_stream_collide3_f64<<<grid3(P), kB3, 0, s>>>(P, a, b);
+            k_stream_collide3_f64q<3><<<grid3(P), kB3, 0, s>>>(P, a, b);
         return cudaGetLastError();
     }
     if (!P.sym5 || P.q1 != kQ1 || P.isothermal) return cudaErrorInvalidValue;
@@ -932,13 +1294,36 @@ cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void
 
 cudaError_t launch_init3(int prec, const LatticeParams& P, const double* rho, const double* ux, const double* uy,
                          const double* uz, const double* theta, void* f, cudaStream_t s) {
-    PLBM_DISPATCH3(prec, (k_init3<S><<<grid3(P), kB3, 0, s>>>(P, rho, ux, uy, uz, theta, static_cast<S*>(f))));
+    if (prec == kF64) {
+        double* d = static_cast<double*>(f);
+        if (P.q1 == 5)
+            k_init3_q<5><<<grid3(P), kB3, 0, s>>>(P, rho, ux, uy, uz, theta, d);
+        else if (P.q1 == 4)
+            k_init3_q<4><<<grid3(P), kB3, 0, s>>>(P, rho, ux, uy, uz, theta, d);
+        else
+            k_init3_q<3><<<grid3(P), kB3, 0, s>>>(P, rho, ux, uy, uz, theta, d);
+        return cudaGetLastError();
+    }
+    if (!P.sym5 || P.isothermal || !theta) return cudaErrorInvalidValue;   // validated at create and init
+    const Rule5FF R = rule5_ff(P);
+    PLBM_LAUNCH3_DEV(k_init3_dev, (P, R, rho, ux, uy, uz, theta, static_cast<S*>(f)))
     return cudaGetLastError();
 }
 
 cudaError_t launch_moments3(int prec, const LatticeParams& P, const void* f, double* rho, double* ux, double* uy,
                             double* uz, double* theta, cudaStream_t s) {
-    PLBM_DISPATCH3(prec, (k_moments3<S><<<grid3(P), kB3, 0, s>>>(P, static_cast<const S*>(f), rho, ux, uy, uz, theta)));
+    if (prec == kF64) {
+        const double* d = static_cast<const double*>(f);
+        if (P.q1 == 5)
+            k_moments3_q<5><<<grid3(P), kB3, 0, s>>>(P, d, rho, ux, uy, uz, theta);
+        else if (P.q1 == 4)
+            k_moments3_q<4><<<grid3(P), kB3, 0, s>>>(P, d, rho, ux, uy, uz, theta);
+        else
+            k_moments3_q<3><<<grid3(P), kB3, 0, s>>>(P, d, rho, ux, uy, uz, theta);
+        return cudaGetLastError();
+    }
+    if (!P.sym5) return cudaErrorInvalidValue;
+    PLBM_LAUNCH3_DEV(k_moments3_dev, (P, static_cast<const S*>(f), rho, ux, uy, uz, theta))
     return cudaGetLastError();
 }
 

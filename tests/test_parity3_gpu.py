@@ -224,3 +224,36 @@ def test_d3q125_bench_size_sampled_nodes(prec, tol):
         mo = lat.moments(lat.run(lat.init(*patch), k))
         for g, o, scale in zip(mg, mo, (1.0, 0.1, 0.1, 0.1, 1.0)):
             assert abs(g[cz, cy, cx] - o[half, half, half]) <= tol * scale, (prec, cx, cy, cz)
+
+
+# Initial state and fields of 16/32-bit handles: one node per thread (odd nz, FP32)
+# and both nodes of a pair (even nz, 16-bit), block remainders, a single column.
+# The stored deviation is the FP64 value f^eq - w0 rounded once to the storage type
+# (half a unit in the last place, plus 4e-16 for the rounding of f^eq, w0 and w0 + g
+# themselves in FP64); the fields are those of the FP64 sums of the stored
+# populations to 3e-14 (125 roundings of 2^-54 times |v|^2 <= 27).
+@pytest.mark.parametrize("prec", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("shape,v,theta0", [((129, 3, 5), V5, 1.0), ((130, 4, 6), V5, 1.0), ((1, 2, 8), V5, 0.9),
+                                            ((37, 1, 14), (0, 1, -1, 2, -2), 0.7)])
+def test_d3q125_initial_state_and_fields_to_the_last_bit_of_storage(prec, shape, v, theta0):
+    from paper_1402_5487_gb300 import plbm
+    nx, ny, nz = shape
+    f = fields3(nx, ny, nz, 11, amp_u=0.05, theta0=theta0)
+    lat = O.Lattice3(v, 1.2, nx, ny, nz, theta0=theta0)
+    want = lat.init(*f).reshape(125, nz, ny, nx)
+    one, zero = np.ones_like(f[0]), np.zeros_like(f[0])
+    w0 = lat.init(one, zero, zero, zero, theta0 * one).reshape(125, nz, ny, nx)
+    s = plbm.Solver(3, v, 1.2, nx, ny, nz=nz, theta0=theta0, prec=prec)
+    s.init(f[0], f[1], f[2], f[4], uz=f[3])
+    got, mom = s.get_populations(), s.moments()
+    s.close()
+    g = np.abs(want - w0)
+    bits, low = {"f32": (24, -149), "f16dev": (11, -24), "bf16dev": (8, -133)}[prec]
+    ulp = np.exp2(np.maximum(np.frexp(np.maximum(g, 1e-300))[1] - bits, low))
+    assert np.all(np.abs(got - want) <= 0.5 * ulp * (1 + 1e-6) + 4e-16)
+    c = np.array([[a, b, d] for a in v for b in v for d in v], dtype=np.float64)
+    rho = got.sum(0)
+    u = [np.tensordot(c[:, k], got, 1) / rho for k in range(3)]
+    th = (np.tensordot((c * c).sum(1), got, 1) / rho - sum(a * a for a in u)) / 3
+    for a, b in zip(mom, (rho, u[0], u[1], u[2], th)):
+        assert np.max(np.abs(a - b)) <= 3e-14
