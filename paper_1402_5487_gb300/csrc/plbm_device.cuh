@@ -32,6 +32,39 @@
 namespace plbm {
 
 // ---------------------------------------------------------------------------
+// Step kernels follow one another on a stream, each reading what the one before
+// wrote.  Launched plainly, a step waits for the last block of the step before, then
+// for its own launch: 2-5 us in which the SMs drain and refill.  They are
+// launched as programmatic dependents instead: a block says at its start that the
+// next grid may be set up (step_begin), whose blocks then take the SM slots that
+// fall free and compute their addresses, and every thread that touches memory
+// waits for the grid before to be complete and flushed (step_wait) first.  A
+// kernel launched without the attribute passes both at once.  Per step: 2048^2 FP32
+// 123.2 -> 120.6 us, FP16 69.7 -> 67.3 us, 512^2 FP32 (graph) 6.56 -> 6.29 us.
+// Grids of fewer than kDependentThreads threads leave slots free for several
+// waiting grids at once, which then crowd the running one (128^2 FP64: 10.2 ->
+// 16.4 us a step); they are launched plainly, as are the persistent batch kernels,
+// which leave no slot free (174 us a step either way).
+// ---------------------------------------------------------------------------
+constexpr long long kDependentThreads = 1 << 16;
+__device__ __forceinline__ void step_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = (long long)grid.x * grid.y * grid.z * block.x >= kDependentThreads ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // Storage traits: how a stored element becomes an arithmetic value.
 // ---------------------------------------------------------------------------
 template <typename S>
@@ -613,8 +646,10 @@ template <typename S, int Q1, int DIM, bool REDUCE>
 __global__ void __launch_bounds__(kBlockX)
 k_stream_collide(const __grid_constant__ LatticeParams P, const S* __restrict__ src,
                  S* __restrict__ dst) {
+    step_begin();
     const int x = blockIdx.x * (REDUCE ? kBlockX : (int)blockDim.x) + threadIdx.x;
     const int y = blockIdx.y;
+    step_wait();
 
     NodeDiag d;       // FP64 storage
     NodeDiagF df;     // 16/32-bit storage
@@ -685,11 +720,8 @@ cudaError_t launch_step_t(const LatticeParams& P, const void* src, void* dst, bo
     S* t = static_cast<S*>(dst);
 #define PLBM_LAUNCH(Q1v, DIMv)                                                              \
     if (P.q1 == Q1v && P.dim == DIMv) {                                                     \
-        if (reduce)                                                                         \
-            k_stream_collide<S, Q1v, DIMv, true><<<grid, block, 0, stream>>>(P, s, t);      \
-        else                                                                                \
-            k_stream_collide<S, Q1v, DIMv, false><<<grid, block, 0, stream>>>(P, s, t);     \
-        return cudaGetLastError();                                                          \
+        return reduce ? launch_dependent(k_stream_collide<S, Q1v, DIMv, true>, grid, block, stream, P, s, t)    \
+                      : launch_dependent(k_stream_collide<S, Q1v, DIMv, false>, grid, block, stream, P, s, t);  \
     }
     PLBM_LAUNCH(3, 1)
     PLBM_LAUNCH(4, 1)

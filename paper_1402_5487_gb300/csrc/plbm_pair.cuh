@@ -325,6 +325,7 @@ k_stream_collide_pair2(const __grid_constant__ PairParams P, const typename Pair
                        typename PairStore<S>::V* __restrict__ dst, int tiles_x, int ntiles) {
     using PS = PairStore<S>;
     using V = typename PS::V;
+    step_begin();
     const int t0 = 2 * blockIdx.x;
     const int ra = t0 / tiles_x;
     const int xa = (t0 - ra * tiles_x) * kPair2Block + threadIdx.x;
@@ -344,6 +345,7 @@ k_stream_collide_pair2(const __grid_constant__ PairParams P, const typename Pair
             for (int j = 0; j < 5; ++j) v[5 * i + j] = PS::raw(src + (5 * i + j) * P.plane2 + (row[j] + col[i]));
         return m;
     };
+    step_wait();
     if (xa < P.nx) ma = load(xa, ra, va);
     if (xb < P.nx) mb = load(xb, rb, vb);
     NodeDiagF d;
@@ -433,9 +435,11 @@ __device__ __forceinline__ void sym5_node(const PairParams& P, const S* __restri
 template <typename S, bool REDUCE>
 __global__ void __launch_bounds__(kBlockX)
 k_stream_collide_sym5(const __grid_constant__ PairParams P, const S* __restrict__ src, S* __restrict__ dst) {
+    step_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     NodeDiagF d;
     if (REDUCE) diagf_zero(d);
+    step_wait();
     if (x < P.nx) sym5_node<S, REDUCE>(P, src, dst, x, blockIdx.y, d);
     if (REDUCE) {
         const int blk = blockIdx.y * gridDim.x + blockIdx.x;
@@ -458,9 +462,11 @@ __global__ void __launch_bounds__(kBlockX, REDUCE ? 0 : PairMinBlocks<S>::value)
 k_stream_collide_pair(const __grid_constant__ PairParams P,
                       const typename PairStore<S>::V* __restrict__ src,
                       typename PairStore<S>::V* __restrict__ dst) {
+    step_begin();
     const int x = blockIdx.x * kBlockX + threadIdx.x;
     NodeDiagF d;
     if (REDUCE) diagf_zero(d);
+    step_wait();
     if (x < P.nx) pair_node<S, REDUCE>(P, src, dst, x, blockIdx.y, d);
     if (REDUCE) {
         const int blk = blockIdx.y * gridDim.x + blockIdx.x;
@@ -479,11 +485,8 @@ cudaError_t launch_step_sym5_t(const LatticeParams& L, const void* src, void* ds
     dim3 grid((P.nx + bx - 1) / bx, P.ny);
     const S* s = static_cast<const S*>(src);
     S* t = static_cast<S*>(dst);
-    if (reduce)
-        k_stream_collide_sym5<S, true><<<grid, kBlockX, 0, stream>>>(P, s, t);
-    else
-        k_stream_collide_sym5<S, false><<<grid, bx, 0, stream>>>(P, s, t);
-    return cudaGetLastError();
+    return reduce ? launch_dependent(k_stream_collide_sym5<S, true>, grid, kBlockX, stream, P, s, t)
+                  : launch_dependent(k_stream_collide_sym5<S, false>, grid, bx, stream, P, s, t);
 }
 
 template <typename S>
@@ -498,15 +501,12 @@ cudaError_t launch_step_pair_t(const LatticeParams& L, const void* src, void* ds
         if (!reduce) {
             const int tiles_x = (P.nx + kPair2Block - 1) / kPair2Block;
             const int ntiles = tiles_x * P.half_ny;
-            k_stream_collide_pair2<S><<<(ntiles + 1) / 2, kPair2Block, 0, stream>>>(P, s, t, tiles_x, ntiles);
-            return cudaGetLastError();
+            return launch_dependent(k_stream_collide_pair2<S>, (ntiles + 1) / 2, kPair2Block, stream, P, s, t, tiles_x,
+                                    ntiles);
         }
     }
-    if (reduce)
-        k_stream_collide_pair<S, true><<<grid, kBlockX, 0, stream>>>(P, s, t);
-    else
-        k_stream_collide_pair<S, false><<<grid, kBlockX, 0, stream>>>(P, s, t);
-    return cudaGetLastError();
+    return reduce ? launch_dependent(k_stream_collide_pair<S, true>, grid, kBlockX, stream, P, s, t)
+                  : launch_dependent(k_stream_collide_pair<S, false>, grid, kBlockX, stream, P, s, t);
 }
 
 // ---------------------------------------------------------------------------

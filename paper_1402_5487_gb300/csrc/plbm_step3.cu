@@ -89,6 +89,7 @@ __device__ __forceinline__ void axis_dev(const LatticeParams& P, float u, float 
 template <typename S>
 __global__ void __launch_bounds__(kB3, 2) k_stream_collide3(const __grid_constant__ LatticeParams P,
                                                            const S* __restrict__ src, S* __restrict__ dst) {
+    step_begin();
     const int x = blockIdx.x * kB3 + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= P.nx) return;
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__(kB3, 2) k_stream_collide3(const __grid_constan
         ys[i] = wrap_add(y, P.vym[i], P.ny);
         zs[i] = wrap_add(z, P.vzm[i], P.nz);
     }
+    step_wait();
     float g[kQ3];
     float Sa[kQ1], Tb[kQ1], Uc[kQ1];
 #pragma unroll
@@ -193,6 +195,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_stream_collide3_split(const _
     __shared__ float sDx[kQ1][kSplitNodes];       // dr^x_a
     __shared__ float sP[kQ1][kQ1][kSplitNodes];   // P_bc = r^y_b r^z_c
     __shared__ float sQ[kQ1][kQ1][kSplitNodes];   // Q_bc = dr^y_b r^z_c + w_b dr^z_c
+    step_begin();
     const int a = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int x = blockIdx.x * kSplitNodes + lane;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -207,6 +210,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_stream_collide3_split(const _
             zr[i] = wrap_add(z, P.vzm[i], P.nz) * P.ny * P.pitch;
         }
         const long long pa = (long long)a * kQ1 * kQ1 * P.plane;
+        step_wait();
 #pragma unroll
         for (int b = 0; b < kQ1; ++b)
 #pragma unroll
@@ -469,9 +473,11 @@ template <typename S>
 __global__ void __launch_bounds__(kZpairBlock) k_stream_collide3_zpair(const __grid_constant__ LatticeParams P,
                                                                       const S* __restrict__ src,
                                                                       S* __restrict__ dst) {
+    step_begin();
     const int x = blockIdx.x * kZpairBlock + threadIdx.x;
     const int y = blockIdx.y, r = blockIdx.z;   // pair row r: nodes z = r and z = r + nz/2
     if (x >= P.nx) return;
+    step_wait();
     bool wrap = false;
 #pragma unroll
     for (int i = 0; i < kQ1; ++i) wrap |= (r - P.v[i] < 0) || (r - P.v[i] >= P.half_nz);
@@ -546,6 +552,7 @@ template <int Q1>
 __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_constant__ LatticeParams P,
                                                               const double* __restrict__ src,
                                                               double* __restrict__ dst) {
+    step_begin();
     const int x = blockIdx.x * kB3 + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
     if (x >= P.nx) return;
@@ -557,6 +564,7 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
         yr[i] = wrap_add(y, P.vym[i], P.ny) * P.pitch;
         zr[i] = wrap_add(z, P.vzm[i], P.nz) * P.ny * P.pitch;
     }
+    step_wait();
     double Sa[Q1], Tb[Q1], Uc[Q1];
 #pragma unroll
     for (int i = 0; i < Q1; ++i) Sa[i] = Tb[i] = Uc[i] = 0.0;
@@ -1253,43 +1261,38 @@ cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void
     if (prec == kF64) {
         const double* a = static_cast<const double*>(src);
         double* b = static_cast<double*>(dst);
-        if (P.q1 == 5)
-            k_stream_collide3_f64q<5><<<grid3(P), kB3, 0, s>>>(P, a, b);
-        else if (P.q1 == 4)
-            k_stream_collide3_f64q<4><<<grid3(P), kB3, 0, s>>>(P, a, b);
-        else
-            k_stream_collide3_f64q<3><<<grid3(P), kB3, 0, s>>>(P, a, b);
-        return cudaGetLastError();
+        switch (P.q1) {
+            case 5: return launch_dependent(k_stream_collide3_f64q<5>, grid3(P), kB3, s, P, a, b);
+            case 4: return launch_dependent(k_stream_collide3_f64q<4>, grid3(P), kB3, s, P, a, b);
+            case 3: return launch_dependent(k_stream_collide3_f64q<3>, grid3(P), kB3, s, P, a, b);
+        }
+        return cudaErrorInvalidValue;
     }
     if (!P.sym5 || P.q1 != kQ1 || P.isothermal) return cudaErrorInvalidValue;
+    const float* f32 = static_cast<const float*>(src);
+    const __half* f16 = static_cast<const __half*>(src);
+    const __nv_bfloat16* b16 = static_cast<const __nv_bfloat16*>(src);
     if (P.zpaired) {
         const dim3 g((P.nx + kZpairBlock - 1) / kZpairBlock, P.ny, P.half_nz);
         if (prec == kF16Dev)
-            k_stream_collide3_zpair<__half><<<g, kZpairBlock, 0, s>>>(P, static_cast<const __half*>(src),
-                                                                       static_cast<__half*>(dst));
-        else if (prec == kBF16Dev)
-            k_stream_collide3_zpair<__nv_bfloat16><<<g, kZpairBlock, 0, s>>>(
-                P, static_cast<const __nv_bfloat16*>(src), static_cast<__nv_bfloat16*>(dst));
-        else
-            return cudaErrorInvalidValue;
-        return cudaGetLastError();
+            return launch_dependent(k_stream_collide3_zpair<__half>, g, kZpairBlock, s, P, f16, static_cast<__half*>(dst));
+        if (prec == kBF16Dev)
+            return launch_dependent(k_stream_collide3_zpair<__nv_bfloat16>, g, kZpairBlock, s, P, b16,
+                                    static_cast<__nv_bfloat16*>(dst));
+        return cudaErrorInvalidValue;
     }
     switch (prec) {
         case kF32:
-            k_stream_collide3_split<float><<<dim3((P.nx + kSplitNodes - 1) / kSplitNodes, P.ny, P.nz), kSplitThreads, 0,
-                                              s>>>(P, static_cast<const float*>(src), static_cast<float*>(dst));
-            break;
+            return launch_dependent(k_stream_collide3_split<float>,
+                                    dim3((P.nx + kSplitNodes - 1) / kSplitNodes, P.ny, P.nz), kSplitThreads, s, P, f32,
+                                    static_cast<float*>(dst));
         case kF16Dev:
-            k_stream_collide3<__half><<<grid3(P), kB3, 0, s>>>(P, static_cast<const __half*>(src), static_cast<__half*>(dst));
-            break;
+            return launch_dependent(k_stream_collide3<__half>, grid3(P), kB3, s, P, f16, static_cast<__half*>(dst));
         case kBF16Dev:
-            k_stream_collide3<__nv_bfloat16><<<grid3(P), kB3, 0, s>>>(P, static_cast<const __nv_bfloat16*>(src),
-                                                                     static_cast<__nv_bfloat16*>(dst));
-            break;
-        default:
-            return cudaErrorInvalidValue;
+            return launch_dependent(k_stream_collide3<__nv_bfloat16>, grid3(P), kB3, s, P, b16,
+                                    static_cast<__nv_bfloat16*>(dst));
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_init3(int prec, const LatticeParams& P, const double* rho, const double* ux, const double* uy,

@@ -729,3 +729,38 @@ def test_plain_and_row_paired_layouts_give_the_same_state(prec, ny, nx):
         assert np.array_equal(out[0][0], o[0])
         for k in ("mass", "jx", "jy", "energy", "rho_min", "theta_min"):
             assert abs(out[0][1][k] - o[1][k]) <= 1e-12 * max(1.0, abs(out[0][1][k])), k
+
+
+# Steps queued back to back (large grids overlap one step's start with the end of the
+# step before; small ones do not) equal steps awaited one by one, bit for bit: every
+# step kernel, on both sides of the size from which its launches overlap.
+@pytest.mark.parametrize("dim,v,shape,prec,kw", [
+    (2, I.SET_013, (256, 256), "f32", {}), (2, I.SET_013, (512, 300), "f32", {}), (2, I.SET_013, (1024, 258), "f16dev", {}),
+    (2, I.SET_013, (1024, 258), "bf16dev", {}), (2, I.SET_013, (513, 257), "f32", {}), (2, I.SET_D1Q3, (520, 300), "f32",
+                                                                                       {"theta0": 1 / 3, "isothermal": True}),
+    (2, I.SET_013, (300, 280), "f64", {}), (1, I.SET_013, (70000, 1), "f64", {}), (3, I.SET_013, (64, 40, 30), "f32", {}),
+    (3, I.SET_013, (64, 64, 34), "f16dev", {}), (3, I.SET_013, (64, 64, 33), "bf16dev", {}), (3, I.SET_013, (64, 40, 30), "f64", {}),
+])
+def test_queued_steps_equal_awaited_steps(dim, v, shape, prec, kw):
+    import torch
+    from paper_1402_5487_gb300 import plbm
+    nx, ny, nz = (tuple(shape) + (1,))[:3]
+    rng = np.random.default_rng(5)
+    shp = (ny, nx) if dim < 3 else (nz, ny, nx)
+    one = np.ones(shp)
+    u = [0.05 * rng.uniform(-1, 1, shp) for _ in range(3)]
+    th = kw.get("theta0", 1.0) * one
+    got = []
+    for await_each in (False, True):
+        s = plbm.Solver(dim, v, 1.1, nx, ny, nz=nz, prec=prec, **kw)
+        if dim == 3:
+            s.init(one, u[0], u[1], theta=th, uz=u[2])
+        else:
+            s.init(one, u[0], u[1] if dim == 2 else None, th)
+        for _ in range(7 if await_each else 1):
+            s.step(1 if await_each else 7)
+            if await_each:
+                torch.cuda.synchronize()
+        got.append(s.get_populations())
+        s.close()
+    assert np.array_equal(got[0], got[1])
