@@ -147,6 +147,14 @@ __device__ __forceinline__ void flag_status(const LatticeParams& P, R rho, R the
     }
 }
 
+// The same for the FP64 step, on the integer pipe: a positive normal number below
+// 3e38 has a high word in [1, hi(3e38)); everything else takes the FP64 comparisons.
+__device__ __forceinline__ void flag_status_f64(const LatticeParams& P, double rho, double theta) {
+    const unsigned top = 0x47ec363cu;   // high word of 3.0e38 (rounded down)
+    const unsigned a = (unsigned)__double2hiint(rho) - 1u, b = (unsigned)__double2hiint(theta) - 1u;
+    if (a >= top - 1u || b >= top - 1u) flag_status<double>(P, rho, theta);
+}
+
 // Float-float numbers: an FP32 pair hi + lo carried through error-free sums
 // (TwoSum) and products (FMA), ~2^-48 relative: FP64-grade sums of FP32 data on
 // the FP32 pipe (GB300's FP64 rate is two operations per SM per cycle).
@@ -453,6 +461,99 @@ struct DirectCore {
 };
 
 // ---------------------------------------------------------------------------
+// FP64 core of the symmetric five-velocity sets (0, +-a, +-b).  The FP64 pipe (two
+// lanes per SM and cycle) bounds these steps, so what counts is the number of FP64
+// instructions: 160 per 2D node against 202 with DirectCore (general velocities and
+// coefficients, FP64 status comparisons).  The rule in constraint form
+// (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b), r_(+-a) = E_a +- O_a,
+// r_(+-b) = E_b +- O_b) takes 19 instructions per axis instead of 31; the column
+// differences T_1 - T_2 come from the row pairs f_i1 + f_i2 that the row sums
+// need anyway; the velocities and factors are FP64 constants of the lattice.
+// Per step: 1024^2 D2Q25 414 -> 312 us (290 us of FP64 issue), 128^2 10.2 -> 8.4 us,
+// the 1000-node D1Q5 tube 4.05 -> 3.2 us.  The identities sum r = 1, sum v^2 r = mu_2
+// hold by construction, so the global sums drift less: mean density of 1024^2 after
+// 40 steps 2e-16 off against 7e-15 (rounded C mu sums), energy 4e-16 against 5e-15.
+// ---------------------------------------------------------------------------
+template <int DIM>
+struct Sym5Core {
+    static constexpr int Q = DIM == 1 ? 5 : 25;
+
+    static __device__ __forceinline__ void axis(const LatticeParams& P, double u, double u2, double th, double th3,
+                                                double th6, double thth3, double (&r)[5]) {
+        const double m2 = u2 + th;
+        const double m3 = u * (u2 + th3);
+        const double m4 = fma(u2, u2 + th6, thth3);
+        const double Ob = fma(-P.da2, u, m3) * P.dkOb;
+        const double Oa = fma(-2.0 * P.db, Ob, u) * P.dkOa;
+        const double Eb = fma(-P.da2, m2, m4) * P.dkEb;
+        const double Ea = fma(-2.0 * P.db2, Eb, m2) * P.dkEa;
+        r[0] = fma(-2.0, Ea + Eb, 1.0);
+        r[1] = Ea + Oa;
+        r[2] = Ea - Oa;
+        r[3] = Eb + Ob;
+        r[4] = Eb - Ob;
+    }
+
+    static __device__ __forceinline__ void collide(double (&f)[Q], const LatticeParams& P, double& rho_o, double& th_o,
+                                                   double& jx_o, double& jy_o, double& e_o) {
+        double S[5], Tp = 0.0, Tq = 0.0, T2 = 0.0, T4 = 0.0;
+        if constexpr (DIM == 2) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const double p = f[5 * i + 1] + f[5 * i + 2], q = f[5 * i + 3] + f[5 * i + 4];
+                S[i] = (f[5 * i] + p) + q;
+                Tp = i ? Tp + p : p;
+                Tq = i ? Tq + q : q;
+                T2 = i ? T2 + f[5 * i + 2] : f[5 * i + 2];
+                T4 = i ? T4 + f[5 * i + 4] : f[5 * i + 4];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) S[i] = f[i];
+        }
+        const double Sp = S[1] + S[2], Sq = S[3] + S[4];
+        const double rho = S[0] + Sp + Sq;
+        const double jx = fma(P.da, S[1] - S[2], P.db * (S[3] - S[4]));
+        double jy = 0.0, e;
+        if constexpr (DIM == 2) {
+            jy = fma(P.da, fma(-2.0, T2, Tp), P.db * fma(-2.0, T4, Tq));
+            e = fma(P.da2, Sp + Tp, P.db2 * (Sq + Tq));
+        } else {
+            e = fma(P.da2, Sp, P.db2 * Sq);
+        }
+        const double inv = 1.0 / rho;
+        const double ux = jx * inv, uy = jy * inv;
+        const double ux2 = ux * ux, uy2 = uy * uy;
+        double th = fma(e, inv, -(DIM == 2 ? ux2 + uy2 : ux2));
+        if constexpr (DIM == 2) th *= 0.5;
+        rho_o = rho;
+        th_o = th;
+        jx_o = jx;
+        jy_o = jy;
+        e_o = e;
+        if (P.isothermal) th = P.theta0;
+        const double th3 = 3.0 * th, th6 = 6.0 * th, thth3 = th3 * th;
+        const double om = P.omega;
+        double rx[5];
+        axis(P, ux, ux2, th, th3, th6, thth3, rx);
+        if constexpr (DIM == 2) {
+            double ry[5];
+            axis(P, uy, uy2, th, th3, th6, thth3, ry);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const double X = rho * rx[i];
+#pragma unroll
+                for (int j = 0; j < 5; ++j)
+                    f[5 * i + j] = fma(om, fma(X, ry[j], -f[5 * i + j]), f[5 * i + j]);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) f[i] = fma(om, fma(rho, rx[i], -f[i]), f[i]);
+        }
+    }
+};
+
+// ---------------------------------------------------------------------------
 // Deviation FP32 core (see the file header for the algebra).
 // ---------------------------------------------------------------------------
 template <int Q1, int DIM>
@@ -589,8 +690,13 @@ __device__ __forceinline__ void node_update(const LatticeParams& P, const S* __r
             }
         }
         double rho, th, jx, jy, e;
-        DirectCore<Q1, DIM>::collide(f, P, rho, th, jx, jy, e);
-        flag_status<double>(P, rho, th);
+        bool sym5 = false;   // uniform over a lattice
+        if constexpr (Q1 == 5) {
+            sym5 = P.sym5;
+            if (sym5) Sym5Core<DIM>::collide(f, P, rho, th, jx, jy, e);
+        }
+        if (!sym5) DirectCore<Q1, DIM>::collide(f, P, rho, th, jx, jy, e);
+        flag_status_f64(P, rho, th);
         if (REDUCE) {
             d.mass = rho;
             d.jx = jx;

@@ -457,6 +457,14 @@ plbm_status plbm_create(const plbm_desc* desc, plbm_handle* out) {
         P.kOb = (float)(1.0 / (2.0 * b * (b * b - a * a)));
         P.kEa = (float)(1.0 / (2.0 * a * a));
         P.kEb = (float)(1.0 / (2.0 * b * b * (b * b - a * a)));
+        P.da = a;
+        P.db = b;
+        P.da2 = a * a;
+        P.db2 = b * b;
+        P.dkOa = 1.0 / (2.0 * a);
+        P.dkOb = 1.0 / (2.0 * b * (b * b - a * a));
+        P.dkEa = 1.0 / (2.0 * a * a);
+        P.dkEb = 1.0 / (2.0 * b * b * (b * b - a * a));
     }
     // Row-paired layout and the two-nodes-per-thread kernel: 2D periodic symmetric
     // five-velocity thermal lattices with an even number of rows, 16/32-bit storage.

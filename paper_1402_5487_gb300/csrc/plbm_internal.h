@@ -49,6 +49,7 @@ struct LatticeParams {
     // sum r = mu_0, sum v^2 r = mu_2, sum v^4 r = mu_4).
     float sa, sb, sa2, sb2;      // a, b, a^2, b^2
     float kOa, kOb, kEa, kEb;    // 1/(2a), 1/(2b(b^2-a^2)), 1/(2a^2), 1/(2b^2(b^2-a^2))
+    double da, db, da2, db2, dkOa, dkOb, dkEa, dkEb;   // the same in FP64
     float w1f[kMaxQ1];           // 1D rest weights r_i(0, theta0)
     float mu0f[kMaxQ1];          // mu_n(0, theta0)
     float W0f[kMaxQ];            // rest equilibrium w0_p (product of 1D weights in 2D)
