@@ -14,6 +14,11 @@ cudaError_t launch_step_f32(const LatticeParams&, const void*, void*, bool, cuda
 cudaError_t launch_step_f16(const LatticeParams&, const void*, void*, bool, cudaStream_t);
 cudaError_t launch_step_bf16(const LatticeParams&, const void*, void*, bool, cudaStream_t);
 
+cudaError_t launch_steps1_f64(const LatticeParams&, const void*, void*, int, cudaStream_t);
+cudaError_t launch_steps1_f32(const LatticeParams&, const void*, void*, int, cudaStream_t);
+cudaError_t launch_steps1_f16(const LatticeParams&, const void*, void*, int, cudaStream_t);
+cudaError_t launch_steps1_bf16(const LatticeParams&, const void*, void*, int, cudaStream_t);
+
 cudaError_t launch_batch_f32(const PairParams*, int, int, int, int, int, const unsigned short*, cudaStream_t);
 cudaError_t launch_batch_f16(const PairParams*, int, int, int, int, int, const unsigned short*, cudaStream_t);
 cudaError_t launch_batch_bf16(const PairParams*, int, int, int, int, int, const unsigned short*, cudaStream_t);
@@ -81,6 +86,40 @@ cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void*
         case kF32: return launch_step_f32(P, src, dst, reduce, stream);
         case kF16Dev: return launch_step_f16(P, src, dst, reduce, stream);
         case kBF16Dev: return launch_step_bf16(P, src, dst, reduce, stream);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// A launch of k steps takes `launch` us (launch, load, store) plus k times a warp's
+// arithmetic, which four warps per SM do side by side (one per SM quarter; an FP64
+// instruction occupies a quarter for 64 cycles) and further ones in rounds.  The
+// constants are fitted to D1Q5 {0, +-1, +-3}, periodic, us per step with one step per
+// launch (graph replays) and with the k this rule takes: FP64 1000 nodes 4.04 (3.2
+// before the symmetric core alone) -> 1.87, 20,000 nodes 5.46 -> 3.54, 100,000 nodes
+// 18.95 -> 14.70 (k = 1); FP32 1.74 -> 0.53, 1.87 -> 0.91, 2.32 -> 1.55.
+int steps_per_launch(int prec, const LatticeParams& P) {
+    if (P.dim != 1) return 1;
+    const int w = halo1(P), sms = device_sm_count();
+    const double launch = 1.5, latency = prec == kF64 ? 1.5 : 0.25;
+    auto time = [&](int k) {   // per step
+        const int m = k == 1 ? 32 : 32 - 2 * w * k;
+        const long long warps = (P.nx + m - 1) / m, rounds = (warps + 4LL * sms - 1) / (4LL * sms);
+        const double work = rounds * (prec == kF64 ? 1.5 : k > 1 ? 0.09 : 0.19);   // k = 1: k_stream_collide
+        const double step = work > latency ? work : latency;
+        return (launch + k * step) / k;
+    };
+    int best = 1;
+    for (int k = 2; k <= 16 && 32 - 2 * w * k >= 2; k *= 2)   // divisors of half a captured run of 32 steps
+        if (time(k) < time(best)) best = k;
+    return best;
+}
+
+cudaError_t launch_steps1(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
+    switch (prec) {
+        case kF64: return launch_steps1_f64(P, src, dst, steps, stream);
+        case kF32: return launch_steps1_f32(P, src, dst, steps, stream);
+        case kF16Dev: return launch_steps1_f16(P, src, dst, steps, stream);
+        case kBF16Dev: return launch_steps1_bf16(P, src, dst, steps, stream);
     }
     return cudaErrorInvalidValue;
 }

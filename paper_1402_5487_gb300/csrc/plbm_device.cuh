@@ -43,15 +43,25 @@ namespace plbm {
 // 123.2 -> 120.6 us, FP16 69.7 -> 67.3 us, 512^2 FP32 (graph) 6.56 -> 6.29 us.
 // Grids of fewer than kDependentThreads threads leave slots free for several
 // waiting grids at once, which then crowd the running one (128^2 FP64: 10.2 ->
-// 16.4 us a step); they are launched plainly, as are the persistent batch kernels,
-// which leave no slot free (174 us a step either way).
+// 16.4 us a step): 16/32-bit ones are launched plainly, FP64 ones, whose arithmetic
+// takes longer than a launch, say so only after it (step_end; 128^2 FP64 8.35 ->
+// 7.95 us a step, tube launches of four steps 8.1 -> 7.6 us).  The persistent batch
+// kernels, which leave no slot free, are launched plainly (174 us a step either way).
 // ---------------------------------------------------------------------------
 constexpr long long kDependentThreads = 1 << 16;
 __device__ __forceinline__ void step_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// FP64 kernels: the trigger at the start of a grid of more than one wave whatever the
+// registers (2^18 threads and up), after the arithmetic of a smaller one.
+__device__ __forceinline__ bool step_large() {
+    return (long long)gridDim.x * gridDim.y * gridDim.z * blockDim.x >= 1 << 18;
+}
+__device__ __forceinline__ void step_end() {
+    if (!step_large()) step_begin();
+}
 
 template <class... P, class... A>
-cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+cudaError_t launch_dependent(bool small_too, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -60,7 +70,7 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, cudaSt
     cfg.blockDim = block;
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = (long long)grid.x * grid.y * grid.z * block.x >= kDependentThreads ? 1 : 0;
+    cfg.numAttrs = small_too || (long long)grid.x * grid.y * grid.z * block.x >= kDependentThreads ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
@@ -460,16 +470,28 @@ struct DirectCore {
     }
 };
 
+// 1 / x in FP64 by one step of Householder's third-order iteration y (1 + e + e^2),
+// e = 1 - x y, from the hardware's 23-bit estimate: three FP64 instructions, within
+// a few 2^-60 of the exact value before the last rounding.  Outside the normal
+// range (zero, subnormal, huge, infinite, NaN) the division.
+__device__ __forceinline__ double recip_f64(double x) {
+    if (((unsigned)__double2hiint(x) & 0x7fffffffu) - 0x00200000u >= 0x7fa00000u) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 // ---------------------------------------------------------------------------
 // FP64 core of the symmetric five-velocity sets (0, +-a, +-b).  The FP64 pipe (two
 // lanes per SM and cycle) bounds these steps, so what counts is the number of FP64
-// instructions: 160 per 2D node against 202 with DirectCore (general velocities and
+// instructions: 150 per 2D node against 202 with DirectCore (general velocities and
 // coefficients, FP64 status comparisons).  The rule in constraint form
 // (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b), r_(+-a) = E_a +- O_a,
-// r_(+-b) = E_b +- O_b) takes 19 instructions per axis instead of 31; the column
+// r_(+-b) = E_b +- O_b) takes 16 instructions per axis instead of 31; the column
 // differences T_1 - T_2 come from the row pairs f_i1 + f_i2 that the row sums
 // need anyway; the velocities and factors are FP64 constants of the lattice.
-// Per step: 1024^2 D2Q25 414 -> 312 us (290 us of FP64 issue), 128^2 10.2 -> 8.4 us,
+// Per step: 1024^2 D2Q25 414 -> 297 us (270 us of FP64 issue), 128^2 10.2 -> 7.9 us,
 // the 1000-node D1Q5 tube 4.05 -> 3.2 us.  The identities sum r = 1, sum v^2 r = mu_2
 // hold by construction, so the global sums drift less: mean density of 1024^2 after
 // 40 steps 2e-16 off against 7e-15 (rounded C mu sums), energy 4e-16 against 5e-15.
@@ -478,20 +500,24 @@ template <int DIM>
 struct Sym5Core {
     static constexpr int Q = DIM == 1 ? 5 : 25;
 
-    static __device__ __forceinline__ void axis(const LatticeParams& P, double u, double u2, double th, double th3,
-                                                double th6, double thth3, double (&r)[5]) {
+    // Products that meet a sum are formed by __dmul_rn, so that every kernel rounds alike.
+    // mu_3 = u A and mu_4 = A^2 - 6 theta^2 with A = u^2 + 3 theta; sixth2 = 6 theta^2.
+    static __device__ __forceinline__ void axis(const LatticeParams& P, double u, double u2, double th, double sixth2,
+                                                double (&r)[5]) {
+        const double A = fma(3.0, th, u2);
         const double m2 = u2 + th;
-        const double m3 = u * (u2 + th3);
-        const double m4 = fma(u2, u2 + th6, thth3);
-        const double Ob = fma(-P.da2, u, m3) * P.dkOb;
-        const double Oa = fma(-2.0 * P.db, Ob, u) * P.dkOa;
-        const double Eb = fma(-P.da2, m2, m4) * P.dkEb;
-        const double Ea = fma(-2.0 * P.db2, Eb, m2) * P.dkEa;
+        const double m3 = __dmul_rn(u, A);
+        const double m4 = fma(A, A, -sixth2);
+        const double yb = fma(-P.da2, u, m3);     // O_b / kOb
+        const double ya = fma(-P.dcb, yb, u);     // O_a / kOa
+        const double zb = fma(-P.da2, m2, m4);    // E_b / kEb
+        const double za = fma(-P.dcb, zb, m2);    // E_a / kEa
+        const double Ea = __dmul_rn(za, P.dkEa), Eb = __dmul_rn(zb, P.dkEb);
         r[0] = fma(-2.0, Ea + Eb, 1.0);
-        r[1] = Ea + Oa;
-        r[2] = Ea - Oa;
-        r[3] = Eb + Ob;
-        r[4] = Eb - Ob;
+        r[1] = fma(P.dkOa, ya, Ea);
+        r[2] = fma(-P.dkOa, ya, Ea);
+        r[3] = fma(P.dkOb, yb, Eb);
+        r[4] = fma(-P.dkOb, yb, Eb);
     }
 
     static __device__ __forceinline__ void collide(double (&f)[Q], const LatticeParams& P, double& rho_o, double& th_o,
@@ -513,35 +539,35 @@ struct Sym5Core {
         }
         const double Sp = S[1] + S[2], Sq = S[3] + S[4];
         const double rho = S[0] + Sp + Sq;
-        const double jx = fma(P.da, S[1] - S[2], P.db * (S[3] - S[4]));
+        const double jx = fma(P.da, S[1] - S[2], __dmul_rn(P.db, S[3] - S[4]));
         double jy = 0.0, e;
         if constexpr (DIM == 2) {
-            jy = fma(P.da, fma(-2.0, T2, Tp), P.db * fma(-2.0, T4, Tq));
-            e = fma(P.da2, Sp + Tp, P.db2 * (Sq + Tq));
+            jy = fma(P.da, fma(-2.0, T2, Tp), __dmul_rn(P.db, fma(-2.0, T4, Tq)));
+            e = fma(P.da2, Sp + Tp, __dmul_rn(P.db2, Sq + Tq));
         } else {
-            e = fma(P.da2, Sp, P.db2 * Sq);
+            e = fma(P.da2, Sp, __dmul_rn(P.db2, Sq));
         }
-        const double inv = 1.0 / rho;
-        const double ux = jx * inv, uy = jy * inv;
-        const double ux2 = ux * ux, uy2 = uy * uy;
+        const double inv = recip_f64(rho);
+        const double ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
+        const double ux2 = __dmul_rn(ux, ux), uy2 = __dmul_rn(uy, uy);
         double th = fma(e, inv, -(DIM == 2 ? ux2 + uy2 : ux2));
-        if constexpr (DIM == 2) th *= 0.5;
+        if constexpr (DIM == 2) th = __dmul_rn(th, 0.5);
         rho_o = rho;
         th_o = th;
         jx_o = jx;
         jy_o = jy;
         e_o = e;
         if (P.isothermal) th = P.theta0;
-        const double th3 = 3.0 * th, th6 = 6.0 * th, thth3 = th3 * th;
+        const double sixth2 = __dmul_rn(__dmul_rn(6.0, th), th);
         const double om = P.omega;
         double rx[5];
-        axis(P, ux, ux2, th, th3, th6, thth3, rx);
+        axis(P, ux, ux2, th, sixth2, rx);
         if constexpr (DIM == 2) {
             double ry[5];
-            axis(P, uy, uy2, th, th3, th6, thth3, ry);
+            axis(P, uy, uy2, th, sixth2, ry);
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
-                const double X = rho * rx[i];
+                const double X = __dmul_rn(rho, rx[i]);
 #pragma unroll
                 for (int j = 0; j < 5; ++j)
                     f[5 * i + j] = fma(om, fma(X, ry[j], -f[5 * i + j]), f[5 * i + j]);
@@ -697,6 +723,7 @@ __device__ __forceinline__ void node_update(const LatticeParams& P, const S* __r
         }
         if (!sym5) DirectCore<Q1, DIM>::collide(f, P, rho, th, jx, jy, e);
         flag_status_f64(P, rho, th);
+        step_end();
         if (REDUCE) {
             d.mass = rho;
             d.jx = jx;
@@ -752,7 +779,7 @@ template <typename S, int Q1, int DIM, bool REDUCE>
 __global__ void __launch_bounds__(kBlockX)
 k_stream_collide(const __grid_constant__ LatticeParams P, const S* __restrict__ src,
                  S* __restrict__ dst) {
-    step_begin();
+    if (sizeof(S) < 8 || step_large()) step_begin();
     const int x = blockIdx.x * (REDUCE ? kBlockX : (int)blockDim.x) + threadIdx.x;
     const int y = blockIdx.y;
     step_wait();
@@ -771,6 +798,122 @@ k_stream_collide(const __grid_constant__ LatticeParams P, const S* __restrict__ 
         else
             block_reduce_diagf<kBlockX>(df, (double)DIM * P.theta0, P.partials + (long long)blk * kPartialStride);
     }
+}
+
+// ---------------------------------------------------------------------------
+// Several steps of a 1D lattice in one launch.  A step of a short lattice (the
+// 1000-node tube) is one warp's work per SM, and of its 3.2 us only 0.6 are the
+// arithmetic; the rest is the launch and the way to memory and back.  Here a warp
+// loads the 32 nodes around m = 32 - 2 w steps output nodes (w = max|v|), keeps
+// them in registers, pulls by shuffles and steps them `steps` times; the outer w
+// lanes of each side hold no valid state after each step and are dropped.  Lanes
+// beyond a fixed end hold the end's populations, which never change.  The arithmetic
+// done twice is free while every warp has an SM quarter to itself; steps_per_launch
+// weighs it against the launches saved.
+// ---------------------------------------------------------------------------
+template <typename S>
+struct Node1 {   // how one node's populations live between two steps
+    using A = float;
+    static __device__ __forceinline__ A load(const S* p) { return Storage<S>::load(p); }
+    static __device__ __forceinline__ A stored(A v) {   // the value a store and a load would give
+        S s;
+        Storage<S>::store(&s, v);
+        return v_of(s);
+    }
+    static __device__ __forceinline__ A v_of(float s) { return s; }
+    static __device__ __forceinline__ A v_of(__half s) { return __half2float(s); }
+    static __device__ __forceinline__ A v_of(__nv_bfloat16 s) { return __bfloat162float(s); }
+};
+template <>
+struct Node1<double> {
+    using A = double;
+    static __device__ __forceinline__ A load(const double* p) { return __ldg(p); }
+    static __device__ __forceinline__ A stored(A v) { return v; }
+};
+
+constexpr int kWarps1 = 4;   // most independent warps per block, one per SM quarter
+
+template <typename S, int Q1, bool SYM5>
+__global__ void __launch_bounds__(32 * kWarps1) k_steps1(const __grid_constant__ LatticeParams P,
+                                                         const S* __restrict__ src, S* __restrict__ dst, int steps,
+                                                         int w, int m) {
+    using A = typename Node1<S>::A;
+    const int lane = threadIdx.x & 31;
+    const long long first = (long long)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * m;   // first output node
+    if (first >= P.nx) return;
+    const int x = (int)first + lane - w * steps;
+    const bool inside = x >= 0 && x < P.nx;
+    A f[Q1];
+    step_wait();
+    if (!inside && P.fixed_ends) {
+#pragma unroll
+        for (int i = 0; i < Q1; ++i) {
+            if constexpr (sizeof(S) == 8) f[i] = x < 0 ? P.ghostL[i] : P.ghostR[i];
+            else f[i] = x < 0 ? P.ghostLg[i] : P.ghostRg[i];
+        }
+    } else {
+        int s = x % P.nx;
+        s = s < 0 ? s + P.nx : s;
+#pragma unroll
+        for (int i = 0; i < Q1; ++i) f[i] = Node1<S>::load(src + i * P.plane + s);
+    }
+    for (int k = 1; k <= steps; ++k) {
+        A g[Q1];
+#pragma unroll
+        for (int i = 0; i < Q1; ++i) g[i] = SYM5 && i == 0 ? f[0] : __shfl_sync(0xffffffffu, f[i], lane - P.v[i]);
+        A rho, th, jx, jy, e;
+        if constexpr (sizeof(S) == 8) {
+            if constexpr (SYM5) Sym5Core<1>::collide(g, P, rho, th, jx, jy, e);
+            else DirectCore<Q1, 1>::collide(g, P, rho, th, jx, jy, e);
+        } else {
+            A drho;
+            DeviationCore<Q1, 1>::collide(g, P, drho, th, jx, jy, e);
+            rho = 1.0f + drho;
+        }
+        if (inside || !P.fixed_ends) {
+            if (lane >= w * k && lane < 32 - w * k) {
+                if constexpr (sizeof(S) == 8) flag_status_f64(P, rho, th);
+                else flag_status<float>(P, rho, th);
+            }
+#pragma unroll
+            for (int i = 0; i < Q1; ++i) f[i] = Node1<S>::stored(g[i]);
+        }
+    }
+    step_begin();   // after the arithmetic, as in step_end
+    if (inside && lane >= w * steps && lane < w * steps + m) {
+#pragma unroll
+        for (int i = 0; i < Q1; ++i) Storage<S>::store(dst + i * P.plane + x, f[i]);
+    }
+}
+
+inline int halo1(const LatticeParams& P) {
+    int w = 0;
+    for (int i = 0; i < P.q1; ++i) w = P.v[i] > w ? P.v[i] : (-P.v[i] > w ? -P.v[i] : w);
+    return w;
+}
+
+template <typename S>
+cudaError_t launch_steps1_t(const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
+    const int w = halo1(P), m = 32 - 2 * w * steps;
+    if (P.dim != 1 || steps < 1 || m < 1) return cudaErrorInvalidValue;
+    // FP64 warps do best spread over the SMs (1000 nodes 1.87 us a step against 2.00), the
+    // others in few blocks (100,000 nodes 1.55 us against 3.34)
+    const int warps = sizeof(S) == 8 ? 1 : kWarps1;
+    const int blocks = ((P.nx + m - 1) / m + warps - 1) / warps;
+    const S* s = static_cast<const S*>(src);
+    S* t = static_cast<S*>(dst);
+    if constexpr (sizeof(S) == 8) {
+        if (P.sym5) return launch_dependent(true, k_steps1<S, 5, true>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+    }
+    switch (P.q1) {
+        case 3: return launch_dependent(true, k_steps1<S, 3, false>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+        case 4: return launch_dependent(true, k_steps1<S, 4, false>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+        case 5: return launch_dependent(true, k_steps1<S, 5, false>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+        case 6: return launch_dependent(true, k_steps1<S, 6, false>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+        case 7: return launch_dependent(true, k_steps1<S, 7, false>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+        case 8: return launch_dependent(true, k_steps1<S, 8, false>, blocks, 32 * warps, stream, P, s, t, steps, w, m);
+    }
+    return cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------
@@ -822,12 +965,13 @@ cudaError_t launch_step_t(const LatticeParams& P, const void* src, void* dst, bo
     if (!reduce && (long long)((P.nx + kBlockX - 1) / kBlockX) * P.ny < 2LL * device_sm_count()) bx = 32;
     dim3 grid((P.nx + bx - 1) / bx, P.ny);
     dim3 block(bx);
+    constexpr bool f64 = sizeof(S) == 8;
     const S* s = static_cast<const S*>(src);
     S* t = static_cast<S*>(dst);
 #define PLBM_LAUNCH(Q1v, DIMv)                                                              \
     if (P.q1 == Q1v && P.dim == DIMv) {                                                     \
-        return reduce ? launch_dependent(k_stream_collide<S, Q1v, DIMv, true>, grid, block, stream, P, s, t)    \
-                      : launch_dependent(k_stream_collide<S, Q1v, DIMv, false>, grid, block, stream, P, s, t);  \
+        return reduce ? launch_dependent(f64, k_stream_collide<S, Q1v, DIMv, true>, grid, block, stream, P, s, t)    \
+                      : launch_dependent(f64, k_stream_collide<S, Q1v, DIMv, false>, grid, block, stream, P, s, t);  \
     }
     PLBM_LAUNCH(3, 1)
     PLBM_LAUNCH(4, 1)

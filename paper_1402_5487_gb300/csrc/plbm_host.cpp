@@ -465,6 +465,7 @@ plbm_status plbm_create(const plbm_desc* desc, plbm_handle* out) {
         P.dkOb = 1.0 / (2.0 * b * (b * b - a * a));
         P.dkEa = 1.0 / (2.0 * a * a);
         P.dkEb = 1.0 / (2.0 * b * b * (b * b - a * a));
+        P.dcb = 1.0 / (b * b - a * a);
     }
     // Row-paired layout and the two-nodes-per-thread kernel: 2D periodic symmetric
     // five-velocity thermal lattices with an even number of rows, 16/32-bit storage.
@@ -667,11 +668,19 @@ plbm_status plbm_step(plbm_handle hh, long n) {
     const int ce = h->desc.check_every;
     long s = 0;
     const long long nodes = (long long)h->P.nx * h->P.ny * h->P.nz;
+    const int per = h->P.dim == 1 ? plbm::steps_per_launch(h->prec, h->P) : 1;   // steps of one launch
+    auto launch = [&](int c, int k, cudaStream_t stream) {   // k <= per steps from array c
+        if (h->P.dim == 3) return plbm::launch_step3(h->prec, h->P, h->f[c], h->f[c ^ 1], stream);
+        if (k > 1) return plbm::launch_steps1(h->prec, h->P, h->f[c], h->f[c ^ 1], k, stream);
+        return plbm::launch_step(h->prec, h->P, h->f[c], h->f[c ^ 1], false, stream);
+    };
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (ce == 0 && nodes <= kGraphMaxNodes && n >= 2 * kGraphSteps &&
         cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         // launch-bound lattices: replay a run of kGraphSteps steps, captured on a
-        // private stream (any stream, the legacy default one included, can launch it)
+        // private stream (any stream, the legacy default one included, can launch it);
+        // its launches are even in number (per divides kGraphSteps / 2), so that a
+        // replay leaves the current array unchanged
         for (; s + kGraphSteps <= n; s += kGraphSteps) {
             cudaGraphExec_t& g = h->sgraph[h->cur];
             if (!g) {
@@ -679,9 +688,8 @@ plbm_status plbm_step(plbm_handle hh, long n) {
                 cudaGraph_t graph = nullptr;
                 CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
                 cudaError_t el = cudaSuccess;
-                for (int k = 0, c = h->cur; k < kGraphSteps && el == cudaSuccess; ++k, c ^= 1)
-                    el = h->P.dim == 3 ? plbm::launch_step3(h->prec, h->P, h->f[c], h->f[c ^ 1], h->cap)
-                                       : plbm::launch_step(h->prec, h->P, h->f[c], h->f[c ^ 1], false, h->cap);
+                for (int k = 0, c = h->cur; k < kGraphSteps && el == cudaSuccess; k += per, c ^= 1)
+                    el = launch(c, per, h->cap);
                 const cudaError_t ec = cudaStreamEndCapture(h->cap, &graph);
                 const cudaError_t ei = (el == cudaSuccess && ec == cudaSuccess)
                                            ? cudaGraphInstantiate(&g, graph, 0) : cudaSuccess;
@@ -694,14 +702,14 @@ plbm_status plbm_step(plbm_handle hh, long n) {
             h->steps += kGraphSteps;
         }
     }
-    for (; s < n; ++s) {
-        if (h->P.dim == 3)
-            CK(plbm::launch_step3(h->prec, h->P, h->f[h->cur], h->f[h->cur ^ 1], h->stream));
-        else
-            CK(plbm::launch_step(h->prec, h->P, h->f[h->cur], h->f[h->cur ^ 1], false, h->stream));
+    while (s < n) {
+        long k = std::min<long>(per, n - s);
+        if (ce > 0) k = std::min<long>(k, ce - s % ce);
+        CK(launch(h->cur, (int)k, h->stream));
         h->cur ^= 1;
-        ++h->steps;
-        if (ce > 0 && ((s + 1) % ce == 0) && s + 1 < n) {
+        h->steps += k;
+        s += k;
+        if (ce > 0 && s % ce == 0 && s < n) {
             st = plbm_check(hh);
             if (st != PLBM_OK) return st;
         }

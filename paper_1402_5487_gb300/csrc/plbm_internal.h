@@ -49,7 +49,8 @@ struct LatticeParams {
     // sum r = mu_0, sum v^2 r = mu_2, sum v^4 r = mu_4).
     float sa, sb, sa2, sb2;      // a, b, a^2, b^2
     float kOa, kOb, kEa, kEb;    // 1/(2a), 1/(2b(b^2-a^2)), 1/(2a^2), 1/(2b^2(b^2-a^2))
-    double da, db, da2, db2, dkOa, dkOb, dkEa, dkEb;   // the same in FP64
+    double da, db, da2, db2, dkOa, dkOb, dkEa, dkEb;   // the same in FP64 ...
+    double dcb;                  // ... and 1 / (b^2 - a^2) = 2 b kOb = 2 b^2 kEb
     float w1f[kMaxQ1];           // 1D rest weights r_i(0, theta0)
     float mu0f[kMaxQ1];          // mu_n(0, theta0)
     float W0f[kMaxQ];            // rest equilibrium w0_p (product of 1D weights in 2D)
@@ -231,6 +232,10 @@ void set_thread_error(const char* msg);
 // on `stream` and return the launch error.
 cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void* dst,
                         bool reduce, cudaStream_t stream);
+// 1D lattices: the number of steps best taken by one launch (1: launch_step), and a
+// launch that takes `steps` of them (2 <= steps <= that number).
+int steps_per_launch(int prec, const LatticeParams& P);
+cudaError_t launch_steps1(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream);
 // Rows [y0, y1) (y1 < 0: to the last row); field pointers index the whole lattice.
 // Batched step of 2D lattices in the plain layout, all of precision prec and
 // q1 velocities per axis (q1 = 3, 4 or 5): tiles of kBlockX nodes of one row.

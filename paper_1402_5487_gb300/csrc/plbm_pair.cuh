@@ -485,8 +485,8 @@ cudaError_t launch_step_sym5_t(const LatticeParams& L, const void* src, void* ds
     dim3 grid((P.nx + bx - 1) / bx, P.ny);
     const S* s = static_cast<const S*>(src);
     S* t = static_cast<S*>(dst);
-    return reduce ? launch_dependent(k_stream_collide_sym5<S, true>, grid, kBlockX, stream, P, s, t)
-                  : launch_dependent(k_stream_collide_sym5<S, false>, grid, bx, stream, P, s, t);
+    return reduce ? launch_dependent(false, k_stream_collide_sym5<S, true>, grid, kBlockX, stream, P, s, t)
+                  : launch_dependent(false, k_stream_collide_sym5<S, false>, grid, bx, stream, P, s, t);
 }
 
 template <typename S>
@@ -501,12 +501,12 @@ cudaError_t launch_step_pair_t(const LatticeParams& L, const void* src, void* ds
         if (!reduce) {
             const int tiles_x = (P.nx + kPair2Block - 1) / kPair2Block;
             const int ntiles = tiles_x * P.half_ny;
-            return launch_dependent(k_stream_collide_pair2<S>, (ntiles + 1) / 2, kPair2Block, stream, P, s, t, tiles_x,
+            return launch_dependent(false, k_stream_collide_pair2<S>, (ntiles + 1) / 2, kPair2Block, stream, P, s, t, tiles_x,
                                     ntiles);
         }
     }
-    return reduce ? launch_dependent(k_stream_collide_pair<S, true>, grid, kBlockX, stream, P, s, t)
-                  : launch_dependent(k_stream_collide_pair<S, false>, grid, kBlockX, stream, P, s, t);
+    return reduce ? launch_dependent(false, k_stream_collide_pair<S, true>, grid, kBlockX, stream, P, s, t)
+                  : launch_dependent(false, k_stream_collide_pair<S, false>, grid, kBlockX, stream, P, s, t);
 }
 
 // ---------------------------------------------------------------------------

@@ -1262,9 +1262,9 @@ cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void
         const double* a = static_cast<const double*>(src);
         double* b = static_cast<double*>(dst);
         switch (P.q1) {
-            case 5: return launch_dependent(k_stream_collide3_f64q<5>, grid3(P), kB3, s, P, a, b);
-            case 4: return launch_dependent(k_stream_collide3_f64q<4>, grid3(P), kB3, s, P, a, b);
-            case 3: return launch_dependent(k_stream_collide3_f64q<3>, grid3(P), kB3, s, P, a, b);
+            case 5: return launch_dependent(false, k_stream_collide3_f64q<5>, grid3(P), kB3, s, P, a, b);
+            case 4: return launch_dependent(false, k_stream_collide3_f64q<4>, grid3(P), kB3, s, P, a, b);
+            case 3: return launch_dependent(false, k_stream_collide3_f64q<3>, grid3(P), kB3, s, P, a, b);
         }
         return cudaErrorInvalidValue;
     }
@@ -1275,21 +1275,21 @@ cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void
     if (P.zpaired) {
         const dim3 g((P.nx + kZpairBlock - 1) / kZpairBlock, P.ny, P.half_nz);
         if (prec == kF16Dev)
-            return launch_dependent(k_stream_collide3_zpair<__half>, g, kZpairBlock, s, P, f16, static_cast<__half*>(dst));
+            return launch_dependent(false, k_stream_collide3_zpair<__half>, g, kZpairBlock, s, P, f16, static_cast<__half*>(dst));
         if (prec == kBF16Dev)
-            return launch_dependent(k_stream_collide3_zpair<__nv_bfloat16>, g, kZpairBlock, s, P, b16,
+            return launch_dependent(false, k_stream_collide3_zpair<__nv_bfloat16>, g, kZpairBlock, s, P, b16,
                                     static_cast<__nv_bfloat16*>(dst));
         return cudaErrorInvalidValue;
     }
     switch (prec) {
         case kF32:
-            return launch_dependent(k_stream_collide3_split<float>,
+            return launch_dependent(false, k_stream_collide3_split<float>,
                                     dim3((P.nx + kSplitNodes - 1) / kSplitNodes, P.ny, P.nz), kSplitThreads, s, P, f32,
                                     static_cast<float*>(dst));
         case kF16Dev:
-            return launch_dependent(k_stream_collide3<__half>, grid3(P), kB3, s, P, f16, static_cast<__half*>(dst));
+            return launch_dependent(false, k_stream_collide3<__half>, grid3(P), kB3, s, P, f16, static_cast<__half*>(dst));
         case kBF16Dev:
-            return launch_dependent(k_stream_collide3<__nv_bfloat16>, grid3(P), kB3, s, P, b16,
+            return launch_dependent(false, k_stream_collide3<__nv_bfloat16>, grid3(P), kB3, s, P, b16,
                                     static_cast<__nv_bfloat16*>(dst));
     }
     return cudaErrorInvalidValue;

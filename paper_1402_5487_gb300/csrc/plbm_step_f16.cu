@@ -18,6 +18,9 @@ cudaError_t launch_batch_f16(const PairParams* inst, int ninst, int total_tiles,
 cudaError_t batch_occupancy_f16(int block_x, int* blocks_per_sm) {
     return batch_occupancy_t<__half>(block_x, blocks_per_sm);
 }
+cudaError_t launch_steps1_f16(const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
+    return launch_steps1_t<__half>(P, src, dst, steps, stream);
+}
 cudaError_t launch_batch_node_f16(int q1, const LatticeParams* inst, const NodeSpan* span, int total_tiles, int ctas,
                                  int parity, const unsigned short* tile_inst, cudaStream_t stream) {
     return launch_batch_node_t<__half>(q1, inst, span, total_tiles, ctas, parity, tile_inst, stream);

@@ -8,6 +8,9 @@ cudaError_t launch_step_f64(const LatticeParams& P, const void* src, void* dst, 
                              cudaStream_t stream) {
     return launch_step_t<double>(P, src, dst, reduce, stream);
 }
+cudaError_t launch_steps1_f64(const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
+    return launch_steps1_t<double>(P, src, dst, steps, stream);
+}
 cudaError_t launch_batch_node_f64(int q1, const LatticeParams* inst, const NodeSpan* span, int total_tiles, int ctas,
                                  int parity, const unsigned short* tile_inst, cudaStream_t stream) {
     return launch_batch_node_t<double>(q1, inst, span, total_tiles, ctas, parity, tile_inst, stream);

@@ -788,3 +788,40 @@ def test_f64_five_velocity_steps_match_oracle(dim, v, theta0, omega, iso, fixed,
     _, fo, mo = oracle_run(dim, v, omega, nx, ny, fields, 60, theta0=theta0, isothermal=iso, **ends)
     assert rel(fg, fo) <= TOL64
     assert O.rel_err(mg[0], mo[0]) <= TOL64 and O.rel_err(mg[3], mo[3]) <= TOL64
+
+
+# Several 1D steps per launch (a warp steps the 32 nodes around its outputs) equal the
+# oracle and, for every split of the same number of steps, each other bit for bit: every
+# q1, periodic and fixed ends, thermal and isothermal, lattices shorter than a warp,
+# of one tile more or less, and long ones that take one step per launch.  (The
+# six-velocity set is linearly unstable, |lambda| = 1.17: any rounding grows 8e4-fold in
+# 71 steps, so it is held to the bitwise comparison alone.)
+@pytest.mark.parametrize("v,theta0,iso,tol32", [((0, 1, -1), 1 / 3, True, 2e-6), ((1, -1, 3, -3), 4 / 3, True, 2e-6),
+                                                ((0, 1, -1, 3, -3), 1.0, False, 1e-5), ((0, 3, -3, 1, -1), 1.0, False, 1e-5),
+                                                ((1, 0, -1, 3, -3), 1.0, False, 1e-5), ((0, 1, -1, 2, -2, 3), 0.8, False, 1e-5),
+                                                ((0, 1, -1, 2, -2, 3, -3), 1.0, False, 1e-5),
+                                                ((0, 1, -1, 2, -2, 3, -3, 4), 1.0, False, 1e-5)])
+@pytest.mark.parametrize("n,bc", [(5, "periodic"), (31, "fixed"), (96, "periodic"), (97, "fixed"), (1000, "fixed"),
+                                  (40000, "periodic")])
+def test_steps_of_one_launch_match_oracle_and_single_steps(v, theta0, iso, tol32, n, bc):
+    x = np.arange(n)
+    rho = (1 + 0.01 * np.sin(2 * np.pi * x / n))[None]
+    ux = (0.01 * np.cos(2 * np.pi * x / n))[None]
+    th = np.full((1, n), theta0)
+    ends = {"left_state": (1.0, 0.01, theta0), "right_state": (1.0, 0.01, theta0)} if bc == "fixed" else {}
+    lat = O.Lattice(1, v, 1.1, n, 1, bc=bc, theta0=theta0, isothermal=iso, **ends)
+    fo = lat.run(lat.init(rho, ux, 0 * ux, th), 71)
+    stable = plbm.linear_stability(1, v, 1.1, theta0, 0.01, isothermal=iso) <= 1 + 1e-9
+    for prec, tol in (("f64", TOL64), ("f32", tol32), ("f16dev", 2e-2), ("bf16dev", 1e-1)):
+        got = []
+        for parts in ((71,), (64, 7), (1,) * 71, (3, 2, 5, 61)):
+            s = plbm.Solver(1, v, 1.1, n, 1, theta0=theta0, prec=prec, bc=bc, isothermal=iso, **ends)
+            s.init(rho, ux, None, None if iso else th)
+            for k in parts:
+                s.step(k)
+            assert s.check() == plbm.PLBM_OK or not stable
+            got.append(s.get_populations())
+            s.close()
+        assert rel(got[0], np.asarray(fo).reshape(got[0].shape)) <= tol or not stable
+        for g in got[1:]:
+            assert np.array_equal(got[0], g, equal_nan=True)
