@@ -44,8 +44,18 @@ THETA0 = 1.0
 ELEM = {"f64": 8, "f32": 4, "f16dev": 2, "bf16dev": 2}
 
 
-KERNEL_NAME = {"f32": "k_stream_collide_pair<float>", "f16dev": "k_stream_collide_pair2<__half>",
+KERNEL_NAME = {"f32": "k_two_steps<float2,96,2>", "f16dev": "k_stream_collide_pair2<__half>",
                "bf16dev": "k_stream_collide_pair<__nv_bfloat16>", "f64": "k_stream_collide<double,5,2>"}
+
+
+def launches(prec, L, steps):
+    """Step kernels that ``steps`` steps of the L x L lattice in one call launch: FP32
+    lattices beyond the second-level cache take two steps a launch, in as many launches as
+    steps modulo 2."""
+    if prec != "f32" or L < 1024:
+        return steps
+    n = (steps + 1) // 2
+    return n + ((n ^ steps) & 1)
 
 
 def kernel_fingerprint(sources):
@@ -827,7 +837,8 @@ def main():
     healthy = solver.check() == 0
     solver.close()
     t_max, value = replica_throughput(torch, t, L * L * args.steps, dist)
-    per_launch = t / args.steps
+    n_launches = launches(args.prec, L, args.steps)
+    per_launch = t / n_launches
     alg_bytes = 2 * q * ELEM[args.prec] * L * L
     peak, peak_kind = read_peaks()
     achieved = alg_bytes / per_launch / 1e9
@@ -888,7 +899,7 @@ def main():
                 "repeats": {"n": REPEATS, "reported": "median",
                             "ms_per_step_each": [r / args.steps * 1e3 for r in runs],
                             "spread": (max(runs) - min(runs)) / t},
-                "e2e": e2e, "gpu_launches": args.steps, "clocks": clock_info,
+                "e2e": e2e, "gpu_launches": n_launches, "clocks": clock_info,
                 "cpu_baseline": cpu, "variants": variants, "variant_summary": variant_summary(variants, peak)}
         print(json.dumps(json_safe(line)))
     if dist is not None:

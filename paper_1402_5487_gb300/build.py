@@ -35,7 +35,7 @@ SOURCES = [
     "plbm_ce.cu",
     "plbm_surrogate.cpp",
 ]
-HEADERS = ["plbm_internal.h", "plbm_device.cuh", "plbm_pair.cuh"]
+HEADERS = ["plbm_internal.h", "plbm_device.cuh", "plbm_pair.cuh", "plbm_fuse.cuh"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -14,6 +14,8 @@ cudaError_t launch_step_f32(const LatticeParams&, const void*, void*, bool, cuda
 cudaError_t launch_step_f16(const LatticeParams&, const void*, void*, bool, cudaStream_t);
 cudaError_t launch_step_bf16(const LatticeParams&, const void*, void*, bool, cudaStream_t);
 
+bool two_steps_f32(const LatticeParams&);
+cudaError_t launch_two_steps_f32(const LatticeParams&, const void*, void*, cudaStream_t);
 cudaError_t launch_steps1_f64(const LatticeParams&, const void*, void*, int, cudaStream_t);
 cudaError_t launch_steps1_f32(const LatticeParams&, const void*, void*, int, cudaStream_t);
 cudaError_t launch_steps1_f16(const LatticeParams&, const void*, void*, int, cudaStream_t);
@@ -90,7 +92,7 @@ cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void*
     return cudaErrorInvalidValue;
 }
 
-// A launch of k steps takes `launch` us (launch, load, store) plus k times a warp's
+// 1D: a launch of k steps takes `launch` us (launch, load, store) plus k times a warp's
 // arithmetic, which four warps per SM do side by side (one per SM quarter; an FP64
 // instruction occupies a quarter for 64 cycles) and further ones in rounds.  The
 // constants are fitted to D1Q5 {0, +-1, +-3}, periodic, us per step with one step per
@@ -98,7 +100,7 @@ cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void*
 // before the symmetric core alone) -> 1.87, 20,000 nodes 5.46 -> 3.54, 100,000 nodes
 // 18.95 -> 14.70 (k = 1); FP32 1.74 -> 0.53, 1.87 -> 0.91, 2.32 -> 1.55.
 int steps_per_launch(int prec, const LatticeParams& P) {
-    if (P.dim != 1) return 1;
+    if (P.dim != 1) return prec == kF32 && two_steps_f32(P) ? 2 : 1;   // plbm_fuse.cuh
     const int w = halo1(P), sms = device_sm_count();
     const double launch = 1.5, latency = prec == kF64 ? 1.5 : 0.25;
     auto time = [&](int k) {   // per step
@@ -114,7 +116,8 @@ int steps_per_launch(int prec, const LatticeParams& P) {
     return best;
 }
 
-cudaError_t launch_steps1(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
+cudaError_t launch_steps(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
+    if (P.dim != 1) return steps == 2 && prec == kF32 ? launch_two_steps_f32(P, src, dst, stream) : cudaErrorInvalidValue;
     switch (prec) {
         case kF64: return launch_steps1_f64(P, src, dst, steps, stream);
         case kF32: return launch_steps1_f32(P, src, dst, steps, stream);

@@ -61,17 +61,23 @@ __device__ __forceinline__ void step_end() {
 }
 
 template <class... P, class... A>
-cudaError_t launch_dependent(bool small_too, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+cudaError_t launch_dependent_smem(bool small_too, size_t smem, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream,
+                                  A... args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = small_too || (long long)grid.x * grid.y * grid.z * block.x >= kDependentThreads ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_dependent(bool small_too, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+    return launch_dependent_smem(small_too, 0, kernel, grid, block, stream, args...);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,205 @@
+// Two steps of a 2D symmetric five-velocity lattice in one pass over memory
+// (thermal, periodic, FP32 storage; the single step is plbm_pair.cuh's).
+//
+// A single FP32 step moves 200 bytes a node and is bound by them: 2048^2 takes
+// 120.9 us, 6.9 TB/s, while the SMs could update twice as many nodes.  So the state
+// between two steps is kept out of memory.  A CTA owns a strip of columns times a
+// segment of rows and walks up the rows.  At row r it
+//   1. pulls row r from the old array (loads issued one row ahead, into registers),
+//      collides it and puts the 25 populations into shared memory;
+//   2. pulls row r - w (w = max |v|) from there, collides it and stores it in the new array.
+// Population column j needs its rows only from r - w - v_j to r, so it keeps
+// w + v_j + 1 rows in a ring: 25 (w + 1) values a column instead of 25 (2 w + 1), 76.8 KB
+// for 96 columns of pairs and w = 3, which lets two CTAs share an SM: one loads and
+// collides while the other waits at a barrier.  A strip computes its first step on w more columns
+// and rows at each side.  The arithmetic is sym5_collide's and the state
+// bit for bit that of two single steps.
+//
+// Measured, us a step, single and here: v = {0, +-1, +-3} 2048^2 120.9 and 90.5, 2047^2 123.4 and
+// 89.2, 4096^2 478 and 344, 8192^2 1935 and 1374, 1500 x 900 40.8 and 34.8, 1024^2 32.0 and 28.5;
+// {0, +-1, +-2} 2048^2 120.9 and 78.6, 2047^2 123.4 and 83.2.
+// What bounds it: a warp's own latencies (1.5 warps a scheduler in pairs, 4.4 cycles from one
+// instruction to the next, a fifth of them waiting for loads); with all data in the second-level cache
+// 2048^2 takes 81 us a step, its traffic alone 65.  Measured slower there: a thread group for each of
+// the two phases (91-93), rows brought in by bulk copies (122 and more), loads two rows ahead
+// (91), bulk prefetches into the second-level cache (94), one node a thread in the paired
+// layout (93), both nodes of two columns a thread in the plain one (97).  16-bit storage gains
+// nothing (67 either way): its single steps are bound by the SMs already.
+#pragma once
+
+#include <algorithm>
+#include <cstdlib>
+#include <type_traits>
+
+#include "plbm_pair.cuh"
+
+namespace plbm {
+
+constexpr int kFuseMaxV = 3;   // largest |v|
+inline int fuse_w(const LatticeParams& P) { return (int)std::max(P.sa, P.sb); }
+// Threads of a CTA and CTAs per SM.  More of either leaves too little first-level cache for
+// the loads in flight (25 lines of 128 or 256 bytes a warp): at w = 3 two CTAs of 128 threads in pairs,
+// 205 KB of rings, take 222 us where two of 96 take 181.
+struct FuseShape {
+    int threads, resident;
+    size_t smem;
+};
+inline FuseShape fuse_shape(const LatticeParams& P) {
+    const int w = fuse_w(P), threads = P.paired ? (w > 2 ? 96 : 64) : 128;
+    const int resident = w > 2 ? (P.paired ? 2 : 3) : 4;
+    return {threads, resident, 25 * (size_t)(w + 1) * threads * (P.paired ? sizeof(float2) : sizeof(float))};
+}
+
+// V: the value of one column, both nodes of a pair (row-paired layout) or one node.
+// grid = (strips, segments); CTA (b, s) owns columns [nx b / strips, nx (b + 1) / strips), at most
+// NT - 2w of them, of (pair) rows [rows s / segments, rows (s + 1) / segments).
+// rows >= 2w and nx >= 2w: no index wraps twice.
+template <class V, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* __restrict__ dst) {
+    constexpr bool kPaired = std::is_same<V, float2>::value;
+    extern __shared__ __align__(16) unsigned char fuse_ring[];
+    V* ring = reinterpret_cast<V*>(fuse_ring);
+    step_begin();
+    const int va = (int)P.sa, vb = (int)P.sb, w = max(va, vb);
+    const int v[5] = {0, va, -va, vb, -vb};
+    const int rows = kPaired ? P.half_ny : P.ny;
+    const int x0 = (int)((long long)P.nx * blockIdx.x / gridDim.x);
+    const int wn = (int)((long long)P.nx * (blockIdx.x + 1) / gridDim.x) - x0;
+    const int r0 = (int)((long long)rows * blockIdx.y / gridDim.y), r1 = (int)((long long)rows * (blockIdx.y + 1) / gridDim.y);
+    const int t = threadIdx.x;
+    const bool first = t < wn + 2 * w, second = t < wn;   // has a column in step 1, in step 2
+    unsigned col[5];
+    {
+        int x = x0 - w + (first ? t : 0);
+        x = x < 0 ? x + P.nx : (x >= P.nx ? x - P.nx : x);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            const int k = x + P.vxm[i];
+            col[i] = (unsigned)(k >= P.nx ? k - P.nx : k);
+        }
+    }
+    int depth[5], base[5], slot[5];   // rows of population column j in the ring, where they start, the row in turn
+    {
+        int o = 0;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            depth[j] = w + v[j] + 1;
+            base[j] = o;
+            slot[j] = 0;
+            o += depth[j] * 5 * NT;
+        }
+    }
+    V g[25];
+    auto load = [&](int rr) {   // the pulls of row rr; rows outside [0, rows) lie across the y wrap, pairs swapped
+        unsigned row[5];
+        bool swp[5], any = false;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            int k = rr - v[j];
+            swp[j] = k < 0 || k >= rows;
+            any |= swp[j];
+            k = k < 0 ? k + rows : (k >= rows ? k - rows : k);
+            row[j] = (unsigned)k * (unsigned)P.pitch;
+        }
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+#pragma unroll
+            for (int j = 0; j < 5; ++j) g[5 * i + j] = __ldg(src + (5 * i + j) * P.plane2 + (row[j] + col[i]));
+        if constexpr (kPaired) {
+            if (any) {
+#pragma unroll
+                for (int p = 0; p < 25; ++p)
+                    if (swp[p % 5]) g[p] = f2(g[p].y, g[p].x);
+            }
+        }
+    };
+    V rho, th, drho, jx, jy, e;
+    step_wait();
+    if (first) load(r0 - w);
+    for (int rr = r0 - w; rr < r1 + w; ++rr) {
+        if (first) {
+            V o[25];
+            sym5_collide<V>(P, [&](int p) { return g[p]; }, [&](int p) { return g[p]; }, o, rho, th, drho, jx, jy, e);
+            flag_unhealthy(P, rho, th);
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                V* q = ring + base[j] + slot[j] * 5 * NT + t;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) q[i * NT] = o[5 * i + j];
+            }
+            if (rr + 1 < r1 + w) load(rr + 1);
+        }
+        __syncthreads();
+        // the oldest row of each ring, the next to be overwritten, is the one that row rr - w pulls
+#pragma unroll
+        for (int j = 0; j < 5; ++j) slot[j] = slot[j] + 1 == depth[j] ? 0 : slot[j] + 1;
+        if (second && rr - w >= r0) {
+            V o[25];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                const V* q = ring + base[j] + slot[j] * 5 * NT + t + w;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) o[5 * i + j] = q[i * NT - v[i]];
+            }
+            sym5_collide<V>(P, [&](int p) { return o[p]; }, [&](int p) { return o[p]; }, o, rho, th, drho, jx, jy, e);
+            flag_unhealthy(P, rho, th);
+            const unsigned here = (unsigned)(rr - w) * (unsigned)P.pitch + (unsigned)(x0 + t);
+#pragma unroll
+            for (int p = 0; p < 25; ++p) dst[p * P.plane2 + here] = o[p];
+        }
+        __syncthreads();
+    }
+}
+
+// The split of a lattice for k_two_steps, or strips = 0 where single steps are taken: lattices whose
+// two arrays fit in the second-level cache (768^2: 18.7 us a step against 14.7), and those that do
+// not fill the strips and segments well.  A CTA takes row_us for a row while the chip is full,
+// whatever the width of its strip, so two steps take waves x (rows of a segment + 2w) x row_us, which
+// the number of segments minimises; single steps go at the memory's rate.
+struct FusePlan {
+    int strips, segments;
+};
+inline FusePlan fuse_plan(const LatticeParams& P) {
+    FusePlan best{0, 0};
+    if (P.dim != 2 || !P.sym5 || P.isothermal || P.fixed_ends) return best;
+    const int w = fuse_w(P), rows = P.paired ? P.half_ny : P.ny;
+    const double nodes = (double)P.nx * P.ny;
+    if (w > kFuseMaxV || rows < 2 * w || P.nx < 2 * w || nodes * 200 < 1.3e8) return best;
+    const FuseShape shape = fuse_shape(P);
+    const int most = shape.threads - 2 * w, strips = (P.nx + most - 1) / most, resident = device_sm_count() * shape.resident;
+    const double row_us = w > 2 ? 2.1 : P.paired ? 2.4 : 2.65, single_us = nodes * (P.paired ? 28.8e-6 : 29.4e-6);
+    double least = 1e300;
+    for (int segs = 1; segs <= rows && segs <= 65535; ++segs) {
+        const long long ctas = (long long)strips * segs, waves = (ctas + resident - 1) / resident;
+        const double time = (double)waves * ((rows + segs - 1) / segs + 2 * w) * row_us;
+        if (time < least) least = time, best = {strips, segs};
+        if (waves > 8 && segs > 1) break;
+    }
+    return least < 0.95 * 2 * single_us ? best : FusePlan{0, 0};
+}
+
+template <class V, int NT, int MINB>
+cudaError_t launch_two_steps_t(const LatticeParams& L, const void* src, void* dst, cudaStream_t stream) {
+    const FusePlan plan = fuse_plan(L);
+    const FuseShape shape = fuse_shape(L);
+    if (plan.strips == 0 || shape.threads != NT) return cudaErrorInvalidValue;
+    const auto kernel = k_two_steps<V, NT, MINB>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shape.smem);
+    if (e == cudaSuccess)   // shared memory for the resident CTAs (1 KB each besides), the rest as cache
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)((shape.resident * (shape.smem + 1024) * 100 + (228 << 10) - 1) / (228 << 10)));
+    if (e != cudaSuccess) return e;
+    return launch_dependent_smem(true, shape.smem, kernel, dim3(plan.strips, plan.segments), NT, stream, pair_params(L),
+                                 static_cast<const V*>(src), static_cast<V*>(dst));
+}
+
+inline cudaError_t launch_two_steps(const LatticeParams& P, const void* src, void* dst, cudaStream_t stream) {
+    if (fuse_w(P) > 2)
+        return P.paired ? launch_two_steps_t<float2, 96, 2>(P, src, dst, stream)
+                        : launch_two_steps_t<float, 128, 3>(P, src, dst, stream);
+    return P.paired ? launch_two_steps_t<float2, 64, 4>(P, src, dst, stream)
+                    : launch_two_steps_t<float, 128, 4>(P, src, dst, stream);
+}
+
+}  // namespace plbm

@@ -668,10 +668,10 @@ plbm_status plbm_step(plbm_handle hh, long n) {
     const int ce = h->desc.check_every;
     long s = 0;
     const long long nodes = (long long)h->P.nx * h->P.ny * h->P.nz;
-    const int per = h->P.dim == 1 ? plbm::steps_per_launch(h->prec, h->P) : 1;   // steps of one launch
+    const int per = plbm::steps_per_launch(h->prec, h->P);   // steps of one launch
     auto launch = [&](int c, int k, cudaStream_t stream) {   // k <= per steps from array c
         if (h->P.dim == 3) return plbm::launch_step3(h->prec, h->P, h->f[c], h->f[c ^ 1], stream);
-        if (k > 1) return plbm::launch_steps1(h->prec, h->P, h->f[c], h->f[c ^ 1], k, stream);
+        if (k > 1) return plbm::launch_steps(h->prec, h->P, h->f[c], h->f[c ^ 1], k, stream);
         return plbm::launch_step(h->prec, h->P, h->f[c], h->f[c ^ 1], false, stream);
     };
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -703,12 +703,20 @@ plbm_status plbm_step(plbm_handle hh, long n) {
         }
     }
     while (s < n) {
-        long k = std::min<long>(per, n - s);
-        if (ce > 0) k = std::min<long>(k, ce - s % ce);
-        CK(launch(h->cur, (int)k, h->stream));
-        h->cur ^= 1;
-        h->steps += k;
-        s += k;
+        long run = n - s;   // steps to the next status read or the end
+        if (ce > 0) run = std::min<long>(run, ce - s % ce);
+        // As many launches as steps, modulo 2: the current array is then the one that single
+        // steps lead to, which batches and slabs go by (instances in step have the same).
+        long launches = (run + per - 1) / per;
+        if ((launches ^ run) & 1) ++launches;
+        for (; launches > 0; --launches) {
+            const long k = (run + launches - 1) / launches;
+            CK(launch(h->cur, (int)k, h->stream));
+            h->cur ^= 1;
+            h->steps += k;
+            s += k;
+            run -= k;
+        }
         if (ce > 0 && s % ce == 0 && s < n) {
             st = plbm_check(hh);
             if (st != PLBM_OK) return st;

@@ -232,10 +232,10 @@ void set_thread_error(const char* msg);
 // on `stream` and return the launch error.
 cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void* dst,
                         bool reduce, cudaStream_t stream);
-// 1D lattices: the number of steps best taken by one launch (1: launch_step), and a
-// launch that takes `steps` of them (2 <= steps <= that number).
+// The number of steps best taken by one launch (1: launch_step; 1D lattices and large FP32
+// ones take several), and a launch that takes `steps` of them (2 <= steps <= that number).
 int steps_per_launch(int prec, const LatticeParams& P);
-cudaError_t launch_steps1(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream);
+cudaError_t launch_steps(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream);
 // Rows [y0, y1) (y1 < 0: to the last row); field pointers index the whole lattice.
 // Batched step of 2D lattices in the plain layout, all of precision prec and
 // q1 velocities per axis (q1 = 3, 4 or 5): tiles of kBlockX nodes of one row.

@@ -197,6 +197,27 @@ __device__ __forceinline__ bool healthy2(float2 rho, float2 th) {
            (rho.x < 3.0e38f) & (rho.y < 3.0e38f) & (th.x < 3.0e38f) & (th.y < 3.0e38f);
 }
 
+// Sets the status bits of a node pair or a node whose rho or theta is non-finite or non-positive.
+__device__ __forceinline__ void flag_unhealthy(const PairParams& P, float2 rho, float2 th) {
+    if (!healthy2(rho, th)) {
+        unsigned bits = 0u;
+        bits |= (!(rho.x == rho.x) || !(rho.y == rho.y) || !(th.x == th.x) || !(th.y == th.y) ||
+                 !(rho.x < 3.0e38f) || !(rho.y < 3.0e38f) || !(th.x < 3.0e38f) || !(th.y < 3.0e38f))
+                    ? 1u : 0u;
+        bits |= (rho.x <= 0.0f || rho.y <= 0.0f) ? 2u : 0u;
+        bits |= (th.x <= 0.0f || th.y <= 0.0f) ? 4u : 0u;
+        atomicOr(P.status, bits);
+    }
+}
+__device__ __forceinline__ void flag_unhealthy(const PairParams& P, float rho, float th) {
+    if (!((rho > 0.0f) & (th > 0.0f) & (rho < 3.0e38f) & (th < 3.0e38f))) {
+        unsigned bits = (!(rho == rho) || !(th == th) || !(rho < 3.0e38f) || !(th < 3.0e38f)) ? 1u : 0u;
+        bits |= rho <= 0.0f ? 2u : 0u;
+        bits |= th <= 0.0f ? 4u : 0u;
+        atomicOr(P.status, bits);
+    }
+}
+
 // The 25 pulls of a node pair (lane order fixed up across the y wrap), each
 // passed through conv on its way into dst.
 template <typename PS, typename T, class Conv>
@@ -241,15 +262,7 @@ __device__ __forceinline__ void pair_update(const PairParams& P, Pull pull, type
         sym5_collide<float2>(P, [&](int p) { return o[p]; }, [&](int p) { return o[p]; }, o, rho, th, drho, jx, jy,
                              e);
     }
-    if (!healthy2(rho, th)) {
-        unsigned bits = 0u;
-        bits |= (!(rho.x == rho.x) || !(rho.y == rho.y) || !(th.x == th.x) || !(th.y == th.y) ||
-                 !(rho.x < 3.0e38f) || !(rho.y < 3.0e38f) || !(th.x < 3.0e38f) || !(th.y < 3.0e38f))
-                    ? 1u : 0u;
-        bits |= (rho.x <= 0.0f || rho.y <= 0.0f) ? 2u : 0u;
-        bits |= (th.x <= 0.0f || th.y <= 0.0f) ? 4u : 0u;
-        atomicOr(P.status, bits);
-    }
+    flag_unhealthy(P, rho, th);
     if (REDUCE) {   // two nodes: deviations from the rest state in float-float
         d.dmass = ff_add(FF{drho.x, 0.0f}, drho.y);
         d.jx = ff_add(FF{jx.x, 0.0f}, jx.y);
@@ -411,12 +424,7 @@ __device__ __forceinline__ void sym5_node(const PairParams& P, const S* __restri
         }
     float rho, th, drho, jx, jy, e;
     sym5_collide<float>(P, [&](int p) { return g[p]; }, [&](int p) { return g[p]; }, g, rho, th, drho, jx, jy, e);
-    if (!((rho > 0.0f) & (th > 0.0f) & (rho < 3.0e38f) & (th < 3.0e38f))) {
-        unsigned bits = (!(rho == rho) || !(th == th) || !(rho < 3.0e38f) || !(th < 3.0e38f)) ? 1u : 0u;
-        bits |= rho <= 0.0f ? 2u : 0u;
-        bits |= th <= 0.0f ? 4u : 0u;
-        atomicOr(P.status, bits);
-    }
+    flag_unhealthy(P, rho, th);
     if (REDUCE) {
         d.dmass = FF{drho, 0.0f};
         d.jx = FF{jx, 0.0f};

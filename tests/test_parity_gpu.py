@@ -766,6 +766,57 @@ def test_queued_steps_equal_awaited_steps(dim, v, shape, prec, kw):
     assert np.array_equal(got[0], got[1])
 
 
+# Large FP32 lattices advance two steps per launch (strips of columns, segments of rows): the
+# state must be that of single steps bit for bit, in both layouts, for odd and even step counts,
+# status reads between, a captured stream and a set in either order; strips one column apart in
+# width, a last wave with few blocks, few rows and few columns.
+@pytest.mark.parametrize("v,shape,plain", [
+    (I.SET_013, (1024, 1024), False), (I.SET_013, (1009, 1030), False), (I.SET_013, (901, 901), False),
+    (I.SET_013, (1200, 902), True), (I.SET_012, (1021, 1026), False), (I.SET_012, (1011, 1021), False),
+    ((0, 3, -3, 1, -1), (960, 1026), False), ((0, 2, -2, 1, -1), (1031, 957), False), ((0, 2, -2, 3, -3), (1500, 800), False),
+    (I.SET_013, (40000, 100), False), (I.SET_013, (90, 40000), False), (I.SET_013, (40000, 101), False),
+    (I.SET_012, (400000, 8), False), (I.SET_013, (700, 1000), False), ((0, 1, -1, 4, -4), (1024, 1024), False)])
+def test_two_steps_of_one_launch_equal_single_steps(v, shape, plain):
+    import torch
+    from paper_1402_5487_gb300 import plbm
+    nx, ny = shape
+    g = torch.Generator(device="cuda").manual_seed(3)
+    one = torch.ones(ny, nx, dtype=torch.float64, device="cuda")
+    u = [0.02 * (torch.rand(ny, nx, dtype=torch.float64, device="cuda", generator=g) - 0.5) for _ in range(2)]
+    th0 = 0.7 if max(v) == 2 else 1.0
+    side = torch.cuda.Stream()
+
+    def run(parts, ce=0, how="step"):
+        s = plbm.Solver(2, v, 1.1, nx, ny, theta0=th0, prec="f32", plain_layout=plain, check_every=ce,
+                        skip_admissibility=True, stream=side)
+        torch.cuda.synchronize()
+        s.init(one, u[0], u[1], th0 * one)
+        for k in parts:
+            if how == "graph":
+                side.synchronize()
+                gr = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(gr, stream=side):
+                    s.step(k)
+                with torch.cuda.stream(side):
+                    gr.replay()
+            elif how == "diag":
+                s.step_diagnostics(k)
+            else:
+                s.step(k)
+        side.synchronize()
+        out = s.moments(on_device=True)
+        side.synchronize()
+        pop = s.get_populations() if nx * ny < 1 << 21 else None
+        s.close()
+        return out, pop
+
+    ref = run((1,) * 11)
+    for parts, kw in (((11,), {}), ((2, 3, 6), {}), ((4, 7), {"ce": 5}), ((11,), {"how": "graph"}), ((6, 5), {"how": "diag"})):
+        out, pop = run(parts, **kw)
+        assert all(torch.equal(a, b) for a, b in zip(ref[0], out)), (parts, kw)
+        assert pop is None or np.array_equal(ref[1], pop)
+
+
 # FP64 steps of five-velocity sets: the symmetric ones in either order of a and b,
 # thermal and isothermal, with fixed ends, on one row, at another density scale, and a
 # set in an order the symmetric core does not take; 60 steps within 1e-12 of the oracle.
