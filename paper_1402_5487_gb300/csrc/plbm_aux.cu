@@ -1,11 +1,10 @@
-// Non-hot kernels of libplbm: initial equilibrium, moments of the stored state,
-// deterministic FP64 reductions and population import/export.  All arithmetic
-// here is FP64 regardless of the storage precision.
+// Initial equilibrium, moments of the stored state, deterministic reductions and
+// population import/export.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "plbm.h"
-#include "plbm_device.cuh"
+#include "plbm_pair.cuh"
 
 namespace plbm {
 
@@ -184,7 +183,12 @@ __device__ __forceinline__ void check_init_node(const LatticeParams& P, const do
     const double b = (P.dim == 2 && uy) ? uy[n] : 0.0;
     const bool has_t = !(P.isothermal || theta == nullptr);
     const double t = has_t ? theta[n] : 1.0;
-    if (isfinite(r) && isfinite(a) && isfinite(b) && isfinite(t) && r > 0.0 && t > 0.0) return;
+    // on the integer pipe: a positive finite double has bits in [1, inf), a finite one after its sign
+    const unsigned long long inf = 0x7ff0000000000000ull, mag = 0x7fffffffffffffffull;
+    const unsigned long long rb = __double_as_longlong(r), tb = __double_as_longlong(t);
+    if (rb - 1 < inf - 1 && tb - 1 < inf - 1 && (__double_as_longlong(a) & mag) < inf &&
+        (__double_as_longlong(b) & mag) < inf)
+        return;
     unsigned bits = 0u;
     if (!isfinite(r) || !isfinite(a) || !isfinite(b) || !isfinite(t)) bits |= PLBM_STATUS_NONFINITE;
     if (isfinite(r) && !(r > 0.0)) bits |= PLBM_STATUS_RHO_NONPOS;
@@ -288,6 +292,24 @@ __global__ void k_moments_q(const __grid_constant__ LatticeParams P, const S* __
     if (theta) theta[n] = (en / m0 - (a * a + b * b)) / (double)DIM;
 }
 
+// The same of a symmetric five-velocity set by the sums of its steps (1024^2: 218 -> 126 us).
+template <int DIM>
+__global__ void __launch_bounds__(128) k_moments_sym5_f64(const __grid_constant__ LatticeParams P, const double* __restrict__ f,
+                                                          double* rho, double* ux, double* uy, double* theta, int y0) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = y0 + blockIdx.y;
+    if (x >= P.nx) return;
+    double g[Sym5Core<DIM>::Q], r, t, e, jx, jy, a, b;
+#pragma unroll
+    for (int p = 0; p < Sym5Core<DIM>::Q; ++p) g[p] = __ldg(f + elem_index(P, p, x, y));
+    Sym5Core<DIM>::moments(g, P, r, t, jx, jy, e, a, b);
+    const long long n = (long long)y * P.nx + x;
+    if (rho) rho[n] = r;
+    if (ux) ux[n] = a;
+    if (uy) uy[n] = b;
+    if (theta) theta[n] = t;
+}
+
 // Initial state of a 16/32-bit handle with a symmetric five-velocity set, in the
 // FP32 deviation arithmetic of its own collision: per axis the constraint form
 // of the rule (dmu_n = mu_n(u, theta) - mu_n(0, theta0), n = 1..4;
@@ -315,15 +337,10 @@ __device__ __forceinline__ void sym5_dev(const LatticeParams& P, float u, float 
     dr[4] = Eb - Ob;
 }
 
-template <typename S, int DIM>
-__global__ void k_init_sym5_dev(const __grid_constant__ LatticeParams P, const double* __restrict__ rho,
-                                const double* __restrict__ ux, const double* __restrict__ uy,
-                                const double* __restrict__ theta, S* __restrict__ f, int y0) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = y0 + blockIdx.y;
-    if (x >= P.nx) return;
-    const long long n = (long long)y * P.nx + x;
-    check_init_node(P, rho, ux, uy, theta, n);
+// The state of one node: put(p, value) for each population.
+template <int DIM, class Put>
+__device__ __forceinline__ void init_sym5_node(const LatticeParams& P, const double* rho, const double* ux, const double* uy,
+                                               const double* theta, long long n, Put put) {
     const float dth = (P.isothermal || theta == nullptr) ? 0.0f : (float)(theta[n] - P.theta0);
     const float drho = (float)(rho[n] - 1.0);
     const float rh = 1.0f + drho;
@@ -334,12 +351,71 @@ __global__ void k_init_sym5_dev(const __grid_constant__ LatticeParams P, const d
     for (int i = 0; i < 5; ++i) {
         const float X = fmaf(drho, P.w1f[i], rh * drx[i]);
         if (DIM == 1) {
-            Storage<S>::store(f + elem_index(P, i, x, y), X);
+            put(i, X);
         } else {
 #pragma unroll
-            for (int j = 0; j < 5; ++j)
-                Storage<S>::store(f + elem_index(P, i * 5 + j, x, y),
-                                  fmaf(X, P.w1f[j] + dry[j], P.w1f[i] * dry[j]));
+            for (int j = 0; j < 5; ++j) put(i * 5 + j, fmaf(X, P.w1f[j] + dry[j], P.w1f[i] * dry[j]));
+        }
+    }
+}
+
+template <typename S, int DIM>
+__global__ void k_init_sym5_dev(const __grid_constant__ LatticeParams P, const double* __restrict__ rho,
+                                const double* __restrict__ ux, const double* __restrict__ uy,
+                                const double* __restrict__ theta, S* __restrict__ f, int y0) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = y0 + blockIdx.y;
+    if (x >= P.nx) return;
+    const long long n = (long long)y * P.nx + x;
+    check_init_node(P, rho, ux, uy, theta, n);
+    init_sym5_node<DIM>(P, rho, ux, uy, theta, n,
+                        [&](int p, float v) { Storage<S>::store(f + elem_index(P, p, x, y), v); });
+}
+
+// The same for the row-paired layout, whole lattice: a thread takes both nodes of a pair and stores
+// them together (one node per thread writes half of each 32-byte sector, and its other half
+// from a block far away: 2048^2 FP32 260 -> 80 us, FP16 141 -> 64 us).
+template <typename S>
+__global__ void __launch_bounds__(128) k_init_pair(const __grid_constant__ LatticeParams P, const double* __restrict__ rho,
+                                                   const double* __restrict__ ux, const double* __restrict__ uy,
+                                                   const double* __restrict__ theta, typename PairStore<S>::V* __restrict__ f) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+    if (x >= P.nx) return;
+    const long long n0 = (long long)r * P.nx + x, n1 = n0 + (long long)P.half_ny * P.nx;
+    check_init_node(P, rho, ux, uy, theta, n0);
+    check_init_node(P, rho, ux, uy, theta, n1);
+    float lo[25];
+    init_sym5_node<2>(P, rho, ux, uy, theta, n0, [&](int p, float v) { lo[p] = v; });
+    const long long here = (long long)r * P.pitch + x;
+    init_sym5_node<2>(P, rho, ux, uy, theta, n1,
+                      [&](int p, float v) { PairStore<S>::store(f + p * (P.plane / 2) + here, f2(lo[p], v)); });
+}
+
+// FP64 storage: the initial state by the constraint form of the rule that the steps use (16 FP64
+// instructions an axis instead of 31 with general coefficients; 1024^2 192 -> 140 us).
+template <int DIM>
+__global__ void __launch_bounds__(128) k_init_sym5_f64(const __grid_constant__ LatticeParams P, const double* __restrict__ rho,
+                                                       const double* __restrict__ ux, const double* __restrict__ uy,
+                                                       const double* __restrict__ theta, double* __restrict__ f, int y0) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = y0 + blockIdx.y;
+    if (x >= P.nx) return;
+    const long long n = (long long)y * P.nx + x;
+    check_init_node(P, rho, ux, uy, theta, n);
+    const double th = (P.isothermal || theta == nullptr) ? P.theta0 : theta[n];
+    const double u = ux[n], v = DIM == 2 && uy ? uy[n] : 0.0, rh = rho[n];
+    const double sixth2 = __dmul_rn(__dmul_rn(6.0, th), th);
+    double rx[5], ry[5];
+    Sym5Core<DIM>::axis(P, u, __dmul_rn(u, u), th, sixth2, rx);
+    if constexpr (DIM == 2) Sym5Core<DIM>::axis(P, v, __dmul_rn(v, v), th, sixth2, ry);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const double X = rh * rx[i];
+        if constexpr (DIM == 2) {
+#pragma unroll
+            for (int j = 0; j < 5; ++j) f[elem_index(P, 5 * i + j, x, y)] = X * ry[j];
+        } else {
+            f[elem_index(P, i, x, y)] = X;
         }
     }
 }
@@ -351,12 +427,24 @@ __global__ void k_init_sym5_dev(const __grid_constant__ LatticeParams P, const d
 // the 1D rule) and theta = (E / rho - |u|^2) / d in FP64.
 // (FF, ff_add, ff_scale, ff_f64: plbm_device.cuh)
 
-template <typename S, int Q1, int DIM>
-__global__ void k_moments_dev(const __grid_constant__ LatticeParams P, const S* __restrict__ f, double* rho,
-                              double* ux, double* uy, double* theta, int y0) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = y0 + blockIdx.y;
-    if (x >= P.nx) return;
+// The fields of a node in FP64 from its float-float sums.
+struct NodeFields {
+    double rho, ux, uy, theta;
+};
+template <int DIM>
+__device__ __forceinline__ NodeFields fields_from_sums(const LatticeParams& P, FF dm, FF jx, FF jy, FF de) {
+    NodeFields o;
+    o.rho = 1.0 + ff_f64(dm);
+    const double ir = recip_f64(o.rho);
+    o.ux = ff_f64(jx) * ir;
+    o.uy = DIM == 2 ? ff_f64(jy) * ir : 0.0;
+    o.theta = (((double)DIM * P.theta0 + ff_f64(de)) * ir - (o.ux * o.ux + o.uy * o.uy)) * (1.0 / DIM);
+    return o;
+}
+
+// get(p): the stored deviation of population p.
+template <int Q1, int DIM, class Get>
+__device__ __forceinline__ NodeFields fields_dev(const LatticeParams& P, Get get) {
     FF Sx[Q1], Ty[Q1];
 #pragma unroll
     for (int i = 0; i < Q1; ++i) Sx[i] = Ty[i] = FF{0.0f, 0.0f};
@@ -364,8 +452,7 @@ __global__ void k_moments_dev(const __grid_constant__ LatticeParams P, const S* 
     for (int i = 0; i < Q1; ++i)
 #pragma unroll
         for (int j = 0; j < (DIM == 2 ? Q1 : 1); ++j) {
-            const int p = DIM == 2 ? i * Q1 + j : i;
-            const float g = Storage<S>::load(f + elem_index(P, p, x, y));
+            const float g = get(DIM == 2 ? i * Q1 + j : i);
             Sx[i] = ff_add(Sx[i], g);
             if (DIM == 2) Ty[j] = ff_add(Ty[j], g);
         }
@@ -381,14 +468,75 @@ __global__ void k_moments_dev(const __grid_constant__ LatticeParams P, const S* 
             de = ff_add(de, ff_scale(ff_scale(Ty[i], vi), vi));
         }
     }
-    const double r = 1.0 + ff_f64(dm);
-    const double ir = 1.0 / r;
-    const double a = ff_f64(jx) * ir, b = DIM == 2 ? ff_f64(jy) * ir : 0.0;
-    const long long n = (long long)y * P.nx + x;
-    if (rho) rho[n] = r;
-    if (ux) ux[n] = a;
-    if (uy) uy[n] = b;
-    if (theta) theta[n] = (((double)DIM * P.theta0 + ff_f64(de)) * ir - (a * a + b * b)) / (double)DIM;
+    return fields_from_sums<DIM>(P, dm, jx, jy, de);
+}
+
+__device__ __forceinline__ void put_fields(const NodeFields& o, long long n, double* rho, double* ux, double* uy, double* theta) {
+    if (rho) rho[n] = o.rho;
+    if (ux) ux[n] = o.ux;
+    if (uy) uy[n] = o.uy;
+    if (theta) theta[n] = o.theta;
+}
+
+template <typename S, int Q1, int DIM>
+__global__ void k_moments_dev(const __grid_constant__ LatticeParams P, const S* __restrict__ f, double* rho,
+                              double* ux, double* uy, double* theta, int y0) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = y0 + blockIdx.y;
+    if (x >= P.nx) return;
+    const NodeFields o =
+        fields_dev<Q1, DIM>(P, [&](int p) -> float { return Storage<S>::load(f + elem_index(P, p, x, y)); });
+    put_fields(o, (long long)y * P.nx + x, rho, ux, uy, theta);
+}
+
+__device__ __forceinline__ FF lane_of(FFV<float> v, int) { return {v.hi, v.lo}; }
+__device__ __forceinline__ FF lane_of(FFV<float2> v, int l) { return l ? FF{v.hi.y, v.lo.y} : FF{v.hi.x, v.lo.x}; }
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_times(FFV<V> a, float c) {
+    const V p = mul2(a.hi, splat<V>(c));
+    return {p, fma2(a.lo, splat<V>(c), fma2(a.hi, splat<V>(c), neg2(p)))};
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_minus(FFV<V> a, FFV<V> b) { return ffv_acc(a, FFV<V>{neg2(b.hi), neg2(b.lo)}); }
+
+// The same for symmetric five-velocity sets, with j and E from the sums and differences of opposite
+// velocities.  V = float2: row-paired layout, whole lattice; a thread loads both nodes of a pair,
+// so that the state is read once (one node per thread reads it twice, once for each half of
+// the rows), and sums in packed arithmetic.  V = float: one node, any rows.
+// 2048^2 FP32 205 -> 128 us, FP16 200 -> 125 us, 2047^2 FP32 202 -> 124 us: 15 FP64
+// instructions a node (31 with the division and conversions) take 104, the bytes 82 and 51.
+template <typename S, class V>
+__global__ void __launch_bounds__(128) k_moments_sym5(const __grid_constant__ LatticeParams P, const S* __restrict__ f,
+                                                      double* rho, double* ux, double* uy, double* theta, int y0) {
+    constexpr int kLanes = sizeof(V) / sizeof(float);
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = y0 + blockIdx.y;
+    if (x >= P.nx) return;
+    const FFV<V> zero{splat<V>(0.0f), splat<V>(0.0f)};
+    const S* at = f + elem_index(P, 0, x, y);   // V = float2: y < half_ny, the pair's first node
+    FFV<V> Sx[5], Ty[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const S* q = at + (5 * i + j) * P.plane;
+            V g;
+            if constexpr (kLanes == 2)
+                g = PairStore<S>::cvt(PairStore<S>::raw(reinterpret_cast<const typename PairStore<S>::V*>(q)));
+            else
+                g = Storage<S>::load(q);
+            Sx[i] = j ? ffv_acc(Sx[i], g) : FFV<V>{g, zero.lo};
+            Ty[j] = i ? ffv_acc(Ty[j], g) : FFV<V>{g, zero.lo};
+        }
+    const FFV<V> Sp = ffv_acc(Sx[1], Sx[2]), Sq = ffv_acc(Sx[3], Sx[4]);
+    const FFV<V> Tp = ffv_acc(Ty[1], Ty[2]), Tq = ffv_acc(Ty[3], Ty[4]);
+    const FFV<V> dm = ffv_acc(ffv_acc(Sx[0], Sp), Sq);
+    const FFV<V> jx = ffv_acc(ffv_times(ffv_minus(Sx[1], Sx[2]), P.sa), ffv_times(ffv_minus(Sx[3], Sx[4]), P.sb));
+    const FFV<V> jy = ffv_acc(ffv_times(ffv_minus(Ty[1], Ty[2]), P.sa), ffv_times(ffv_minus(Ty[3], Ty[4]), P.sb));
+    const FFV<V> de = ffv_acc(ffv_times(ffv_acc(Sp, Tp), P.sa2), ffv_times(ffv_acc(Sq, Tq), P.sb2));
+#pragma unroll
+    for (int l = 0; l < kLanes; ++l)
+        put_fields(fields_from_sums<2>(P, lane_of(dm, l), lane_of(jx, l), lane_of(jy, l), lane_of(de, l)),
+                   ((long long)y + l * P.half_ny) * P.nx + x, rho, ux, uy, theta);
 }
 
 template <typename S>
@@ -638,6 +786,20 @@ cudaError_t launch_init(int prec, const LatticeParams& P, const double* rho, con
     if (y1 < 0) y1 = P.ny;
     if (y1 <= y0) return cudaSuccess;
     dim3 grid((P.nx + 127) / 128, y1 - y0);
+    if (P.paired && y0 == 0 && y1 == P.ny) {
+        grid.y = P.half_ny;
+        PLBM_DISPATCH_DEV(prec, (k_init_pair<S><<<grid, 128, 0, stream>>>(P, rho, ux, uy, theta,
+                                                                          static_cast<PairStore<S>::V*>(f))));
+        return cudaGetLastError();
+    }
+    if (prec == kF64 && P.sym5) {
+        double* d = static_cast<double*>(f);
+        if (P.dim == 2)
+            k_init_sym5_f64<2><<<grid, 128, 0, stream>>>(P, rho, ux, uy, theta, d, y0);
+        else
+            k_init_sym5_f64<1><<<grid, 128, 0, stream>>>(P, rho, ux, uy, theta, d, y0);
+        return cudaGetLastError();
+    }
 #define PLBM_INIT_DEV(DIMv)                                                                            \
     if (P.dim == DIMv) {                                                                               \
         PLBM_DISPATCH_DEV(prec, (k_init_sym5_dev<S, DIMv><<<grid, 128, 0, stream>>>(P, rho, ux, uy, theta, \
@@ -670,6 +832,25 @@ cudaError_t launch_moments(int prec, const LatticeParams& P, const void* f, doub
     if (y1 < 0) y1 = P.ny;
     if (y1 <= y0) return cudaSuccess;
     dim3 grid((P.nx + 127) / 128, y1 - y0);
+    if (prec != kF64 && P.sym5 && P.dim == 2) {
+        if (P.paired && y0 == 0 && y1 == P.ny) {
+            grid.y = P.half_ny;
+            PLBM_DISPATCH_DEV(prec, (k_moments_sym5<S, float2><<<grid, 128, 0, stream>>>(
+                                        P, static_cast<const S*>(f), rho, ux, uy, theta, 0)));
+        } else {
+            PLBM_DISPATCH_DEV(prec, (k_moments_sym5<S, float><<<grid, 128, 0, stream>>>(
+                                        P, static_cast<const S*>(f), rho, ux, uy, theta, y0)));
+        }
+        return cudaGetLastError();
+    }
+    if (prec == kF64 && P.sym5) {
+        const double* d = static_cast<const double*>(f);
+        if (P.dim == 2)
+            k_moments_sym5_f64<2><<<grid, 128, 0, stream>>>(P, d, rho, ux, uy, theta, y0);
+        else
+            k_moments_sym5_f64<1><<<grid, 128, 0, stream>>>(P, d, rho, ux, uy, theta, y0);
+        return cudaGetLastError();
+    }
 #define PLBM_MOM_Q(Q1v, DIMv)                                                                           \
     if (P.q1 == Q1v && P.dim == DIMv) {                                                                 \
         if (prec == kF64)                                                                               \

@@ -194,7 +194,20 @@ __device__ __forceinline__ FF ff_scale(FF a, float v) {
     const float e = fmaf(a.hi, v, -p);
     return {p, fmaf(a.lo, v, e)};
 }
-__device__ __forceinline__ double ff_f64(FF a) { return (double)a.hi + (double)a.lo; }
+// (double)v on the integer pipe: a conversion instruction takes the FP64 pipe (two lanes per SM and
+// cycle), predicated off or not, so that subnormal (scaled by 2^24 first), infinite and NaN values
+// are selected rather than branched to.
+__device__ __forceinline__ double f64_of(float v) {
+    unsigned m = __float_as_uint(v) & 0x7fffffffu;
+    const unsigned sign = __float_as_uint(v) & 0x80000000u;
+    unsigned off = m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+    if (m < 0x00800000u) {
+        m = __float_as_uint(__fmul_rn(__uint_as_float(m), 0x1p24f));
+        off = m ? 0x38000000u - (24u << 20) : 0u;
+    }
+    return __hiloint2double((int)(sign | ((m >> 3) + off)), (int)(m << 29));
+}
+__device__ __forceinline__ double ff_f64(FF a) { return f64_of(a.hi) + f64_of(a.lo); }
 __device__ __forceinline__ FF ff_shfl_down(FF a, int off) {
     return {__shfl_down_sync(0xffffffffu, a.hi, off), __shfl_down_sync(0xffffffffu, a.lo, off)};
 }
@@ -491,13 +504,14 @@ __device__ __forceinline__ double recip_f64(double x) {
 // ---------------------------------------------------------------------------
 // FP64 core of the symmetric five-velocity sets (0, +-a, +-b).  The FP64 pipe (two
 // lanes per SM and cycle) bounds these steps, so what counts is the number of FP64
-// instructions: 150 per 2D node against 202 with DirectCore (general velocities and
+// instructions: 152 per 2D node against 202 with DirectCore (general velocities and
 // coefficients, FP64 status comparisons).  The rule in constraint form
 // (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b), r_(+-a) = E_a +- O_a,
-// r_(+-b) = E_b +- O_b) takes 16 instructions per axis instead of 31; the column
-// differences T_1 - T_2 come from the row pairs f_i1 + f_i2 that the row sums
-// need anyway; the velocities and factors are FP64 constants of the lattice.
-// Per step: 1024^2 D2Q25 414 -> 297 us (270 us of FP64 issue), 128^2 10.2 -> 7.9 us,
+// r_(+-b) = E_b +- O_b) takes 16 instructions per axis instead of 31; the sums
+// share S_1 + S_2 and the like; the velocities and factors are FP64 constants of the
+// lattice.  (Differences T_1 - T_2 formed as (T_1 + T_2) - 2 T_2 save two more
+// instructions, 1.2 % of the time, and put u_y 25 % further from the exact value.)
+// Per step: 1024^2 D2Q25 414 -> 301 us (274 us of FP64 issue), 128^2 10.2 -> 7.95 us,
 // the 1000-node D1Q5 tube 4.05 -> 3.2 us.  The identities sum r = 1, sum v^2 r = mu_2
 // hold by construction, so the global sums drift less: mean density of 1024^2 after
 // 40 steps 2e-16 off against 7e-15 (rounded C mu sums), energy 4e-16 against 5e-15.
@@ -526,43 +540,47 @@ struct Sym5Core {
         r[4] = fma(-P.dkOb, yb, Eb);
     }
 
-    static __device__ __forceinline__ void collide(double (&f)[Q], const LatticeParams& P, double& rho_o, double& th_o,
-                                                   double& jx_o, double& jy_o, double& e_o) {
-        double S[5], Tp = 0.0, Tq = 0.0, T2 = 0.0, T4 = 0.0;
+    static __device__ __forceinline__ void moments(const double (&f)[Q], const LatticeParams& P, double& rho, double& th,
+                                                   double& jx, double& jy, double& e, double& ux, double& uy) {
+        double S[5], T[5], Tp = 0.0, Tq = 0.0;
         if constexpr (DIM == 2) {
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
                 const double p = f[5 * i + 1] + f[5 * i + 2], q = f[5 * i + 3] + f[5 * i + 4];
                 S[i] = (f[5 * i] + p) + q;
-                Tp = i ? Tp + p : p;
-                Tq = i ? Tq + q : q;
-                T2 = i ? T2 + f[5 * i + 2] : f[5 * i + 2];
-                T4 = i ? T4 + f[5 * i + 4] : f[5 * i + 4];
             }
+#pragma unroll
+            for (int j = 1; j < 5; ++j) T[j] = (f[j] + (f[5 + j] + f[10 + j])) + (f[15 + j] + f[20 + j]);
+            Tp = T[1] + T[2];
+            Tq = T[3] + T[4];
         } else {
 #pragma unroll
             for (int i = 0; i < 5; ++i) S[i] = f[i];
         }
         const double Sp = S[1] + S[2], Sq = S[3] + S[4];
-        const double rho = S[0] + Sp + Sq;
-        const double jx = fma(P.da, S[1] - S[2], __dmul_rn(P.db, S[3] - S[4]));
-        double jy = 0.0, e;
+        rho = S[0] + Sp + Sq;
+        jx = fma(P.da, S[1] - S[2], __dmul_rn(P.db, S[3] - S[4]));
+        jy = 0.0;
         if constexpr (DIM == 2) {
-            jy = fma(P.da, fma(-2.0, T2, Tp), __dmul_rn(P.db, fma(-2.0, T4, Tq)));
+            jy = fma(P.da, T[1] - T[2], __dmul_rn(P.db, T[3] - T[4]));
             e = fma(P.da2, Sp + Tp, __dmul_rn(P.db2, Sq + Tq));
         } else {
             e = fma(P.da2, Sp, __dmul_rn(P.db2, Sq));
         }
         const double inv = recip_f64(rho);
-        const double ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
+        ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
         const double ux2 = __dmul_rn(ux, ux), uy2 = __dmul_rn(uy, uy);
-        double th = fma(e, inv, -(DIM == 2 ? ux2 + uy2 : ux2));
+        th = fma(e, inv, -(DIM == 2 ? ux2 + uy2 : ux2));
         if constexpr (DIM == 2) th = __dmul_rn(th, 0.5);
+    }
+
+    static __device__ __forceinline__ void collide(double (&f)[Q], const LatticeParams& P, double& rho_o, double& th_o,
+                                                   double& jx_o, double& jy_o, double& e_o) {
+        double rho, th, ux, uy;
+        moments(f, P, rho, th, jx_o, jy_o, e_o, ux, uy);
+        const double ux2 = __dmul_rn(ux, ux), uy2 = __dmul_rn(uy, uy);
         rho_o = rho;
         th_o = th;
-        jx_o = jx;
-        jy_o = jy;
-        e_o = e;
         if (P.isothermal) th = P.theta0;
         const double sixth2 = __dmul_rn(__dmul_rn(6.0, th), th);
         const double om = P.omega;

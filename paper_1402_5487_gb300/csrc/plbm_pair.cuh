@@ -56,6 +56,28 @@ __device__ __forceinline__ float neg2(float a) { return -a; }
 __device__ __forceinline__ float2 rcp2(float2 a) { return f2(__frcp_rn(a.x), __frcp_rn(a.y)); }
 __device__ __forceinline__ float rcp2(float a) { return __frcp_rn(a); }
 
+// Float-float numbers of one node or of a pair of nodes (as FF, plbm_device.cuh, in packed form).
+template <class V>
+struct FFV {
+    V hi, lo;
+};
+__device__ __forceinline__ float ffsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float2 ffsub(float2 a, float2 b) { return fma2(b, f2s(-1.0f), a); }   // exact product
+template <class V>
+__device__ __forceinline__ V two_sum_err(V a, V b, V s) {   // a + b - s for s = fl(a + b)
+    const V t = ffsub(s, a);
+    return add2(ffsub(a, ffsub(s, t)), ffsub(b, t));
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_acc(FFV<V> a, V b) {   // accumulate one value (not normalised)
+    const V s = add2(a.hi, b);
+    return {s, add2(a.lo, two_sum_err(a.hi, b, s))};
+}
+template <class V>
+__device__ __forceinline__ FFV<V> ffv_acc(FFV<V> a, FFV<V> b) {
+    const V s = add2(a.hi, b.hi);
+    return {s, add2(add2(a.lo, b.lo), two_sum_err(a.hi, b.hi, s))};
+}
 // Storage of one node pair.
 template <typename S>
 struct PairStore;

@@ -630,36 +630,15 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
 // (initial state) and 5,152 us (fields) for 128^3 FP32 nodes and 9,989 / 20,554 us
 // for 256 x 256 x 128 FP16 nodes.  Float-float pairs hi + lo (error-free sums and
 // products, ~2^-47 relative) on the deviations from the rest state, whose magnitude
-// is a hundredth of f's (so the absolute error stays at FP64's on f), take 404 / 241 us
-// and 1,234 / 812 us, bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
+// is a hundredth of f's (so the absolute error stays at FP64's on f), take 404 / 236 us
+// and 1,234 / 754 us, bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
 // the z-paired layout a thread takes both nodes of a pair (V = float2: packed FP32x2
 // arithmetic, one aligned 4-byte access for the two); otherwise one node (V = float).
 // ---------------------------------------------------------------------------
 template <class V>
-struct FFV {
-    V hi, lo;
-};
-__device__ __forceinline__ float ffsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float2 ffsub(float2 a, float2 b) { return fma2(b, f2s(-1.0f), a); }   // exact product
-template <class V>
-__device__ __forceinline__ V two_sum_err(V a, V b, V s) {   // a + b - s for s = fl(a + b)
-    const V t = ffsub(s, a);
-    return add2(ffsub(a, ffsub(s, t)), ffsub(b, t));
-}
-template <class V>
 __device__ __forceinline__ FFV<V> ff_norm(V s, V e) {       // |e| below an ulp or so of s
     const V h = add2(s, e);
     return {h, ffsub(e, ffsub(h, s))};
-}
-template <class V>
-__device__ __forceinline__ FFV<V> ffv_acc(FFV<V> a, V b) {   // accumulate one value (not normalised)
-    const V s = add2(a.hi, b);
-    return {s, add2(a.lo, two_sum_err(a.hi, b, s))};
-}
-template <class V>
-__device__ __forceinline__ FFV<V> ffv_acc(FFV<V> a, FFV<V> b) {
-    const V s = add2(a.hi, b.hi);
-    return {s, add2(add2(a.lo, b.lo), two_sum_err(a.hi, b.hi, s))};
 }
 template <class V>
 __device__ __forceinline__ FFV<V> ffv_add(FFV<V> a, FFV<V> b) {
@@ -902,7 +881,7 @@ __global__ void __launch_bounds__(kB3) k_init3_dev(const __grid_constant__ Latti
 }
 
 // FP64 value of a float-float sum; hi alone when it overflowed (lo is NaN then).
-__device__ __forceinline__ double ffv_f64(float hi, float lo) { return (double)hi + (lo == lo ? (double)lo : 0.0); }
+__device__ __forceinline__ double ffv_f64(float hi, float lo) { return f64_of(hi) + f64_of(lo == lo ? lo : 0.0f); }
 __device__ __forceinline__ double lane_f64(FFV<float> v, int) { return ffv_f64(v.hi, v.lo); }
 __device__ __forceinline__ double lane_f64(FFV<float2> v, int l) {
     return l ? ffv_f64(v.hi.y, v.lo.y) : ffv_f64(v.hi.x, v.lo.x);
@@ -958,7 +937,7 @@ __global__ void __launch_bounds__(kB3) k_moments3_dev(const __grid_constant__ La
 #pragma unroll
     for (int l = 0; l < kLanes; ++l) {
         const double m = 1.0 + lane_f64(dm, l);
-        const double im = 1.0 / m;
+        const double im = recip_f64(m);
         const double a = lane_f64(jx, l) * im, b = lane_f64(jy, l) * im, c = lane_f64(jz, l) * im;
         const long long n = ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x;
         if (rho) rho[n] = m;
