@@ -774,7 +774,8 @@ plbm_status plbm_diagnostics(plbm_handle hh, plbm_diag* out) {
     else
         CK(plbm::launch_reduce_state(h->prec, h->P, h->f[h->cur], h->result, h->stream));
     CK(cudaMemcpyAsync(h->host_buf, h->result, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(h->host_buf + 8, h->status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+    if (h->P.dim == 3)
+        CK(cudaMemcpyAsync(h->host_buf + 8, h->status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     out->mass = h->host_buf[0];
     out->jx = h->host_buf[1];
@@ -782,7 +783,7 @@ plbm_status plbm_diagnostics(plbm_handle hh, plbm_diag* out) {
     out->energy = h->host_buf[3];
     out->rho_min = h->host_buf[4];
     out->theta_min = h->host_buf[5];
-    std::memcpy(&out->status, h->host_buf + 8, sizeof(unsigned));
+    std::memcpy(&out->status, h->host_buf + (h->P.dim == 3 ? 8 : 6), sizeof(unsigned));   // 2D: written by launch_finalize
     out->steps = h->steps;
     return PLBM_OK;
 }
@@ -805,7 +806,6 @@ plbm_status plbm_step_diagnostics(plbm_handle hh, long n, plbm_diag* out) {
     ++h->steps;
     CK(plbm::launch_finalize(h->P, plbm::step_blocks(h->P), h->result, h->stream));
     CK(cudaMemcpyAsync(h->host_buf, h->result, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(h->host_buf + 8, h->status, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     out->mass = h->host_buf[0];
     out->jx = h->host_buf[1];
@@ -813,7 +813,7 @@ plbm_status plbm_step_diagnostics(plbm_handle hh, long n, plbm_diag* out) {
     out->energy = h->host_buf[3];
     out->rho_min = h->host_buf[4];
     out->theta_min = h->host_buf[5];
-    std::memcpy(&out->status, h->host_buf + 8, sizeof(unsigned));
+    std::memcpy(&out->status, h->host_buf + 6, sizeof(unsigned));   // written by launch_finalize
     out->steps = h->steps;
     return PLBM_OK;
 }

@@ -268,7 +268,7 @@ cudaError_t launch_moments_pack_batch(int prec, const LatticeParams& P, const La
 // writing out[0..5] = mass, jx, jy, energy, rho_min, theta_min.
 cudaError_t launch_reduce_state(int prec, const LatticeParams& P, const void* f, double* out,
                                 cudaStream_t stream);
-// Final pass over the partials written by a reducing step kernel.
+// Final pass over the partials written by a reducing kernel; out[6] receives the status word.
 cudaError_t launch_finalize(const LatticeParams& P, int nblocks, double* out, cudaStream_t stream);
 cudaError_t launch_get_populations(int prec, const LatticeParams& P, const void* f, double* out,
                                    cudaStream_t stream);

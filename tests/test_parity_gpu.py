@@ -766,6 +766,42 @@ def test_queued_steps_equal_awaited_steps(dim, v, shape, prec, kw):
     assert np.array_equal(got[0], got[1])
 
 
+# The final pass of the reductions (a cluster of blocks over one record per block of a step):
+# fewer records than blocks, one per thread, one more, several per thread.  The sums of the
+# populations themselves within 1e-13 of the sum of magnitudes, minima those of the fields.
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16dev"])
+@pytest.mark.parametrize("shape", [(5, 2), (100, 14), (128, 510), (129, 512), (128, 2049), (130, 4098), (1500, 900)])
+def test_final_pass_of_the_reductions(prec, shape):
+    from paper_1402_5487_gb300 import plbm
+    nx, ny = shape
+    rng = np.random.default_rng(7)
+    s = plbm.Solver(2, I.SET_013, 1.1, nx, ny, prec=prec)
+    one = np.ones((ny, nx))
+    s.init(one + 0.01 * rng.uniform(-1, 1, (ny, nx)), *(0.02 * rng.uniform(-1, 1, (2, ny, nx))), one)
+    s.step(2)
+    # 16/32-bit steps take their sums in FP32 arithmetic before the state is rounded to storage
+    for d in ([s.step_diagnostics(3)] if prec == "f64" else []) + [s.diagnostics()]:
+        f = s.get_populations().reshape(5, 5, -1)
+        v = np.array(I.SET_013, float)
+        e2 = v[:, None] ** 2 + v[None, :] ** 2
+        for key, w in (("mass", np.ones((5, 5))), ("jx", v[:, None] + 0 * v), ("jy", v[None, :] + 0 * v[:, None]), ("energy", e2)):
+            w = np.broadcast_to(w, (5, 5))
+            exact = math.fsum((w[:, :, None] * f).ravel())
+            assert abs(d[key] - exact) <= 1e-13 * np.sum(np.abs(w[:, :, None] * f)), (key, d[key], exact)
+        rho, _, _, th = s.moments()
+        assert abs(d["rho_min"] - rho.min()) <= 1e-13 and abs(d["theta_min"] - th.min()) <= 1e-12
+        assert d["status"] == 0
+    s.close()
+    bad = plbm.Solver(2, I.SET_013, 1.1, nx, ny, prec=prec)
+    bad.init(one, 0 * one, 0 * one, one)
+    g = bad.get_populations()
+    g[0, ny - 1, nx - 1] = np.nan
+    bad.set_populations(g)
+    d = bad.diagnostics()
+    assert d["status"] & 1 and np.isnan(d["mass"]) and abs(d["rho_min"] - 1.0) <= 0.02
+    bad.close()
+
+
 # Large FP32 lattices advance two steps per launch (strips of columns, segments of rows): the
 # state must be that of single steps bit for bit, in both layouts, for odd and even step counts,
 # status reads between, a captured stream and a set in either order; strips one column apart in
