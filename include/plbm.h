@@ -280,10 +280,13 @@ plbm_status plbm_device_populations(plbm_handle h, void **ptr);
  *   PLBM_BATCH_PERSISTENT           one persistent launch per step and group of
  *                                   instances (CTAs walk a global tile list;
  *                                   per-instance parameters in a device table);
- *   PLBM_BATCH_PERSISTENT_GRAPH     the same, two steps per CUDA graph replay;
+ *   PLBM_BATCH_PERSISTENT_GRAPH     the same, two or four steps per CUDA graph
+ *                                   replay;
  *   PLBM_BATCH_PER_INSTANCE         one launch per instance per step;
  *   PLBM_BATCH_PER_INSTANCE_GRAPH   the same, captured in a CUDA graph.
- * All four give bit-identical populations.
+ * All four give bit-identical populations.  In the persistent schemes a group of
+ * thermal FP32 lattices of sets (0, a, -a, b, -b) beyond the second-level cache takes two
+ * steps per launch in every run of four.
  * ------------------------------------------------------------------------ */
 typedef struct plbm_batch_s *plbm_batch;
 

@@ -35,7 +35,6 @@
 
 namespace plbm {
 
-constexpr int kFuseMaxV = 3;   // largest |v|
 inline int fuse_w(const LatticeParams& P) { return (int)std::max(P.sa, P.sb); }
 // Threads of a CTA and CTAs per SM.  More of either leaves too little first-level cache for
 // the loads in flight (25 lines of 128 or 256 bytes a warp): at w = 3 two CTAs of 128 threads in pairs,
@@ -50,35 +49,34 @@ inline FuseShape fuse_shape(const LatticeParams& P) {
     return {threads, resident, 25 * (size_t)(w + 1) * threads * (P.paired ? sizeof(float2) : sizeof(float))};
 }
 
-// V: the value of one column, both nodes of a pair (row-paired layout) or one node.
-// grid = (strips, segments); CTA (b, s) owns columns [nx b / strips, nx (b + 1) / strips), at most
-// NT - 2w of them, of (pair) rows [rows s / segments, rows (s + 1) / segments).
-// rows >= 2w and nx >= 2w: no index wraps twice.
-template <class V, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB)
-k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* __restrict__ dst) {
-    constexpr bool kPaired = std::is_same<V, float2>::value;
-    extern __shared__ __align__(16) unsigned char fuse_ring[];
-    V* ring = reinterpret_cast<V*>(fuse_ring);
-    step_begin();
+// Two steps of columns [x0, x0 + wn) of (pair) rows [r0, r1); wn + 2w <= NC.  E: what the arrays hold of
+// a column (float2: both nodes of a pair; float: one node), V: what a thread takes, one column
+// (V = E) or, in the plain layout, columns t and t + NT (E = float, V = float2).
+// rows >= 2w and nx >= 2w: no index wraps twice.  begin() is called before the first load.
+template <class E, class V, int NT, class Begin>
+__device__ __forceinline__ void two_steps(const PairParams& P, const E* __restrict__ src, E* __restrict__ dst, E* ring, int x0,
+                                          int wn, int r0, int r1, Begin begin) {
+    constexpr bool kPaired = std::is_same<E, float2>::value, kTwo = !std::is_same<E, V>::value;
+    constexpr int NC = kTwo ? 2 * NT : NT;   // columns of a ring row
     const int va = (int)P.sa, vb = (int)P.sb, w = max(va, vb);
     const int v[5] = {0, va, -va, vb, -vb};
     const int rows = kPaired ? P.half_ny : P.ny;
-    const int x0 = (int)((long long)P.nx * blockIdx.x / gridDim.x);
-    const int wn = (int)((long long)P.nx * (blockIdx.x + 1) / gridDim.x) - x0;
-    const int r0 = (int)((long long)rows * blockIdx.y / gridDim.y), r1 = (int)((long long)rows * (blockIdx.y + 1) / gridDim.y);
     const int t = threadIdx.x;
     const bool first = t < wn + 2 * w, second = t < wn;   // has a column in step 1, in step 2
-    unsigned col[5];
-    {
-        int x = x0 - w + (first ? t : 0);
+    // kTwo, the second column: t + NT, or the last one again in a narrow strip (stored in the ring twice, not in dst)
+    const int t1 = min(t + NT, wn + 2 * w - 1), t2 = min(t + NT, wn - 1);
+    auto pulled_columns = [&](int c, unsigned (&col)[5]) {
+        int x = x0 - w + c;
         x = x < 0 ? x + P.nx : (x >= P.nx ? x - P.nx : x);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             const int k = x + P.vxm[i];
             col[i] = (unsigned)(k >= P.nx ? k - P.nx : k);
         }
-    }
+    };
+    unsigned col[5], col1[5];
+    pulled_columns(first ? t : 0, col);
+    if constexpr (kTwo) pulled_columns(t1, col1);
     int depth[5], base[5], slot[5];   // rows of population column j in the ring, where they start, the row in turn
     {
         int o = 0;
@@ -87,7 +85,7 @@ k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* 
             depth[j] = w + v[j] + 1;
             base[j] = o;
             slot[j] = 0;
-            o += depth[j] * 5 * NT;
+            o += depth[j] * 5 * NC;
         }
     }
     V g[25];
@@ -105,7 +103,13 @@ k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* 
 #pragma unroll
         for (int i = 0; i < 5; ++i)
 #pragma unroll
-            for (int j = 0; j < 5; ++j) g[5 * i + j] = __ldg(src + (5 * i + j) * P.plane2 + (row[j] + col[i]));
+            for (int j = 0; j < 5; ++j) {
+                const E* q = src + (5 * i + j) * P.plane2;
+                if constexpr (kTwo)
+                    g[5 * i + j] = f2(__ldg(q + (row[j] + col[i])), __ldg(q + (row[j] + col1[i])));
+                else
+                    g[5 * i + j] = __ldg(q + (row[j] + col[i]));
+            }
         if constexpr (kPaired) {
             if (any) {
 #pragma unroll
@@ -115,7 +119,7 @@ k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* 
         }
     };
     V rho, th, drho, jx, jy, e;
-    step_wait();
+    begin();
     if (first) load(r0 - w);
     for (int rr = r0 - w; rr < r1 + w; ++rr) {
         if (first) {
@@ -124,9 +128,14 @@ k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* 
             flag_unhealthy(P, rho, th);
 #pragma unroll
             for (int j = 0; j < 5; ++j) {
-                V* q = ring + base[j] + slot[j] * 5 * NT + t;
+                E* q = ring + base[j] + slot[j] * 5 * NC;
 #pragma unroll
-                for (int i = 0; i < 5; ++i) q[i * NT] = o[5 * i + j];
+                for (int i = 0; i < 5; ++i) {
+                    if constexpr (kTwo)
+                        q[i * NC + t] = o[5 * i + j].x, q[i * NC + t1] = o[5 * i + j].y;
+                    else
+                        q[i * NC + t] = o[5 * i + j];
+                }
             }
             if (rr + 1 < r1 + w) load(rr + 1);
         }
@@ -138,18 +147,68 @@ k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* 
             V o[25];
 #pragma unroll
             for (int j = 0; j < 5; ++j) {
-                const V* q = ring + base[j] + slot[j] * 5 * NT + t + w;
+                const E* q = ring + base[j] + slot[j] * 5 * NC + w;
 #pragma unroll
-                for (int i = 0; i < 5; ++i) o[5 * i + j] = q[i * NT - v[i]];
+                for (int i = 0; i < 5; ++i) {
+                    if constexpr (kTwo)
+                        o[5 * i + j] = f2(q[i * NC + t - v[i]], q[i * NC + t2 - v[i]]);
+                    else
+                        o[5 * i + j] = q[i * NC + t - v[i]];
+                }
             }
             sym5_collide<V>(P, [&](int p) { return o[p]; }, [&](int p) { return o[p]; }, o, rho, th, drho, jx, jy, e);
             flag_unhealthy(P, rho, th);
-            const unsigned here = (unsigned)(rr - w) * (unsigned)P.pitch + (unsigned)(x0 + t);
+            E* q = dst + ((unsigned)(rr - w) * (unsigned)P.pitch + (unsigned)(x0 + t));
 #pragma unroll
-            for (int p = 0; p < 25; ++p) dst[p * P.plane2 + here] = o[p];
+            for (int p = 0; p < 25; ++p) {
+                if constexpr (kTwo) {
+                    q[p * P.plane2] = o[p].x;
+                    if (t + NT < wn) q[p * P.plane2 + NT] = o[p].y;
+                } else {
+                    q[p * P.plane2] = o[p];
+                }
+            }
         }
         __syncthreads();
     }
+}
+
+// One lattice: grid = (strips, segments), CTA (b, s) owns columns [nx b / strips, nx (b + 1) / strips) of
+// (pair) rows [rows s / segments, rows (s + 1) / segments).
+template <class V, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+k_two_steps(const __grid_constant__ PairParams P, const V* __restrict__ src, V* __restrict__ dst) {
+    extern __shared__ __align__(16) unsigned char fuse_ring[];
+    step_begin();
+    const int rows = std::is_same<V, float2>::value ? P.half_ny : P.ny;
+    const int x0 = (int)((long long)P.nx * blockIdx.x / gridDim.x);
+    const int x1 = (int)((long long)P.nx * (blockIdx.x + 1) / gridDim.x);
+    const int r0 = (int)((long long)rows * blockIdx.y / gridDim.y);
+    const int r1 = (int)((long long)rows * (blockIdx.y + 1) / gridDim.y);
+    two_steps<V, V, NT>(P, src, dst, reinterpret_cast<V*>(fuse_ring), x0, x1 - x0, r0, r1, [] { step_wait(); });
+}
+
+// The lattices of a batch in one launch: CTA c takes piece c of the list, longest first (FusePiece,
+// plbm_internal.h).  Both layouts run on one shape of CTA, 96 threads and two resident: the plain one takes
+// two columns a thread (97 against 89 us a step at 2047^2, but no second launch with its own tail).
+// 16 lattices of 58 to 932 rows of pairs or nodes, 6.0 M nodes: 174 us a step by k_batch_pair, 120 here.
+__global__ void __launch_bounds__(kBatchFuseThreads, 2)
+k_batch_two_steps(const PairParams* __restrict__ inst, const FusePiece* __restrict__ pieces, int parity) {
+    extern __shared__ __align__(16) unsigned char fuse_ring[];
+    __shared__ PairParams sp;
+    step_begin();
+    const FusePiece p = pieces[blockIdx.x];
+    for (int k = threadIdx.x; k < (int)(sizeof(PairParams) / sizeof(int)); k += kBatchFuseThreads)
+        reinterpret_cast<int*>(&sp)[k] = reinterpret_cast<const int*>(&inst[p.inst])[k];
+    __syncthreads();
+    if (sp.paired)
+        two_steps<float2, float2, kBatchFuseThreads>(sp, static_cast<const float2*>(sp.f[parity]), static_cast<float2*>(sp.f[parity ^ 1]),
+                                                     reinterpret_cast<float2*>(fuse_ring), p.x0, p.wn, p.r0, p.r1,
+                                                     [] { step_wait(); });
+    else
+        two_steps<float, float2, kBatchFuseThreads>(sp, static_cast<const float*>(sp.f[parity]), static_cast<float*>(sp.f[parity ^ 1]),
+                                                    reinterpret_cast<float*>(fuse_ring), p.x0, p.wn, p.r0, p.r1,
+                                                    [] { step_wait(); });
 }
 
 // The split of a lattice for k_two_steps, or strips = 0 where single steps are taken: lattices whose
@@ -179,16 +238,21 @@ inline FusePlan fuse_plan(const LatticeParams& P) {
     return least < 0.95 * 2 * single_us ? best : FusePlan{0, 0};
 }
 
+// Shared memory for the resident CTAs (1 KB each besides what they ask for), the rest as cache.
+inline cudaError_t fuse_shared_memory(const void* kernel, size_t smem, int resident) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                (int)((resident * (smem + 1024) * 100 + (228 << 10) - 1) / (228 << 10)));
+}
+
 template <class V, int NT, int MINB>
 cudaError_t launch_two_steps_t(const LatticeParams& L, const void* src, void* dst, cudaStream_t stream) {
     const FusePlan plan = fuse_plan(L);
     const FuseShape shape = fuse_shape(L);
     if (plan.strips == 0 || shape.threads != NT) return cudaErrorInvalidValue;
     const auto kernel = k_two_steps<V, NT, MINB>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shape.smem);
-    if (e == cudaSuccess)   // shared memory for the resident CTAs (1 KB each besides), the rest as cache
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)((shape.resident * (shape.smem + 1024) * 100 + (228 << 10) - 1) / (228 << 10)));
+    const cudaError_t e = fuse_shared_memory(reinterpret_cast<const void*>(kernel), shape.smem, shape.resident);
     if (e != cudaSuccess) return e;
     return launch_dependent_smem(true, shape.smem, kernel, dim3(plan.strips, plan.segments), NT, stream, pair_params(L),
                                  static_cast<const V*>(src), static_cast<V*>(dst));
@@ -200,6 +264,15 @@ inline cudaError_t launch_two_steps(const LatticeParams& P, const void* src, voi
                         : launch_two_steps_t<float, 128, 3>(P, src, dst, stream);
     return P.paired ? launch_two_steps_t<float2, 64, 4>(P, src, dst, stream)
                     : launch_two_steps_t<float, 128, 4>(P, src, dst, stream);
+}
+
+constexpr size_t kBatchFuseSmem = 25 * (size_t)(kFuseMaxV + 1) * kBatchFuseThreads * sizeof(float2);
+inline cudaError_t launch_batch_two_steps(const PairParams* inst, const FusePiece* pieces, int npieces, int parity,
+                                          cudaStream_t stream) {
+    // 500 bytes and more of static shared memory besides the ring
+    const cudaError_t e = fuse_shared_memory(reinterpret_cast<const void*>(k_batch_two_steps), kBatchFuseSmem + 1024, 2);
+    if (e != cudaSuccess) return e;
+    return launch_dependent_smem(true, kBatchFuseSmem, k_batch_two_steps, npieces, kBatchFuseThreads, stream, inst, pieces, parity);
 }
 
 }  // namespace plbm

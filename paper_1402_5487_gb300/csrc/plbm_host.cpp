@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <vector>
 
@@ -1143,6 +1144,8 @@ struct PairGroup {
     unsigned short* d_tile_inst = nullptr;   // instance (index into table) of every tile
     size_t max_tiles = 0;                    // tiles at the smallest block_x
     int total_tiles = 0;
+    std::vector<plbm::FusePiece> pieces;     // two steps per launch (empty: single steps)
+    plbm::FusePiece* d_pieces = nullptr;
 };
 
 struct NodeGroup {
@@ -1166,7 +1169,7 @@ struct Batch {
     std::vector<NodeGroup> nodes;
     int order = PLBM_BATCH_ORDER_INTERLEAVED;
     int block_x = 128, ctas_per_sm = 0, sms = 0;
-    cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};  // [kind][start parity]
+    cudaGraphExec_t graph[3][2] = {};  // [persistent, per instance, runs of two-step launches][start parity]
     long long steps = 0;
     char err[512] = "";
 };
@@ -1283,6 +1286,77 @@ plbm_status batch_launch(Batch* b, int scheme, int parity, int ctas) {
     return PLBM_OK;
 }
 
+// Four steps of every instance (scheme 0): groups with pieces take them in two launches.
+plbm_status batch_launch4(Batch* b, int parity, int ctas) {
+    for (const PairGroup& g : b->pairs)
+        for (int k = 0; k < (g.pieces.empty() ? 4 : 2); ++k) {
+            if (g.pieces.empty())
+                BCK(plbm::launch_batch(g.prec, g.d_table, (int)g.table.size(), g.total_tiles, b->block_x, ctas,
+                                       parity ^ (k & 1), b->order == PLBM_BATCH_ORDER_INTERLEAVED ? g.d_tile_inst : nullptr,
+                                       b->stream));
+            else
+                BCK(plbm::launch_batch_two_steps_f32(g.d_table, g.d_pieces, (int)g.pieces.size(), parity ^ (k & 1), b->stream));
+        }
+    for (const NodeGroup& g : b->nodes)
+        for (int k = 0; k < 4; ++k)
+            BCK(plbm::launch_batch_node(g.prec, g.q1, g.d_params, g.d_span, g.total_tiles, g.ctas, parity ^ (k & 1),
+                                        g.d_tile_inst, b->stream));
+    return PLBM_OK;
+}
+
+// The pieces of an FP32 group for k_batch_two_steps: strips of at most 96 (node pairs) or 192 columns
+// less the halo, cut into segments of about `rows` rows, longest first; `rows` is the one whose
+// pieces, handed out in that order to 2 CTAs per SM, are done first.  Empty (single steps) for
+// groups with another |v| or fewer rows than a halo, for groups that fit in the second-level cache and where
+// the pieces would take longer than the memory takes for single steps (29 ns per 1,000 nodes, measured 174 us
+// for 6.0 M nodes; a row of a piece takes 2.15 us).
+std::vector<plbm::FusePiece> batch_pieces(const Batch* b, const PairGroup& g) {
+    std::vector<plbm::FusePiece> best;
+    if (g.prec != plbm::kF32) return best;
+    double nodes = 0;
+    for (int i : g.members) {
+        const plbm::LatticeParams& P = b->inst[i]->P;
+        const int w = (int)std::max(P.sa, P.sb), rows = P.paired ? P.half_ny : P.ny;
+        if (w > plbm::kFuseMaxV || rows < 2 * w || P.nx < 2 * w) return best;
+        nodes += (double)P.nx * P.ny;
+    }
+    if (nodes * 200 < 1.3e8) return best;
+    double least = 0.95 * 2 * nodes * 29e-6 / 2.15;   // rows
+    for (int rows : {16, 24, 32, 40, 48, 56, 64, 80, 96, 128, 160, 192, 256, 512, 1024}) {
+        struct Cut {
+            int cost;
+            plbm::FusePiece p;
+        };
+        std::vector<Cut> cuts;
+        for (size_t m = 0; m < g.members.size(); ++m) {
+            const plbm::LatticeParams& P = b->inst[g.members[m]]->P;
+            const int w = (int)std::max(P.sa, P.sb), all = P.paired ? P.half_ny : P.ny;
+            const int most = plbm::kBatchFuseThreads * (P.paired ? 1 : 2) - 2 * w;
+            const int strips = (P.nx + most - 1) / most, segs = (all + rows - 1) / rows;
+            for (int s = 0; s < segs; ++s)
+                for (int c = 0; c < strips; ++c) {
+                    const int x0 = (int)((long long)P.nx * c / strips), x1 = (int)((long long)P.nx * (c + 1) / strips);
+                    const int r0 = (int)((long long)all * s / segs), r1 = (int)((long long)all * (s + 1) / segs);
+                    cuts.push_back({r1 - r0 + 2 * w + 1, {(int)m, x0, x1 - x0, r0, r1}});
+                }
+        }
+        if (cuts.size() > 1u << 20) continue;
+        std::stable_sort(cuts.begin(), cuts.end(), [](const Cut& a, const Cut& c) { return a.cost > c.cost; });
+        std::vector<int> load(2 * (size_t)std::max(b->sms, 1), 0);   // a heap, least first
+        for (const Cut& c : cuts) {
+            std::pop_heap(load.begin(), load.end(), std::greater<int>());
+            load.back() += c.cost;
+            std::push_heap(load.begin(), load.end(), std::greater<int>());
+        }
+        const double time = *std::max_element(load.begin(), load.end());
+        if (time >= least) continue;
+        least = time;
+        best.clear();
+        for (const Cut& c : cuts) best.push_back(c.p);
+    }
+    return best;
+}
+
 // Groups the created instances and builds the groups' device tables.
 plbm_status batch_groups(Batch* b) {
     for (size_t i = 0; i < b->inst.size(); ++i) {
@@ -1323,6 +1397,7 @@ plbm_status batch_groups(Batch* b) {
         if (g.members.size() > 65535) { batch_err(b, "at most 65535 row-paired instances per precision"); return PLBM_E_ARG; }
     for (const NodeGroup& g : b->nodes)
         if (g.members.size() > 65535) { batch_err(b, "at most 65535 instances per group"); return PLBM_E_ARG; }
+    for (PairGroup& g : b->pairs) g.pieces = batch_pieces(b, g);
     // one allocation for every group's tables
     size_t total = 0;
     std::vector<size_t> off;
@@ -1331,6 +1406,8 @@ plbm_status batch_groups(Batch* b) {
         total += align_up(sizeof(plbm::PairParams) * g.members.size(), 256);
         off.push_back(total);
         total += align_up(sizeof(unsigned short) * std::max<size_t>(g.max_tiles, 1), 256);
+        off.push_back(total);
+        total += align_up(sizeof(plbm::FusePiece) * std::max<size_t>(g.pieces.size(), 1), 256);
     }
     std::vector<std::vector<unsigned short>> node_tiles(b->nodes.size());
     std::vector<std::vector<plbm::NodeSpan>> spans(b->nodes.size());
@@ -1371,6 +1448,10 @@ plbm_status batch_groups(Batch* b) {
     for (PairGroup& g : b->pairs) {
         g.d_table = reinterpret_cast<plbm::PairParams*>(b->tables + off[o++]);
         g.d_tile_inst = reinterpret_cast<unsigned short*>(b->tables + off[o++]);
+        g.d_pieces = reinterpret_cast<plbm::FusePiece*>(b->tables + off[o++]);
+        if (!g.pieces.empty())
+            BCK(cudaMemcpyAsync(g.d_pieces, g.pieces.data(), sizeof(plbm::FusePiece) * g.pieces.size(),
+                                cudaMemcpyHostToDevice, b->stream));
         for (int i : g.members) {
             const Handle* h = b->inst[i];
             plbm::PairParams Q = plbm::pair_params(h->P);
@@ -1524,14 +1605,22 @@ plbm_status plbm_batch_step(plbm_batch bb, long n, int mode) {
     int parity = parity0;
     long done = 0;
     const int ctas = batch_ctas(b);  // occupancy query outside any stream capture
+    bool fused = false;              // runs of four steps, two per launch where a group can
+    for (const PairGroup& g : b->pairs) fused |= scheme == 0 && !g.pieces.empty();
+    if (fused && !use_graph)
+        for (; done + 4 <= n; done += 4) {
+            const plbm_status st = batch_launch4(b, parity, ctas);
+            if (st != PLBM_OK) return st;
+        }
     if (use_graph) {
-        for (; done + 2 <= n; done += 2) {
-            cudaGraphExec_t& g = b->graph[scheme][parity];
+        while (done + 2 <= n) {
+            const int run = fused && done + 4 <= n ? 4 : 2;
+            cudaGraphExec_t& g = b->graph[run == 4 ? 2 : scheme][parity];
             if (!g) {
                 cudaGraph_t graph = nullptr;
                 BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-                plbm_status st = batch_launch(b, scheme, parity, ctas);
-                if (st == PLBM_OK) st = batch_launch(b, scheme, parity ^ 1, ctas);
+                plbm_status st = run == 4 ? batch_launch4(b, parity, ctas) : batch_launch(b, scheme, parity, ctas);
+                if (st == PLBM_OK && run == 2) st = batch_launch(b, scheme, parity ^ 1, ctas);
                 cudaError_t ec = cudaStreamEndCapture(b->stream, &graph);
                 cudaError_t ei = (st == PLBM_OK && ec == cudaSuccess) ? cudaGraphInstantiate(&g, graph, 0)
                                                                        : cudaSuccess;
@@ -1541,6 +1630,7 @@ plbm_status plbm_batch_step(plbm_batch bb, long n, int mode) {
                 BCK(ei);
             }
             BCK(cudaGraphLaunch(g, b->stream));
+            done += run;
         }
     }
     for (; done < n; ++done) {

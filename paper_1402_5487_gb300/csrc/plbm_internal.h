@@ -86,6 +86,13 @@ struct PairParams {
     int paired;                   // 1: row-paired layout, plane2 in pairs; 0: plain, plane2 in elements
 };
 
+// Two steps per launch (plbm_fuse.cuh): the largest |v|, and a CTA's part of a batch, columns
+// [x0, x0 + wn) of (pair) rows [r0, r1) of lattice inst of the group's table.
+constexpr int kFuseMaxV = 3, kBatchFuseThreads = 96;
+struct FusePiece {
+    int inst, x0, wn, r0, r1;
+};
+
 // Rows of tiles of a lattice in the batched runner: pair rows or rows.
 inline int tile_rows(const PairParams& Q) { return Q.paired ? Q.half_ny : Q.ny; }
 
@@ -282,6 +289,9 @@ cudaError_t launch_set_populations(int prec, const LatticeParams& P, const doubl
 // with tile_inst[t] the instance of global tile t.
 cudaError_t launch_batch(int prec, const PairParams* inst, int ninst, int total_tiles, int block_x,
                          int ctas, int parity, const unsigned short* tile_inst, cudaStream_t stream);
+// Two steps of every lattice of an FP32 group (thermal, sets with |v| <= kFuseMaxV), a CTA per piece.
+cudaError_t launch_batch_two_steps_f32(const PairParams* inst, const FusePiece* pieces, int npieces, int parity,
+                                       cudaStream_t stream);
 cudaError_t batch_occupancy(int prec, int block_x, int* blocks_per_sm);
 
 // Number of blocks of a step launch (row-paired kernels cover two rows per block row).

@@ -22,6 +22,10 @@ bool two_steps_f32(const LatticeParams& P) { return fuse_plan(P).strips > 0; }
 cudaError_t launch_two_steps_f32(const LatticeParams& P, const void* src, void* dst, cudaStream_t stream) {
     return launch_two_steps(P, src, dst, stream);
 }
+cudaError_t launch_batch_two_steps_f32(const PairParams* inst, const FusePiece* pieces, int npieces, int parity,
+                                       cudaStream_t stream) {
+    return launch_batch_two_steps(inst, pieces, npieces, parity, stream);
+}
 cudaError_t launch_steps1_f32(const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
     return launch_steps1_t<float>(P, src, dst, steps, stream);
 }

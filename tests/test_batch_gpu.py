@@ -170,6 +170,33 @@ def test_mixed_batch_instances_vs_oracle_100_steps():
     b.close()
 
 
+# FP32 lattices beyond the second-level cache take two steps per launch in runs of four: both layouts,
+# sets with w = 2 and 3 in either order, strips of one column more or less, a thin lattice, beside
+# groups that take single steps; every scheme, and instances stepped alone between (an even number).
+def test_two_steps_per_launch_of_a_batch_equal_single_steps():
+    mk = lambda k, L, v, om, th, prec=None: I.Instance(index=k, L=L, v=v, omega=om, theta0=th, kind="kh", seed=900 + k, prec=prec)
+    v2, v3 = I.SET_012, I.SET_013
+    inst = [mk(0, 514, v3, 1.3, 1.0), mk(1, 513, v2, 1.2, 0.7), mk(2, 181, v3, 1.1, 1.0), mk(3, 98, v3, 1.2, 0.9),
+            mk(4, 60, v2, 1.1, 0.8), mk(5, 640, (0, 3, -3, 1, -1), 1.2, 1.0), mk(6, 187, (0, 2, -2, 1, -1), 1.1, 0.7),
+            mk(7, 12, v3, 1.2, 1.0), mk(8, 9, v2, 1.2, 0.7), mk(9, 72, v3, 1.3, 1.0, "f64"), mk(10, 66, v3, 1.2, 1.0, "f16dev")]
+    got = []
+    for parts, mode in (((11,), "per_instance"), ((11,), "persistent"), ((11,), "persistent_graph"), ((4, 6, 1), "persistent_graph"),
+                        ((1, 10), "persistent"), ((5, -2, 4), "persistent_graph")):
+        b = B.Batch(inst, prec="f32")
+        b.init()
+        for k in parts:
+            if k > 0:
+                b.step(k, mode)
+            else:
+                for s in b.solvers:
+                    s.step(-k)
+        assert b.check()[0] == plbm.PLBM_OK
+        got.append([s.get_populations() for s in b.solvers])
+        b.close()
+    for g in got[1:]:
+        assert all(np.array_equal(x, y) for x, y in zip(got[0], g))
+
+
 def test_full_sweep_sampled_nodes():
     # The bench's sweep (256 instances drawn by the R8 gates, sides over every
     # integer of [64, 1024], 1.0e8 nodes) in its timed launch scheme: after k steps a
