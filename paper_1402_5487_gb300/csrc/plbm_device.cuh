@@ -501,17 +501,45 @@ __device__ __forceinline__ double recip_f64(double x) {
     return fma(y, fma(e, e, e), y);
 }
 
+// Sums of doubles on the integer pipe.  x = fixed_of(f, E) is f in units of 2^(E - 1080), E the largest
+// biased exponent among the terms: five bits below the last place of the largest, so that a sum of up to
+// 25 of them fits in 63 bits and is exact but for the rounding of each term, 2^-57 of the largest (the
+// last bit of a term that loses bits is set to 1, which errs to either side alike; an FP64 sum rounds
+// each addition to 2^-53 of itself).  f64_of_fixed rounds the sum to nearest even.
+__device__ __forceinline__ long long fixed_of(double f, int E) {
+    const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
+    const int e = (int)((hi >> 20) & 0x7ffu), d = min(E - e, 63);
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+    const long long x = (long long)(((m << 5) >> d) | (d > 5 ? 1ull : 0ull));
+    const long long s = (long long)((int)hi >> 31);
+    return (x ^ s) - s;
+}
+__device__ __forceinline__ double f64_of_fixed(long long x, int E) {
+    const long long s = x >> 63;
+    unsigned long long m = (unsigned long long)((x ^ s) - s);
+    const int lz = __clzll((long long)m);
+    m <<= lz & 63;
+    const unsigned rem = (unsigned)m & 0x7ffu;
+    unsigned long long q = m >> 11;
+    q += (rem + ((unsigned)q & 1u)) > 0x400u ? 1u : 0u;
+    const unsigned long long bits = q + ((unsigned long long)(unsigned)(E + 5 - lz) << 52);   // q carries the exponent's last unit
+    return __longlong_as_double(x ? (long long)(bits | ((unsigned long long)s & 0x8000000000000000ull)) : 0ll);
+}
+
 // ---------------------------------------------------------------------------
 // FP64 core of the symmetric five-velocity sets (0, +-a, +-b).  The FP64 pipe (two
-// lanes per SM and cycle) bounds these steps, so what counts is the number of FP64
-// instructions: 152 per 2D node against 202 with DirectCore (general velocities and
-// coefficients, FP64 status comparisons).  The rule in constraint form
-// (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b), r_(+-a) = E_a +- O_a,
-// r_(+-b) = E_b +- O_b) takes 16 instructions per axis instead of 31; the sums
-// share S_1 + S_2 and the like; the velocities and factors are FP64 constants of the
-// lattice.  (Differences T_1 - T_2 formed as (T_1 + T_2) - 2 T_2 save two more
-// instructions, 1.2 % of the time, and put u_y 25 % further from the exact value.)
-// Per step: 1024^2 D2Q25 414 -> 301 us (274 us of FP64 issue), 128^2 10.2 -> 7.95 us,
+// lanes per SM and cycle: 64 cycles of an SM quarter for a warp's instruction) bounds
+// these steps, so what counts is the number of FP64 instructions: 105 per 2D node against
+// 202 with DirectCore (general velocities and coefficients, FP64 status comparisons).
+// The rule in constraint form (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b),
+// r_(+-a) = E_a +- O_a, r_(+-b) = E_b +- O_b) takes 16 instructions per axis instead of
+// 31; the velocities and factors are FP64 constants of the lattice; and in 2D the 47
+// additions of the moment sums run on the integer pipe (fixed_of: 15 integer instructions a
+// population, where an FP64 one leaves room for 64), exact but for 2^-57 of the largest
+// population: after 200 steps of the 128^2 shear layer u_y is 2.0e-13 from the exact
+// value (2.06e-13 with FP64 sums, 2.34e-13 with DirectCore), the others 1.6-30 times nearer.
+// Per step: 1024^2 D2Q25 414 us with DirectCore, 301 with FP64 sums, 206 now (189 of FP64
+// issue), 128^2 10.2, 7.95 and 7.0,
 // the 1000-node D1Q5 tube 4.05 -> 3.2 us.  The identities sum r = 1, sum v^2 r = mu_2
 // hold by construction, so the global sums drift less: mean density of 1024^2 after
 // 40 steps 2e-16 off against 7e-15 (rounded C mu sums), energy 4e-16 against 5e-15.
@@ -540,33 +568,71 @@ struct Sym5Core {
         r[4] = fma(-P.dkOb, yb, Eb);
     }
 
-    static __device__ __forceinline__ void moments(const double (&f)[Q], const LatticeParams& P, double& rho, double& th,
-                                                   double& jx, double& jy, double& e, double& ux, double& uy) {
-        double S[5], T[5], Tp = 0.0, Tq = 0.0;
+    // What the moments need of the populations: rho and per axis the differences and sums of the
+    // columns of opposite velocities (dp = S_1 - S_2, dq = S_3 - S_4; ep, eq: the sums over both axes).
+    struct Sums {
+        double rho, dpx, dqx, dpy, dqy, ep, eq;
+    };
+    static __device__ __forceinline__ Sums sums_f64(const double (&f)[Q]) {
+        double S[5];
+        Sums o;
         if constexpr (DIM == 2) {
+            double T[5];
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                const double p = f[5 * i + 1] + f[5 * i + 2], q = f[5 * i + 3] + f[5 * i + 4];
-                S[i] = (f[5 * i] + p) + q;
-            }
+            for (int i = 0; i < 5; ++i)
+                S[i] = (f[5 * i] + (f[5 * i + 1] + f[5 * i + 2])) + (f[5 * i + 3] + f[5 * i + 4]);
 #pragma unroll
             for (int j = 1; j < 5; ++j) T[j] = (f[j] + (f[5 + j] + f[10 + j])) + (f[15 + j] + f[20 + j]);
-            Tp = T[1] + T[2];
-            Tq = T[3] + T[4];
+            o.dpy = T[1] - T[2];
+            o.dqy = T[3] - T[4];
+            o.ep = T[1] + T[2];
+            o.eq = T[3] + T[4];
         } else {
 #pragma unroll
             for (int i = 0; i < 5; ++i) S[i] = f[i];
+            o.dpy = o.dqy = o.ep = o.eq = 0.0;
         }
         const double Sp = S[1] + S[2], Sq = S[3] + S[4];
-        rho = S[0] + Sp + Sq;
-        jx = fma(P.da, S[1] - S[2], __dmul_rn(P.db, S[3] - S[4]));
-        jy = 0.0;
+        o.rho = S[0] + Sp + Sq;
+        o.dpx = S[1] - S[2];
+        o.dqx = S[3] - S[4];
+        o.ep = DIM == 2 ? Sp + o.ep : Sp;
+        o.eq = DIM == 2 ? Sq + o.eq : Sq;
+        return o;
+    }
+
+    static __device__ __forceinline__ Sums sums(const double (&f)[Q]) {
         if constexpr (DIM == 2) {
-            jy = fma(P.da, T[1] - T[2], __dmul_rn(P.db, T[3] - T[4]));
-            e = fma(P.da2, Sp + Tp, __dmul_rn(P.db2, Sq + Tq));
+            unsigned top = 0u;
+#pragma unroll
+            for (int p = 0; p < Q; ++p) top = max(top, (unsigned)__double2hiint(f[p]) & 0x7fffffffu);
+            const int E = (int)(top >> 20);
+            if (E < 64 || E > 1900) return sums_f64(f);   // NaN, infinite, near either end of the range
+            long long S[5], T[5];
+#pragma unroll
+            for (int i = 0; i < 5; ++i)
+#pragma unroll
+                for (int j = 0; j < 5; ++j) {
+                    const long long x = fixed_of(f[5 * i + j], E);
+                    S[i] = j ? S[i] + x : x;
+                    if (j) T[j] = i ? T[j] + x : x;
+                }
+            const long long Sp = S[1] + S[2], Sq = S[3] + S[4];
+            return {f64_of_fixed(S[0] + Sp + Sq, E),          f64_of_fixed(S[1] - S[2], E), f64_of_fixed(S[3] - S[4], E),
+                    f64_of_fixed(T[1] - T[2], E),             f64_of_fixed(T[3] - T[4], E),
+                    f64_of_fixed(Sp + (T[1] + T[2]), E),      f64_of_fixed(Sq + (T[3] + T[4]), E)};
         } else {
-            e = fma(P.da2, Sp, __dmul_rn(P.db2, Sq));
+            return sums_f64(f);
         }
+    }
+
+    static __device__ __forceinline__ void moments(const double (&f)[Q], const LatticeParams& P, double& rho, double& th,
+                                                   double& jx, double& jy, double& e, double& ux, double& uy) {
+        const Sums s = sums(f);
+        rho = s.rho;
+        jx = fma(P.da, s.dpx, __dmul_rn(P.db, s.dqx));
+        jy = DIM == 2 ? fma(P.da, s.dpy, __dmul_rn(P.db, s.dqy)) : 0.0;
+        e = fma(P.da2, s.ep, __dmul_rn(P.db2, s.eq));
         const double inv = recip_f64(rho);
         ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
         const double ux2 = __dmul_rn(ux, ux), uy2 = __dmul_rn(uy, uy);

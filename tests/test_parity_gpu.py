@@ -766,6 +766,46 @@ def test_queued_steps_equal_awaited_steps(dim, v, shape, prec, kw):
     assert np.array_equal(got[0], got[1])
 
 
+# FP64 sums of five-velocity sets on the integer pipe: fields of given populations against exact
+# rational sums, over the exponent range and past both of its ends (there in FP64), with zeros,
+# negative values, a spread of 1e-9 and equal values.  A term is held to 2^-57 of the largest, a
+# sum and each operation after it round once: 25 2^-57 + 4 2^-53 of the sum of magnitudes.
+@pytest.mark.parametrize("kind", ["spread", "mixed", "equal", "zeros"])
+@pytest.mark.parametrize("scale", [1.0, 2.0**-958, 2.0**-961, 1e-300, 1e200, 2.0**876, 2.0**879, 1e300])
+def test_f64_sums_on_the_integer_pipe(kind, scale):
+    from fractions import Fraction as F
+    from paper_1402_5487_gb300 import plbm
+    nx, ny, v = 5, 4, I.SET_013
+    rng = np.random.default_rng(11)
+    f = rng.uniform(0.5, 1.0, (25, ny, nx))
+    if kind == "spread":
+        f *= 10.0 ** rng.uniform(-9, 0, f.shape)
+    elif kind == "mixed":
+        f *= np.where(rng.uniform(size=f.shape) < 0.2, -0.1, 1.0)
+    elif kind == "equal":
+        f[:] = 1.0
+    else:
+        f[rng.uniform(size=f.shape) < 0.5] = 0.0
+    f *= scale
+    s = plbm.Solver(2, v, 1.1, nx, ny, prec="f64")
+    s.set_populations(f)
+    rho, ux, uy, th = s.moments()
+    s.close()
+    for y in range(ny):
+        for x in range(nx):
+            g = [F(float(a)) for a in f[:, y, x]]
+            vx, vy = [v[p // 5] for p in range(25)], [v[p % 5] for p in range(25)]
+            m, size = sum(g), sum(abs(a) for a in g)
+            jx, jy = sum(a * b for a, b in zip(vx, g)), sum(a * b for a, b in zip(vy, g))
+            e = sum((a * a + b * b) * c for a, b, c in zip(vx, vy, g))
+            tol = F(25, 2**57) + F(4, 2**53)
+            assert abs(F(float(rho[y, x])) - m) <= tol * size
+            amp = size / m   # how much the sums cancel
+            assert abs(F(float(ux[y, x])) - jx / m) <= 2 * 3 * tol * amp * amp
+            assert abs(F(float(uy[y, x])) - jy / m) <= 2 * 3 * tol * amp * amp
+            assert abs(F(float(th[y, x])) - (e / m - (jx / m) ** 2 - (jy / m) ** 2) / 2) <= 40 * tol * amp * amp * amp
+
+
 # The final pass of the reductions (a cluster of blocks over one record per block of a step):
 # fewer records than blocks, one per thread, one more, several per thread.  The sums of the
 # populations themselves within 1e-13 of the sum of magnitudes, minima those of the fields.
