@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(128) k_moments_sym5_f64(const __grid_constant_
     double g[Sym5Core<DIM>::Q], r, t, e, jx, jy, a, b;
 #pragma unroll
     for (int p = 0; p < Sym5Core<DIM>::Q; ++p) g[p] = __ldg(f + elem_index(P, p, x, y));
-    Sym5Core<DIM>::moments(g, P, r, t, jx, jy, e, a, b);
+    Sym5Core<DIM>::moments(g, P, false, r, t, jx, jy, e, a, b);
     const long long n = (long long)y * P.nx + x;
     if (rho) rho[n] = r;
     if (ux) ux[n] = a;
@@ -404,10 +404,8 @@ __global__ void __launch_bounds__(128) k_init_sym5_f64(const __grid_constant__ L
     check_init_node(P, rho, ux, uy, theta, n);
     const double th = (P.isothermal || theta == nullptr) ? P.theta0 : theta[n];
     const double u = ux[n], v = DIM == 2 && uy ? uy[n] : 0.0, rh = rho[n];
-    const double sixth2 = __dmul_rn(__dmul_rn(6.0, th), th);
     double rx[5], ry[5];
-    Sym5Core<DIM>::axis(P, u, __dmul_rn(u, u), th, sixth2, rx);
-    if constexpr (DIM == 2) Sym5Core<DIM>::axis(P, v, __dmul_rn(v, v), th, sixth2, ry);
+    Sym5Core<DIM>::rule(P, u, v, th, false, rx, ry);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         const double X = rh * rx[i];

@@ -501,11 +501,16 @@ __device__ __forceinline__ double recip_f64(double x) {
     return fma(y, fma(e, e, e), y);
 }
 
+// A launch with no more than a few warps per SM quarter.
+__device__ __forceinline__ bool few_threads() { return (long long)gridDim.x * gridDim.y * blockDim.x < 1 << 16; }
+
 // Sums of doubles on the integer pipe.  x = fixed_of(f, E) is f in units of 2^(E - 1080), E the largest
 // biased exponent among the terms: five bits below the last place of the largest, so that a sum of up to
 // 25 of them fits in 63 bits and is exact but for the rounding of each term, 2^-57 of the largest (the
 // last bit of a term that loses bits is set to 1, which errs to either side alike; an FP64 sum rounds
-// each addition to 2^-53 of itself).  f64_of_fixed rounds the sum to nearest even.
+// each addition to 2^-53 of itself).  f64_of_fixed rounds the sum to nearest even, by the conversion
+// instruction, which takes the FP64 pipe, where there are few warps (few: their latency counts;
+// 128^2 7.2 -> 6.7 us a step) and by integer ones otherwise (1024^2 175 -> 160 us).
 __device__ __forceinline__ long long fixed_of(double f, int E) {
     const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
     const int e = (int)((hi >> 20) & 0x7ffu), d = min(E - e, 63);
@@ -514,7 +519,11 @@ __device__ __forceinline__ long long fixed_of(double f, int E) {
     const long long s = (long long)((int)hi >> 31);
     return (x ^ s) - s;
 }
-__device__ __forceinline__ double f64_of_fixed(long long x, int E) {
+__device__ __forceinline__ double f64_of_fixed(long long x, int E, bool few) {
+    if (few) {
+        const double d = __ll2double_rn(x);
+        return x ? __hiloint2double(__double2hiint(d) + (E - 1080) * (1 << 20), __double2loint(d)) : 0.0;
+    }
     const long long s = x >> 63;
     unsigned long long m = (unsigned long long)((x ^ s) - s);
     const int lz = __clzll((long long)m);
@@ -526,20 +535,39 @@ __device__ __forceinline__ double f64_of_fixed(long long x, int E) {
     return __longlong_as_double(x ? (long long)(bits | ((unsigned long long)s & 0x8000000000000000ull)) : 0ll);
 }
 
+// The product of two fixed-point numbers x / 2^m and y / 2^n as one over 2^(m + n - 63): the high
+// word of the product, whose lost bits are replaced by their mean (errs to either side alike).
+__device__ __forceinline__ long long fixed_mul(long long x, long long y) { return (__mul64hi(x, y) << 1) | 1; }
+// x times a small positive integer: two multiply instructions.
+__device__ __forceinline__ long long fixed_times(long long x, unsigned c) {
+    const unsigned long long lo = (unsigned long long)(unsigned)x * c;
+    return (long long)(((unsigned long long)((unsigned)(x >> 32) * c) << 32) + lo);
+}
+// x in units of 2^-n for |x| < 2^(63 - n); the last bit of one that loses bits is set to 1, as above.
+__device__ __forceinline__ long long fixed_n(double x, int n) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int e = (int)((hi >> 20) & 0x7ffu), d = min(1085 - n - e, 63);
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+    const long long q = (long long)(((m << 10) >> d) | (d > 10 ? 1ull : 0ull));
+    const long long s = (long long)((int)hi >> 31);
+    return (q ^ s) - s;
+}
+
 // ---------------------------------------------------------------------------
 // FP64 core of the symmetric five-velocity sets (0, +-a, +-b).  The FP64 pipe (two
 // lanes per SM and cycle: 64 cycles of an SM quarter for a warp's instruction) bounds
-// these steps, so what counts is the number of FP64 instructions: 105 per 2D node against
+// these steps, so what counts is the number of FP64 instructions: 71 per 2D node against
 // 202 with DirectCore (general velocities and coefficients, FP64 status comparisons).
-// The rule in constraint form (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b),
-// r_(+-a) = E_a +- O_a, r_(+-b) = E_b +- O_b) takes 16 instructions per axis instead of
-// 31; the velocities and factors are FP64 constants of the lattice; and in 2D the 47
-// additions of the moment sums run on the integer pipe (fixed_of: 15 integer instructions a
-// population, where an FP64 one leaves room for 64), exact but for 2^-57 of the largest
-// population: after 200 steps of the 128^2 shear layer u_y is 2.0e-13 from the exact
-// value (2.06e-13 with FP64 sums, 2.34e-13 with DirectCore), the others 1.6-30 times nearer.
-// Per step: 1024^2 D2Q25 414 us with DirectCore, 301 with FP64 sums, 206 now (189 of FP64
-// issue), 128^2 10.2, 7.95 and 7.0,
+// The moment sums (47 additions in 2D) and the rule run on the integer pipe, which has
+// room for 64 instructions beside an FP64 one: the sums in block fixed point (fixed_of),
+// the rule in constraint form (plbm_pair.cuh, here for r itself: r_0 = 1 - 2 (E_a + E_b),
+// r_(+-a) = E_a +- O_a, r_(+-b) = E_b +- O_b) in 64-bit fixed point, or, outside the range
+// of that, in 16 FP64 instructions per axis instead of 31; the velocities and factors
+// are constants of the lattice.  Both are nearer to the exact value than FP64 is: against
+// 80-bit arithmetic, 200 steps of the 128^2 shear layer leave u_x 6e-15 and u_y 1.4e-13
+// off (DirectCore 1.3e-14, 2.3e-13), 40 of a 192^2 one 1.5e-15 and 2.8e-14 (3.8e-15, 6.1e-14).
+// Per step: 1024^2 D2Q25 414 us with DirectCore, 301 with all of this core in FP64, 206 with the
+// sums on the integer pipe, 154 now (127 of FP64 issue); 128^2 10.2, 7.95, 7.0, 6.7;
 // the 1000-node D1Q5 tube 4.05 -> 3.2 us.  The identities sum r = 1, sum v^2 r = mu_2
 // hold by construction, so the global sums drift less: mean density of 1024^2 after
 // 40 steps 2e-16 off against 7e-15 (rounded C mu sums), energy 4e-16 against 5e-15.
@@ -566,6 +594,55 @@ struct Sym5Core {
         r[2] = fma(-P.dkOa, ya, Ea);
         r[3] = fma(P.dkOb, yb, Eb);
         r[4] = fma(-P.dkOb, yb, Eb);
+    }
+
+    // The same in 64-bit fixed point, for |u| < 1/2, 0 < th < 3/2 and |v| <= 3 (fixed_ok; every number then
+    // fits): bits after the point in the names.  Nothing keeps fewer than 57 (an FP64 mu_4 has 50 to 52), and r
+    // is 13 to 80 times nearer to the exact value before it is rounded to FP64.  O_a and E_a follow from the
+    // rounded O_b and E_b, so that sum r = 1, sum v r = u and sum v^2 r = mu_2 hold without a
+    // systematic error in the last place, which the steps would add up.
+    struct Theta {
+        long long t61, six57;   // theta, 6 theta^2
+    };
+    static __device__ __forceinline__ bool fixed_ok(const LatticeParams& P, double u, double th) {
+        return P.fixed_rule && ((unsigned)__double2hiint(u) & 0x7fffffffu) < 0x3fe00000u &&
+               (unsigned)__double2hiint(th) < 0x3ff80000u;
+    }
+    static __device__ __forceinline__ Theta theta_fixed(double th) {
+        Theta t;
+        t.t61 = fixed_n(th, 61);
+        t.six57 = (3 * fixed_mul(t.t61, t.t61)) >> 1;
+        return t;
+    }
+    static __device__ __forceinline__ void axis_fixed(const LatticeParams& P, double ud, Theta th, bool few, double (&r)[5]) {
+        const long long u60 = fixed_n(ud, 60), u62 = u60 << 2;
+        const long long m61 = fixed_mul(u62, u62) + th.t61;          // mu_2
+        const long long A60 = (m61 >> 1) + th.t61;                   // u^2 + 3 theta
+        const long long yb59 = fixed_mul(u62, A60) - fixed_times(u60 >> 1, P.ia2);
+        const long long zb57 = fixed_mul(A60, A60) - th.six57 - fixed_times(m61 >> 4, P.ia2);
+        const long long Ob = fixed_mul(yb59, P.ikOb65), Eb = fixed_mul(zb57 << 1, P.ikEb65) << 1;   // 61 bits from here
+        const long long w = 2 * (u60 - fixed_times(Ob, P.ib));                   // 2 a O_a, even
+        const long long Oa = P.ia2 == 1 ? w >> 1 : fixed_mul(w, P.ikOa63);
+        const long long Ea = fixed_mul(m61 - fixed_times(Eb, P.ib2x2), P.ikEa63);
+        r[0] = f64_of_fixed((1ll << 61) - 2 * (Ea + Eb), 1019, few);
+        r[1] = f64_of_fixed(Ea + Oa, 1019, few);
+        r[2] = f64_of_fixed(Ea - Oa, 1019, few);
+        r[3] = f64_of_fixed(Eb + Ob, 1019, few);
+        r[4] = f64_of_fixed(Eb - Ob, 1019, few);
+    }
+
+    // r of both axes (ry: 2D).
+    static __device__ __forceinline__ void rule(const LatticeParams& P, double ux, double uy, double th, bool few,
+                                                double (&rx)[5], double (&ry)[5]) {
+        if (fixed_ok(P, ux, th) && (DIM == 1 || fixed_ok(P, uy, th))) {
+            const Theta t = theta_fixed(th);
+            axis_fixed(P, ux, t, few, rx);
+            if constexpr (DIM == 2) axis_fixed(P, uy, t, few, ry);
+        } else {
+            const double sixth2 = __dmul_rn(__dmul_rn(6.0, th), th);
+            axis(P, ux, __dmul_rn(ux, ux), th, sixth2, rx);
+            if constexpr (DIM == 2) axis(P, uy, __dmul_rn(uy, uy), th, sixth2, ry);
+        }
     }
 
     // What the moments need of the populations: rho and per axis the differences and sums of the
@@ -601,7 +678,7 @@ struct Sym5Core {
         return o;
     }
 
-    static __device__ __forceinline__ Sums sums(const double (&f)[Q]) {
+    static __device__ __forceinline__ Sums sums(const double (&f)[Q], bool few) {
         if constexpr (DIM == 2) {
             unsigned top = 0u;
 #pragma unroll
@@ -618,17 +695,17 @@ struct Sym5Core {
                     if (j) T[j] = i ? T[j] + x : x;
                 }
             const long long Sp = S[1] + S[2], Sq = S[3] + S[4];
-            return {f64_of_fixed(S[0] + Sp + Sq, E),          f64_of_fixed(S[1] - S[2], E), f64_of_fixed(S[3] - S[4], E),
-                    f64_of_fixed(T[1] - T[2], E),             f64_of_fixed(T[3] - T[4], E),
-                    f64_of_fixed(Sp + (T[1] + T[2]), E),      f64_of_fixed(Sq + (T[3] + T[4]), E)};
+            auto out = [&](long long x) { return f64_of_fixed(x, E, few); };
+            return {out(S[0] + Sp + Sq),      out(S[1] - S[2]),          out(S[3] - S[4]),         out(T[1] - T[2]),
+                    out(T[3] - T[4]),         out(Sp + (T[1] + T[2])),   out(Sq + (T[3] + T[4]))};
         } else {
             return sums_f64(f);
         }
     }
 
-    static __device__ __forceinline__ void moments(const double (&f)[Q], const LatticeParams& P, double& rho, double& th,
-                                                   double& jx, double& jy, double& e, double& ux, double& uy) {
-        const Sums s = sums(f);
+    static __device__ __forceinline__ void moments(const double (&f)[Q], const LatticeParams& P, bool few, double& rho,
+                                                   double& th, double& jx, double& jy, double& e, double& ux, double& uy) {
+        const Sums s = sums(f, few);
         rho = s.rho;
         jx = fma(P.da, s.dpx, __dmul_rn(P.db, s.dqx));
         jy = DIM == 2 ? fma(P.da, s.dpy, __dmul_rn(P.db, s.dqy)) : 0.0;
@@ -640,21 +717,25 @@ struct Sym5Core {
         if constexpr (DIM == 2) th = __dmul_rn(th, 0.5);
     }
 
+    // few: see f64_of_fixed; one branch around the whole, as one at each conversion costs more than it gains
     static __device__ __forceinline__ void collide(double (&f)[Q], const LatticeParams& P, double& rho_o, double& th_o,
                                                    double& jx_o, double& jy_o, double& e_o) {
+        if (DIM == 2 && few_threads())   // 1D (1000 nodes): 1.80 us a step without the branch, 1.83 with it
+            collide_as(f, P, true, rho_o, th_o, jx_o, jy_o, e_o);
+        else
+            collide_as(f, P, false, rho_o, th_o, jx_o, jy_o, e_o);
+    }
+    static __device__ __forceinline__ void collide_as(double (&f)[Q], const LatticeParams& P, bool few, double& rho_o,
+                                                      double& th_o, double& jx_o, double& jy_o, double& e_o) {
         double rho, th, ux, uy;
-        moments(f, P, rho, th, jx_o, jy_o, e_o, ux, uy);
-        const double ux2 = __dmul_rn(ux, ux), uy2 = __dmul_rn(uy, uy);
+        moments(f, P, few, rho, th, jx_o, jy_o, e_o, ux, uy);
         rho_o = rho;
         th_o = th;
         if (P.isothermal) th = P.theta0;
-        const double sixth2 = __dmul_rn(__dmul_rn(6.0, th), th);
         const double om = P.omega;
-        double rx[5];
-        axis(P, ux, ux2, th, sixth2, rx);
+        double rx[5], ry[5];
+        rule(P, ux, uy, th, few, rx, ry);
         if constexpr (DIM == 2) {
-            double ry[5];
-            axis(P, uy, uy2, th, sixth2, ry);
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
                 const double X = __dmul_rn(rho, rx[i]);

@@ -467,6 +467,28 @@ plbm_status plbm_create(const plbm_desc* desc, plbm_handle* out) {
         P.dkEa = 1.0 / (2.0 * a * a);
         P.dkEb = 1.0 / (2.0 * b * b * (b * b - a * a));
         P.dcb = 1.0 / (b * b - a * a);
+        P.fixed_rule = a <= 3.0 && b <= 3.0;
+        if (P.fixed_rule) {   // 1 / n in units of 2^-k, rounded; all below 2^63
+            auto inv = [](int n, int k) {
+                const unsigned m = (unsigned)std::abs(n);
+                unsigned long long q = 0, rem = 1;   // 2^k / m by long division
+                for (int i = 0; i < k; ++i) {
+                    rem *= 2;
+                    q *= 2;
+                    if (rem >= m) rem -= m, ++q;
+                }
+                if (2 * rem >= m) ++q;
+                return n < 0 ? -(long long)q : (long long)q;
+            };
+            const int ia = v[1], ib = v[3], d = ib * ib - ia * ia;
+            P.ia2 = (unsigned)(ia * ia);
+            P.ib = (unsigned)ib;
+            P.ib2x2 = (unsigned)(2 * ib * ib);
+            P.ikEa63 = inv(2 * ia * ia, 63);
+            P.ikOa63 = inv(2 * ia, 63);
+            P.ikEb65 = inv(2 * ib * ib * d, 65);
+            P.ikOb65 = inv(2 * ib * d, 65);
+        }
     }
     // Row-paired layout and the two-nodes-per-thread kernel: 2D periodic symmetric
     // five-velocity thermal lattices with an even number of rows, 16/32-bit storage.

@@ -51,6 +51,11 @@ struct LatticeParams {
     float kOa, kOb, kEa, kEb;    // 1/(2a), 1/(2b(b^2-a^2)), 1/(2a^2), 1/(2b^2(b^2-a^2))
     double da, db, da2, db2, dkOa, dkOb, dkEa, dkEb;   // the same in FP64 ...
     double dcb;                  // ... and 1 / (b^2 - a^2) = 2 b kOb = 2 b^2 kEb
+    // the same for the rule in 64-bit fixed point (1: velocities of at most 3): a^2, b and 2 b^2, kEa and kOa times 2^63,
+    // kEb and kOb times 2^65
+    int fixed_rule;
+    unsigned ia2, ib, ib2x2;
+    long long ikEa63, ikEb65, ikOa63, ikOb65;
     float w1f[kMaxQ1];           // 1D rest weights r_i(0, theta0)
     float mu0f[kMaxQ1];          // mu_n(0, theta0)
     float W0f[kMaxQ];            // rest equilibrium w0_p (product of 1D weights in 2D)

@@ -806,6 +806,35 @@ def test_f64_sums_on_the_integer_pipe(kind, scale):
             assert abs(F(float(th[y, x])) - (e / m - (jx / m) ** 2 - (jy / m) ** 2) / 2) <= 40 * tol * amp * amp * amp
 
 
+# The FP64 rule in fixed point, on both sides of the range it is taken in (|u| < 1/2, theta < 3/2, |v| <= 3):
+# initial state and one step against the oracle.  Its C mu rule sums five terms of at most 30 (mu_4), 2^-53
+# of each; two axes; f' adds omega times that: 1e-12 of the largest population.
+@pytest.mark.parametrize("dim", [1, 2])
+@pytest.mark.parametrize("iso", [False, True])
+@pytest.mark.parametrize("v", [I.SET_013, I.SET_012, (0, 2, -2, 1, -1), (0, 3, -3, 1, -1), (0, 2, -2, 3, -3), (0, 1, -1, 4, -4)])
+def test_f64_rule_in_and_out_of_the_fixed_point_range(dim, iso, v):
+    rng = np.random.default_rng(13)
+    nx, ny = 40, 9 if dim == 2 else 1
+    edge = [0.5, np.nextafter(0.5, 0), -0.5, -np.nextafter(0.5, 0), 0.0, -0.0, 1e-300, 2.0**-9, 2.0**-30]
+    u = rng.uniform(-0.7, 0.7, (2, ny, nx))
+    u[0, 0, :9], u[1, 0, 9:18] = edge, edge
+    th = rng.uniform(0.2, 2.0, (ny, nx))
+    th[0, :4] = [1.5, np.nextafter(1.5, 0), 1e-12, 1e-300]
+    rho = rng.uniform(0.5, 2.0, (ny, nx))
+    s = plbm.Solver(dim, v, 1.2, nx, ny, theta0=1.0, prec="f64", isothermal=iso, skip_admissibility=True)
+    s.init(rho, u[0], u[1] if dim == 2 else None, None if iso else th)
+    lat = O.Lattice(dim, v, 1.2, nx, ny, theta0=1.0, isothermal=iso)
+    fo = lat.init(rho, u[0], u[1] if dim == 2 else 0 * u[1], 0 * th + 1.0 if iso else th)
+    for k in range(2):
+        g = s.get_populations()
+        o = np.asarray(fo).reshape(g.shape)
+        assert np.max(np.abs(g - o)) <= 1e-12 * np.max(np.abs(o)), k
+        if k == 0:
+            s.step(1)
+            fo = lat.run(fo, 1)
+    s.close()
+
+
 # The final pass of the reductions (a cluster of blocks over one record per block of a step):
 # fewer records than blocks, one per thread, one more, several per thread.  The sums of the
 # populations themselves within 1e-13 of the sum of magnitudes, minima those of the fields.
