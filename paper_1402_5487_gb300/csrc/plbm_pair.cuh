@@ -486,14 +486,14 @@ struct PairMinBlocks {
     static constexpr int value = PairStore<S>::kReconvert ? 7 : 0;
 };
 
-// grid = (ceil(nx / kBlockX), ny / 2); thread (x, r) owns nodes (x, r) and (x, r + ny/2).
+// grid = (ceil(nx / blockDim.x), ny / 2), blockDim.x = kBlockX when REDUCE; thread (x, r) owns nodes (x, r) and (x, r + ny/2).
 template <typename S, bool REDUCE>
 __global__ void __launch_bounds__(kBlockX, REDUCE ? 0 : PairMinBlocks<S>::value)
 k_stream_collide_pair(const __grid_constant__ PairParams P,
                       const typename PairStore<S>::V* __restrict__ src,
                       typename PairStore<S>::V* __restrict__ dst) {
     step_begin();
-    const int x = blockIdx.x * kBlockX + threadIdx.x;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
     NodeDiagF d;
     if (REDUCE) diagf_zero(d);
     step_wait();
@@ -510,7 +510,7 @@ template <typename S>
 cudaError_t launch_step_sym5_t(const LatticeParams& L, const void* src, void* dst, bool reduce,
                                cudaStream_t stream) {
     const PairParams P = pair_params(L);
-    int bx = kBlockX;
+    int bx = reduce ? kBlockX : 64;   // 511^2 6.49 -> 6.47 us a step, 255^2 3.14 -> 3.01 (128 before)
     if (!reduce && (long long)((P.nx + kBlockX - 1) / kBlockX) * P.ny < 2LL * device_sm_count()) bx = 32;
     dim3 grid((P.nx + bx - 1) / bx, P.ny);
     const S* s = static_cast<const S*>(src);
@@ -519,12 +519,22 @@ cudaError_t launch_step_sym5_t(const LatticeParams& L, const void* src, void* ds
                   : launch_dependent(false, k_stream_collide_sym5<S, false>, grid, bx, stream, P, s, t);
 }
 
+// Threads of a block without the reduction.  FP32: 64, whose slots refill in smaller pieces in the last wave (512^2,
+// 1.35 waves: 6.21 -> 5.96 us a step; 128, 96 and 32: 6.21, 6.05, 6.09), or 32 where that leaves
+// an SM fewer than five blocks (256^2 3.03 -> 2.83 us).  BF16: 128, the seven CTAs of PairMinBlocks.
+template <typename S>
+int pair_block(const PairParams& P) {
+    if (!std::is_same<S, float>::value) return kBlockX;
+    return (long long)P.nx * P.half_ny < 320LL * device_sm_count() ? 32 : 64;
+}
+
 template <typename S>
 cudaError_t launch_step_pair_t(const LatticeParams& L, const void* src, void* dst, bool reduce,
                                cudaStream_t stream) {
     using V = typename PairStore<S>::V;
     const PairParams P = pair_params(L);
-    dim3 grid((P.nx + kBlockX - 1) / kBlockX, P.half_ny);
+    const int bx = reduce ? kBlockX : pair_block<S>(P);
+    dim3 grid((P.nx + bx - 1) / bx, P.half_ny);
     const V* s = static_cast<const V*>(src);
     V* t = static_cast<V*>(dst);
     if constexpr (std::is_same<S, __half>::value) {
@@ -536,7 +546,7 @@ cudaError_t launch_step_pair_t(const LatticeParams& L, const void* src, void* ds
         }
     }
     return reduce ? launch_dependent(false, k_stream_collide_pair<S, true>, grid, kBlockX, stream, P, s, t)
-                  : launch_dependent(false, k_stream_collide_pair<S, false>, grid, kBlockX, stream, P, s, t);
+                  : launch_dependent(false, k_stream_collide_pair<S, false>, grid, bx, stream, P, s, t);
 }
 
 // ---------------------------------------------------------------------------
