@@ -43,9 +43,9 @@ namespace plbm {
 // 123.2 -> 120.6 us, FP16 69.7 -> 67.3 us, 512^2 FP32 (graph) 6.56 -> 6.29 us.
 // Grids of fewer than kDependentThreads threads leave slots free for several
 // waiting grids at once, which then crowd the running one (128^2 FP64: 10.2 ->
-// 16.4 us a step): 16/32-bit ones are launched plainly, FP64 ones, whose arithmetic
-// takes longer than a launch, say so only after it (step_end; 128^2 FP64 8.35 ->
-// 7.95 us a step, tube launches of four steps 8.1 -> 7.6 us).  The persistent batch
+// 16.4 us a step): FP64 kernels (step_end; 128^2 8.35 -> 7.95 us a step, tube launches of
+// four steps 8.1 -> 7.6 us) and 16/32-bit ones of five-velocity sets (LATE, plbm_pair.cuh) then
+// say so only after their arithmetic, others are launched plainly.  The persistent batch
 // kernels, which leave no slot free, are launched plainly (174 us a step either way).
 // ---------------------------------------------------------------------------
 constexpr long long kDependentThreads = 1 << 16;
