@@ -895,6 +895,7 @@ def main():
                              "frac": achieved / peak, "traffic": read_traffic(args.prec),
                              "peak_source": peak_kind + " (copy bandwidth, MEASURED_PEAKS.json hbm_gbs)",
                              "algorithmic_bytes_per_launch": alg_bytes,
+                             "steps_per_launch": args.steps / n_launches,
                              "kernel": KERNEL_NAME[args.prec]},
                 "repeats": {"n": REPEATS, "reported": "median",
                             "ms_per_step_each": [r / args.steps * 1e3 for r in runs],
