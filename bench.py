@@ -44,15 +44,14 @@ THETA0 = 1.0
 ELEM = {"f64": 8, "f32": 4, "f16dev": 2, "bf16dev": 2}
 
 
-KERNEL_NAME = {"f32": "k_two_steps<float2,96,2>", "f16dev": "k_stream_collide_pair2<__half>",
-               "bf16dev": "k_stream_collide_pair<__nv_bfloat16>", "f64": "k_stream_collide<double,5,2>"}
+KERNEL_NAME = {"f32": "k_two_steps<float2,96,2>", "f16dev": "k_two_steps<__half2,128,3>",
+               "bf16dev": "k_two_steps<__nv_bfloat162,128,3>", "f64": "k_stream_collide<double,5,2>"}
 
 
 def launches(prec, L, steps):
-    """Step kernels that ``steps`` steps of the L x L lattice in one call launch: FP32
-    lattices beyond the second-level cache take two steps a launch, in as many launches as
-    steps modulo 2."""
-    if prec != "f32" or L < 1024:
+    """Step kernels that ``steps`` steps of the L x L lattice (even L) in one call launch: large
+    16/32-bit lattices take two steps a launch, in as many launches as steps modulo 2."""
+    if L < {"f32": 1024, "f16dev": 2048, "bf16dev": 2048}.get(prec, 1 << 30):
         return steps
     n = (steps + 1) // 2
     return n + ((n ^ steps) & 1)

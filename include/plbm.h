@@ -194,8 +194,8 @@ plbm_status plbm_init(plbm_handle h, const double *rho, const double *ux, const 
  * launches, advance by replays of a CUDA graph of 32 steps (captured at first
  * use on a private stream, launched on the handle's stream; not when
  * check_every > 0 or while the handle's stream is being captured).  1D lattices
- * and 2D thermal FP32 lattices of a set (0, a, -a, b, -b) beyond the second-level
- * cache take several steps in one launch; the state is that of single steps. */
+ * and large 2D thermal 16/32-bit lattices of a set (0, a, -a, b, -b) take several
+ * steps in one launch; the state is that of single steps. */
 plbm_status plbm_step(plbm_handle h, long n);
 
 /* Read the device status word (synchronises the stream).  Returns

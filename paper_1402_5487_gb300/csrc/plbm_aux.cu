@@ -14,7 +14,11 @@ cudaError_t launch_step_f16(const LatticeParams&, const void*, void*, bool, cuda
 cudaError_t launch_step_bf16(const LatticeParams&, const void*, void*, bool, cudaStream_t);
 
 bool two_steps_f32(const LatticeParams&);
+bool two_steps_f16(const LatticeParams&);
+bool two_steps_bf16(const LatticeParams&);
 cudaError_t launch_two_steps_f32(const LatticeParams&, const void*, void*, cudaStream_t);
+cudaError_t launch_two_steps_f16(const LatticeParams&, const void*, void*, cudaStream_t);
+cudaError_t launch_two_steps_bf16(const LatticeParams&, const void*, void*, cudaStream_t);
 cudaError_t launch_steps1_f64(const LatticeParams&, const void*, void*, int, cudaStream_t);
 cudaError_t launch_steps1_f32(const LatticeParams&, const void*, void*, int, cudaStream_t);
 cudaError_t launch_steps1_f16(const LatticeParams&, const void*, void*, int, cudaStream_t);
@@ -99,7 +103,8 @@ cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void*
 // before the symmetric core alone) -> 1.87, 20,000 nodes 5.46 -> 3.54, 100,000 nodes
 // 18.95 -> 14.70 (k = 1); FP32 1.74 -> 0.53, 1.87 -> 0.91, 2.32 -> 1.55.
 int steps_per_launch(int prec, const LatticeParams& P) {
-    if (P.dim != 1) return prec == kF32 && two_steps_f32(P) ? 2 : 1;   // plbm_fuse.cuh
+    if (P.dim != 1)   // plbm_fuse.cuh
+        return (prec == kF32 && two_steps_f32(P)) || (prec == kF16Dev && two_steps_f16(P)) || (prec == kBF16Dev && two_steps_bf16(P)) ? 2 : 1;
     const int w = halo1(P), sms = device_sm_count();
     const double launch = 1.5, latency = prec == kF64 ? 1.5 : 0.25;
     auto time = [&](int k) {   // per step
@@ -116,7 +121,15 @@ int steps_per_launch(int prec, const LatticeParams& P) {
 }
 
 cudaError_t launch_steps(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
-    if (P.dim != 1) return steps == 2 && prec == kF32 ? launch_two_steps_f32(P, src, dst, stream) : cudaErrorInvalidValue;
+    if (P.dim != 1) {
+        if (steps != 2) return cudaErrorInvalidValue;
+        switch (prec) {
+            case kF32: return launch_two_steps_f32(P, src, dst, stream);
+            case kF16Dev: return launch_two_steps_f16(P, src, dst, stream);
+            case kBF16Dev: return launch_two_steps_bf16(P, src, dst, stream);
+        }
+        return cudaErrorInvalidValue;
+    }
     switch (prec) {
         case kF64: return launch_steps1_f64(P, src, dst, steps, stream);
         case kF32: return launch_steps1_f32(P, src, dst, steps, stream);

@@ -244,7 +244,7 @@ void set_thread_error(const char* msg);
 // on `stream` and return the launch error.
 cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void* dst,
                         bool reduce, cudaStream_t stream);
-// The number of steps best taken by one launch (1: launch_step; 1D lattices and large FP32
+// The number of steps best taken by one launch (1: launch_step; 1D lattices and large 2D 16/32-bit
 // ones take several), and a launch that takes `steps` of them (2 <= steps <= that number).
 int steps_per_launch(int prec, const LatticeParams& P);
 cudaError_t launch_steps(int prec, const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream);

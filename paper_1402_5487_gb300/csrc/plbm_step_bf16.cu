@@ -2,7 +2,7 @@
 // templates live in plbm_device.cuh; this unit only instantiates them so the
 // four precisions compile in parallel.  Row-paired lattices take the
 // two-nodes-per-thread kernel of plbm_pair.cuh.
-#include "plbm_pair.cuh"
+#include "plbm_fuse.cuh"
 
 namespace plbm {
 cudaError_t launch_step_bf16(const LatticeParams& P, const void* src, void* dst, bool reduce,
@@ -17,6 +17,10 @@ cudaError_t launch_batch_bf16(const PairParams* inst, int ninst, int total_tiles
 }
 cudaError_t batch_occupancy_bf16(int block_x, int* blocks_per_sm) {
     return batch_occupancy_t<__nv_bfloat16>(block_x, blocks_per_sm);
+}
+bool two_steps_bf16(const LatticeParams& P) { return fuse_plan<__nv_bfloat16>(P).strips > 0; }
+cudaError_t launch_two_steps_bf16(const LatticeParams& P, const void* src, void* dst, cudaStream_t stream) {
+    return launch_two_steps<__nv_bfloat16>(P, src, dst, stream);
 }
 cudaError_t launch_steps1_bf16(const LatticeParams& P, const void* src, void* dst, int steps, cudaStream_t stream) {
     return launch_steps1_t<__nv_bfloat16>(P, src, dst, steps, stream);

@@ -18,9 +18,9 @@ cudaError_t launch_batch_f32(const PairParams* inst, int ninst, int total_tiles,
 cudaError_t batch_occupancy_f32(int block_x, int* blocks_per_sm) {
     return batch_occupancy_t<float>(block_x, blocks_per_sm);
 }
-bool two_steps_f32(const LatticeParams& P) { return fuse_plan(P).strips > 0; }
+bool two_steps_f32(const LatticeParams& P) { return fuse_plan<float>(P).strips > 0; }
 cudaError_t launch_two_steps_f32(const LatticeParams& P, const void* src, void* dst, cudaStream_t stream) {
-    return launch_two_steps(P, src, dst, stream);
+    return launch_two_steps<float>(P, src, dst, stream);
 }
 cudaError_t launch_batch_two_steps_f32(const PairParams* inst, const FusePiece* pieces, int npieces, int parity,
                                        cudaStream_t stream) {

@@ -871,17 +871,20 @@ def test_final_pass_of_the_reductions(prec, shape):
     bad.close()
 
 
-# Large FP32 lattices advance two steps per launch (strips of columns, segments of rows): the
+# Large lattices advance two steps per launch (strips of columns, segments of rows): the
 # state must be that of single steps bit for bit, in both layouts, for odd and even step counts,
 # status reads between, a captured stream and a set in either order; strips one column apart in
 # width, a last wave with few blocks, few rows and few columns.
-@pytest.mark.parametrize("v,shape,plain", [
+@pytest.mark.parametrize("prec,v,shape,plain", [("f32", *c) for c in [
     (I.SET_013, (1024, 1024), False), (I.SET_013, (1009, 1030), False), (I.SET_013, (901, 901), False),
     (I.SET_013, (1200, 902), True), (I.SET_012, (1021, 1026), False), (I.SET_012, (1011, 1021), False),
     ((0, 3, -3, 1, -1), (960, 1026), False), ((0, 2, -2, 1, -1), (1031, 957), False), ((0, 2, -2, 3, -3), (1500, 800), False),
     (I.SET_013, (40000, 100), False), (I.SET_013, (90, 40000), False), (I.SET_013, (40000, 101), False),
-    (I.SET_012, (400000, 8), False), (I.SET_013, (700, 1000), False), ((0, 1, -1, 4, -4), (1024, 1024), False)])
-def test_two_steps_of_one_launch_equal_single_steps(v, shape, plain):
+    (I.SET_012, (400000, 8), False), (I.SET_013, (700, 1000), False), ((0, 1, -1, 4, -4), (1024, 1024), False)]] + [
+    ("f16dev", I.SET_013, (2051, 2050), False), ("f16dev", I.SET_012, (1900, 1726), False),
+    ("bf16dev", I.SET_013, (2301, 2204), False), ("bf16dev", (0, 3, -3, 1, -1), (1150, 4412), False),
+    ("f16dev", I.SET_013, (2500, 2501), False), ("bf16dev", (0, 2, -2, 1, -1), (2611, 2444), True), ("f16dev", I.SET_013, (1500, 900), False)])
+def test_two_steps_of_one_launch_equal_single_steps(prec, v, shape, plain):
     import torch
     from paper_1402_5487_gb300 import plbm
     nx, ny = shape
@@ -892,7 +895,7 @@ def test_two_steps_of_one_launch_equal_single_steps(v, shape, plain):
     side = torch.cuda.Stream()
 
     def run(parts, ce=0, how="step"):
-        s = plbm.Solver(2, v, 1.1, nx, ny, theta0=th0, prec="f32", plain_layout=plain, check_every=ce,
+        s = plbm.Solver(2, v, 1.1, nx, ny, theta0=th0, prec=prec, plain_layout=plain, check_every=ce,
                         skip_admissibility=True, stream=side)
         torch.cuda.synchronize()
         s.init(one, u[0], u[1], th0 * one)
