@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
 // for 256 x 256 x 128 FP16 nodes.  Float-float pairs hi + lo (error-free sums and
 // products, ~2^-47 relative) on the deviations from the rest state, whose magnitude
 // is a hundredth of f's (so the absolute error stays at FP64's on f), take 404 / 236 us
-// and 1,234 / 754 us, bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
+// and 1,234 / 754 us (388 by exact integer sums), bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
 // the z-paired layout a thread takes both nodes of a pair (V = float2: packed FP32x2
 // arithmetic, one aligned 4-byte access for the two); otherwise one node (V = float).
 // ---------------------------------------------------------------------------
@@ -890,13 +890,23 @@ __device__ __forceinline__ double lane_f64(FFV<float2> v, int l) {
 // Row sums R_ab = sum_c g, S_a, T_b, U_c of the stored deviations, then
 // rho - 1 = sum S, j = sum v S (per axis), E - 3 theta0 = sum v^2 (S + T + U); the
 // fields of each node in FP64.
+// The fields of a node from rho - 1, j and E - 3 theta0.
+__device__ __forceinline__ void put_fields3(const LatticeParams& P, long long n, double dm, double jx, double jy, double jz, double de,
+                                            double* rho, double* ux, double* uy, double* uz, double* theta) {
+    const double m = 1.0 + dm;
+    const double im = recip_f64(m);
+    const double a = jx * im, b = jy * im, c = jz * im;
+    if (rho) rho[n] = m;
+    if (ux) ux[n] = a;
+    if (uy) uy[n] = b;
+    if (uz) uz[n] = c;
+    if (theta) theta[n] = ((3.0 * P.theta0 + de) * im - (a * a + b * b + c * c)) * (1.0 / 3.0);
+}
+
 template <typename S, class V>
-__global__ void __launch_bounds__(kB3) k_moments3_dev(const __grid_constant__ LatticeParams P, const S* __restrict__ f,
-                                                      double* rho, double* ux, double* uy, double* uz, double* theta) {
+__device__ __forceinline__ void moments3_ff(const LatticeParams& P, const S* __restrict__ f, double* rho, double* ux, double* uy,
+                                            double* uz, double* theta, int x, int y, int z) {
     constexpr int kLanes = sizeof(V) / sizeof(float);
-    const int x = blockIdx.x * kB3 + threadIdx.x;
-    const int y = blockIdx.y, z = blockIdx.z;
-    if (x >= P.nx) return;
     const long long here = node3(P, x, y, z);
     const FFV<V> zero{splat<V>(0.0f), splat<V>(0.0f)};
     FFV<V> Sa[kQ1], Tb[kQ1], Uc[kQ1];
@@ -935,16 +945,79 @@ __global__ void __launch_bounds__(kB3) k_moments3_dev(const __grid_constant__ La
         de = ffv_acc(de, ffv_small(ffv_acc(ffv_acc(Sa[i], Tb[i]), Uc[i]), vi * vi));
     }
 #pragma unroll
-    for (int l = 0; l < kLanes; ++l) {
-        const double m = 1.0 + lane_f64(dm, l);
-        const double im = recip_f64(m);
-        const double a = lane_f64(jx, l) * im, b = lane_f64(jy, l) * im, c = lane_f64(jz, l) * im;
-        const long long n = ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x;
-        if (rho) rho[n] = m;
-        if (ux) ux[n] = a;
-        if (uy) uy[n] = b;
-        if (uz) uz[n] = c;
-        if (theta) theta[n] = ((3.0 * P.theta0 + lane_f64(de, l)) * im - (a * a + b * b + c * c)) * (1.0 / 3.0);
+    for (int l = 0; l < kLanes; ++l)
+        put_fields3(P, ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x, lane_f64(dm, l), lane_f64(jx, l), lane_f64(jy, l),
+                    lane_f64(jz, l), lane_f64(de, l), rho, ux, uy, uz, theta);
+}
+
+template <typename S, class V>
+__global__ void __launch_bounds__(kB3) k_moments3_dev(const __grid_constant__ LatticeParams P, const S* __restrict__ f,
+                                                      double* rho, double* ux, double* uy, double* uz, double* theta) {
+    const int x = blockIdx.x * kB3 + threadIdx.x;
+    if (x < P.nx) moments3_ff<S, V>(P, f, rho, ux, uy, uz, theta, x, blockIdx.y, blockIdx.z);
+}
+
+// FP16 pairs: every value is a multiple of 2^-24, so that below 1/4 (every healthy deviation) the sums are
+// exact 32-bit integers: the bits of g + 3/4 are 2^24 g and a constant, and a sum of n of them (modulo
+// 2^32) n constants off.  9 instructions a pair of values instead of 17 in float-float: 256 x 256 x 128
+// 754 -> 388 us (the bytes: 360).  A thread that meets a larger value, an infinity or a NaN starts over in float-float.
+__global__ void __launch_bounds__(kB3) k_moments3_f16pair(const __grid_constant__ LatticeParams P, const __half* __restrict__ f,
+                                                          double* rho, double* ux, double* uy, double* uz, double* theta) {
+    const int x = blockIdx.x * kB3 + threadIdx.x;
+    const int y = blockIdx.y, z = blockIdx.z;
+    if (x >= P.nx) return;
+    const unsigned* at = reinterpret_cast<const unsigned*>(f + node3(P, x, y, z));
+    const long long plane = P.plane / 2;
+    int2 S[kQ1], T[kQ1], U[kQ1];
+    __half2 most = __float2half2_rn(0.0f);
+#pragma unroll
+    for (int i = 0; i < kQ1; ++i) S[i] = T[i] = U[i] = make_int2(0, 0);
+#pragma unroll
+    for (int a = 0; a < kQ1; ++a)
+#pragma unroll
+        for (int b = 0; b < kQ1; ++b) {
+            int2 R = make_int2(0, 0);
+#pragma unroll
+            for (int c = 0; c < kQ1; ++c) {
+                const unsigned w = __ldg(at + ((a * kQ1 + b) * kQ1 + c) * plane);
+                __half2 h;
+                memcpy(&h, &w, 4);
+                most = __hmax2_nan(most, __habs2(h));
+                const float2 g = add2(__half22float2(h), f2s(0.75f));
+                const int gx = __float_as_int(g.x), gy = __float_as_int(g.y);
+                R.x += gx;
+                R.y += gy;
+                U[c].x += gx;
+                U[c].y += gy;
+            }
+            S[a].x += R.x;
+            S[a].y += R.y;
+            T[b].x += R.x;
+            T[b].y += R.y;
+        }
+    const float2 top = __half22float2(most);
+    if (!(top.x < 0.25f && top.y < 0.25f)) {
+        moments3_ff<__half, float2>(P, f, rho, ux, uy, uz, theta, x, y, z);
+        return;
+    }
+    const unsigned off = 25u * 0x3f400000u;   // 25 times the bits of 3/4
+    const long long va = P.v[1], vb = P.v[3];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        auto sum = [&](const int2& v) { return (long long)(int)((unsigned)(l ? v.y : v.x) - off); };
+        long long j[3], p = 0, q = 0, m = 0;
+        const int2* const axis[3] = {S, T, U};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const long long s1 = sum(axis[d][1]), s2 = sum(axis[d][2]), s3 = sum(axis[d][3]), s4 = sum(axis[d][4]);
+            if (d == 0) m = sum(S[0]) + (s1 + s2) + (s3 + s4);
+            j[d] = va * (s1 - s2) + vb * (s3 - s4);
+            p += s1 + s2;
+            q += s3 + s4;
+        }
+        auto value = [](long long i) { return f64_of_fixed(i, 1056, false); };   // units of 2^-24
+        put_fields3(P, ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x, value(m), value(j[0]), value(j[1]), value(j[2]),
+                    value(va * va * p + vb * vb * q), rho, ux, uy, uz, theta);
     }
 }
 
@@ -1305,6 +1378,12 @@ cudaError_t launch_moments3(int prec, const LatticeParams& P, const void* f, dou
         return cudaGetLastError();
     }
     if (!P.sym5) return cudaErrorInvalidValue;
+    if (prec == kF16Dev && P.zpaired) {
+        dim3 grid = grid3(P);
+        grid.z = P.half_nz;
+        k_moments3_f16pair<<<grid, kB3, 0, s>>>(P, static_cast<const __half*>(f), rho, ux, uy, uz, theta);
+        return cudaGetLastError();
+    }
     PLBM_LAUNCH3_DEV(k_moments3_dev, (P, static_cast<const S*>(f), rho, ux, uy, uz, theta))
     return cudaGetLastError();
 }

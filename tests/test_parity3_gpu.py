@@ -257,3 +257,39 @@ def test_d3q125_initial_state_and_fields_to_the_last_bit_of_storage(prec, shape,
     th = (np.tensordot((c * c).sum(1), got, 1) / rho - sum(a * a for a in u)) / 3
     for a, b in zip(mom, (rho, u[0], u[1], u[2], th)):
         assert np.max(np.abs(a - b)) <= 3e-14
+
+
+# Fields of FP16 pairs from exact 32-bit sums below 1/4 and in float-float from there on (and beside
+# non-finite values): random deviations with none, one at either edge, and large ones; sums of the
+# stored populations, 125 roundings of 2^-53 of the sum of magnitudes.
+@pytest.mark.parametrize("extra", [None, 0.25, -0.25, 0.2498779296875, -0.2498779296875, 2.0**-24, 7.5, -300.0, np.inf, np.nan])
+def test_d3q125_fp16_fields_from_exact_sums(extra):
+    from paper_1402_5487_gb300 import plbm
+    nx, ny, nz = 37, 3, 8
+    v = V5
+    rng = np.random.default_rng(17)
+    s = plbm.Solver(3, v, 1.1, nx, ny, nz=nz, theta0=1.0, prec="f16dev")
+    one = np.ones((nz, ny, nx))
+    s.init(one, 0 * one, 0 * one, theta=one, uz=0 * one)
+    f = s.get_populations().reshape(125, nz, ny, nx)
+    g = (0.01 * rng.uniform(-1, 1, f.shape) * 10.0 ** rng.uniform(-5, 0, f.shape)).astype(np.float16).astype(np.float64)
+    if extra is not None:
+        g[7, 1, 2, 5] = g[80, 6, 0, 36] = extra
+    s.set_populations((f + g).reshape(s.get_populations().shape))
+    p = s.get_populations().reshape(125, nz, ny, nx)
+    rho, ux, uy, uz, th = s.moments()
+    s.close()
+    c = np.array([(v[k // 25], v[k // 5 % 5], v[k % 5]) for k in range(125)], float)
+    ok = np.isfinite(p).all(axis=0)
+    assert ok.sum() == ok.size - (2 if extra is not None and not np.isfinite(extra) else 0)
+    p = np.where(ok, p, 1.0)
+    m, size = p.sum(0), np.abs(p).sum(0)
+    j = np.einsum("ka,kzyx->azyx", c, p)
+    e = np.einsum("k,kzyx->zyx", (c ** 2).sum(1), p)
+    tol = 125 * 2.0**-53 * size / np.abs(m)
+    assert np.all((np.abs(rho - m) <= tol * np.abs(m))[ok])
+    for a, b in zip((ux, uy, uz), j):
+        assert np.all((np.abs(a - b / m) <= 2 * 3 * tol * size / np.abs(m))[ok])
+    t = (e / m - ((j / m) ** 2).sum(0)) / 3
+    assert np.all((np.abs(th - t) <= 2 * 27 * tol * (size / m) ** 2)[ok])
+    assert not np.isfinite(rho[~ok]).any()
