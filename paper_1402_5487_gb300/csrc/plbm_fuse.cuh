@@ -314,7 +314,8 @@ FusePlan fuse_plan(const LatticeParams& P) {
     return least < (sizeof(S) == 2 ? 0.99 : 0.95) * 2 * single_us ? best : FusePlan{0, 0};
 }
 
-// Shared memory for the resident CTAs (1 KB each besides what they ask for), the rest as cache.
+// Shared memory for the resident CTAs (1 KB each besides what they ask for), the rest as cache.  Every
+// caller gives a kernel the same values, so that threads that launch it at once do not disturb each other.
 inline cudaError_t fuse_shared_memory(const void* kernel, size_t smem, int resident) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -322,13 +323,15 @@ inline cudaError_t fuse_shared_memory(const void* kernel, size_t smem, int resid
                                 (int)((resident * (smem + 1024) * 100 + (228 << 10) - 1) / (228 << 10)));
 }
 
-template <typename S, class E, int NT, int MINB>
+// WMAX: the largest w this kernel is launched for.
+template <typename S, class E, int NT, int MINB, int WMAX>
 cudaError_t launch_two_steps_t(const LatticeParams& L, const void* src, void* dst, cudaStream_t stream) {
     const FusePlan plan = fuse_plan<S>(L);
     const FuseShape shape = fuse_shape<S>(L);
-    if (plan.strips == 0 || shape.threads != NT) return cudaErrorInvalidValue;
+    constexpr size_t kMost = 25 * (size_t)(WMAX + 1) * NT * sizeof(E);
+    if (plan.strips == 0 || shape.threads != NT || shape.smem > kMost) return cudaErrorInvalidValue;
     const auto kernel = k_two_steps<E, NT, MINB>;
-    const cudaError_t e = fuse_shared_memory(reinterpret_cast<const void*>(kernel), shape.smem, shape.resident);
+    const cudaError_t e = fuse_shared_memory(reinterpret_cast<const void*>(kernel), kMost, MINB);
     if (e != cudaSuccess) return e;
     return launch_dependent_smem(true, shape.smem, kernel, dim3(plan.strips, plan.segments), NT, stream, pair_params(L),
                                  static_cast<const E*>(src), static_cast<E*>(dst));
@@ -338,11 +341,13 @@ template <typename S>
 cudaError_t launch_two_steps(const LatticeParams& P, const void* src, void* dst, cudaStream_t stream) {
     using V = typename PairStore<S>::V;
     if constexpr (sizeof(S) == 2)
-        return P.paired ? launch_two_steps_t<S, V, 128, 3>(P, src, dst, stream) : launch_two_steps_t<S, S, 128, 5>(P, src, dst, stream);
+        return P.paired ? launch_two_steps_t<S, V, 128, 3, kFuseMaxV>(P, src, dst, stream)
+                        : launch_two_steps_t<S, S, 128, 5, kFuseMaxV>(P, src, dst, stream);
     else if (fuse_w(P) > 2)
-        return P.paired ? launch_two_steps_t<S, V, 96, 2>(P, src, dst, stream) : launch_two_steps_t<S, S, 128, 3>(P, src, dst, stream);
+        return P.paired ? launch_two_steps_t<S, V, 96, 2, kFuseMaxV>(P, src, dst, stream)
+                        : launch_two_steps_t<S, S, 128, 3, kFuseMaxV>(P, src, dst, stream);
     else
-        return P.paired ? launch_two_steps_t<S, V, 64, 4>(P, src, dst, stream) : launch_two_steps_t<S, S, 128, 4>(P, src, dst, stream);
+        return P.paired ? launch_two_steps_t<S, V, 64, 4, 2>(P, src, dst, stream) : launch_two_steps_t<S, S, 128, 4, 2>(P, src, dst, stream);
 }
 
 constexpr size_t kBatchFuseSmem = 25 * (size_t)(kFuseMaxV + 1) * kBatchFuseThreads * sizeof(float2);

@@ -925,6 +925,44 @@ def test_two_steps_of_one_launch_equal_single_steps(prec, v, shape, plain):
         assert pop is None or np.array_equal(ref[1], pop)
 
 
+# Two lattices whose rings differ in size (w = 2 and 3), stepped by two threads on streams of their own.
+@pytest.mark.parametrize("prec", ["f32", "f16dev"])
+def test_two_steps_of_one_launch_from_two_threads(prec):
+    import threading
+    import torch
+    from paper_1402_5487_gb300 import plbm
+    L = 2048
+    one = torch.ones(L, L, dtype=torch.float64, device="cuda")
+    x = torch.arange(L, dtype=torch.float64, device="cuda")
+    u = 0.01 * torch.sin(2 * math.pi * x / L)[None, :] * one
+
+    def make(v):
+        s = plbm.Solver(2, v, 1.1, L, L, theta0=0.7 if max(v) == 2 else 1.0, prec=prec, stream=torch.cuda.Stream())
+        torch.cuda.synchronize()
+        s.init(one, u, -u, (0.7 if max(v) == 2 else 1.0) * one)
+        return s
+
+    got = []
+    for threads in (False, True):
+        sols = [make(v) for v in (I.SET_012, I.SET_013)]
+        work = [threading.Thread(target=lambda s=s: [s.step(4) for _ in range(30)]) for s in sols]
+        for w in work:
+            w.start()
+            if not threads:
+                w.join()
+        for w in work:
+            w.join()
+        torch.cuda.synchronize()
+        assert all(s.check() == plbm.PLBM_OK for s in sols)
+        out = [s.moments(on_device=True) for s in sols]
+        torch.cuda.synchronize()
+        got.append(out)
+        for s in sols:
+            s.close()
+    for a, b in zip(*got):
+        assert all(torch.equal(p, q) for p, q in zip(a, b))
+
+
 # FP64 steps of five-velocity sets: the symmetric ones in either order of a and b,
 # thermal and isothermal, with fixed ends, on one row, at another density scale, and a
 # set in an order the symmetric core does not take; 60 steps within 1e-12 of the oracle.
