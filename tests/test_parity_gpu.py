@@ -881,7 +881,8 @@ def test_final_pass_of_the_reductions(prec, shape):
     ((0, 3, -3, 1, -1), (960, 1026), False), ((0, 2, -2, 1, -1), (1031, 957), False), ((0, 2, -2, 3, -3), (1500, 800), False),
     (I.SET_013, (40000, 100), False), (I.SET_013, (90, 40000), False), (I.SET_013, (40000, 101), False),
     (I.SET_012, (400000, 8), False), (I.SET_013, (700, 1000), False), ((0, 1, -1, 4, -4), (1024, 1024), False)]] + [
-    ("f16dev", I.SET_013, (2051, 2050), False), ("f16dev", I.SET_012, (1900, 1726), False),
+    ("f16dev", I.SET_013, (2051, 2050), False), ("f16dev", (0, 3, -3, 1, -1), (2051, 2050), False), ("f16dev", (0, 2, -2, 3, -3), (2050, 2052), False),
+    ("f16dev", I.SET_012, (1900, 1726), False),
     ("bf16dev", I.SET_013, (2301, 2204), False), ("bf16dev", (0, 3, -3, 1, -1), (1150, 4412), False),
     ("f16dev", I.SET_013, (2500, 2501), False), ("bf16dev", (0, 2, -2, 1, -1), (2611, 2444), True), ("f16dev", I.SET_013, (1500, 900), False)])
 def test_two_steps_of_one_launch_equal_single_steps(prec, v, shape, plain):
