@@ -517,11 +517,9 @@ __device__ __forceinline__ FFV<V> ffv_minus(FFV<V> a, FFV<V> b) { return ffv_acc
 // 2048^2 FP32 205 -> 128 us, FP16 200 -> 125 us, 2047^2 FP32 202 -> 124 us: 15 FP64
 // instructions a node (31 with the division and conversions) take 104, the bytes 82 and 51.
 template <typename S, class V>
-__global__ void __launch_bounds__(128) k_moments_sym5(const __grid_constant__ LatticeParams P, const S* __restrict__ f,
-                                                      double* rho, double* ux, double* uy, double* theta, int y0) {
+__device__ __forceinline__ void moments_sym5(const LatticeParams& P, const S* __restrict__ f, double* rho, double* ux, double* uy,
+                                             double* theta, int x, int y) {
     constexpr int kLanes = sizeof(V) / sizeof(float);
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = y0 + blockIdx.y;
-    if (x >= P.nx) return;
     const FFV<V> zero{splat<V>(0.0f), splat<V>(0.0f)};
     const S* at = f + elem_index(P, 0, x, y);   // V = float2: y < half_ny, the pair's first node
     FFV<V> Sx[5], Ty[5];
@@ -548,6 +546,61 @@ __global__ void __launch_bounds__(128) k_moments_sym5(const __grid_constant__ La
     for (int l = 0; l < kLanes; ++l)
         put_fields(fields_from_sums<2>(P, lane_of(dm, l), lane_of(jx, l), lane_of(jy, l), lane_of(de, l)),
                    ((long long)y + l * P.half_ny) * P.nx + x, rho, ux, uy, theta);
+}
+
+template <typename S, class V>
+__global__ void __launch_bounds__(128) k_moments_sym5(const __grid_constant__ LatticeParams P, const S* __restrict__ f,
+                                                      double* rho, double* ux, double* uy, double* theta, int y0) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x < P.nx) moments_sym5<S, V>(P, f, rho, ux, uy, theta, x, y0 + blockIdx.y);
+}
+
+// FP16 pairs: every value is a multiple of 2^-24, so that below 1/4 (every healthy deviation) the sums are
+// exact 32-bit integers (the bits of g + 3/4 are 2^24 g and a constant), rho needs no FP64 instruction and
+// a node 10 instead of 15: 2048^2 125 -> 85 us.  A thread that meets a larger value, an infinity or a NaN
+// starts over in float-float.
+__global__ void __launch_bounds__(128) k_moments_f16pair(const __grid_constant__ LatticeParams P, const __half* __restrict__ f,
+                                                         double* rho, double* ux, double* uy, double* theta) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+    if (x >= P.nx) return;
+    const __half2* at = reinterpret_cast<const __half2*>(f + elem_index(P, 0, x, y));
+    int2 S[5], T[5];
+    __half2 most = __float2half2_rn(0.0f);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) S[i] = T[i] = make_int2(0, 0);
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const __half2 h = __ldg(at + (5 * i + j) * (P.plane / 2));
+            most = __hmax2_nan(most, __habs2(h));
+            const float2 g = add2(__half22float2(h), f2s(0.75f));
+            S[i].x += __float_as_int(g.x);
+            S[i].y += __float_as_int(g.y);
+            T[j].x += __float_as_int(g.x);
+            T[j].y += __float_as_int(g.y);
+        }
+    const float2 top = __half22float2(most);
+    if (!(top.x < 0.25f && top.y < 0.25f)) {
+        moments_sym5<__half, float2>(P, f, rho, ux, uy, theta, x, y);
+        return;
+    }
+    const unsigned off = 5u * 0x3f400000u;   // five times the bits of 3/4
+    const long long a = P.v[1], b = P.v[3];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        auto sum = [&](const int2& v) { return (long long)(int)((unsigned)(l ? v.y : v.x) - off); };
+        const long long sp = sum(S[1]) + sum(S[2]), sq = sum(S[3]) + sum(S[4]);
+        const long long tp = sum(T[1]) + sum(T[2]), tq = sum(T[3]) + sum(T[4]);
+        auto value = [](long long i) { return f64_of_fixed(i, 1056, false); };   // units of 2^-24
+        NodeFields o;
+        o.rho = value((1ll << 24) + sum(S[0]) + sp + sq);
+        const double ir = recip_f64(o.rho);
+        o.ux = value(a * (sum(S[1]) - sum(S[2])) + b * (sum(S[3]) - sum(S[4]))) * ir;
+        o.uy = value(a * (sum(T[1]) - sum(T[2])) + b * (sum(T[3]) - sum(T[4]))) * ir;
+        o.theta = ((2.0 * P.theta0 + value(a * a * (sp + tp) + b * b * (sq + tq))) * ir - (o.ux * o.ux + o.uy * o.uy)) * 0.5;
+        put_fields(o, ((long long)y + l * P.half_ny) * P.nx + x, rho, ux, uy, theta);
+    }
 }
 
 template <typename S>
@@ -883,6 +936,10 @@ cudaError_t launch_moments(int prec, const LatticeParams& P, const void* f, doub
     if (prec != kF64 && P.sym5 && P.dim == 2) {
         if (P.paired && y0 == 0 && y1 == P.ny) {
             grid.y = P.half_ny;
+            if (prec == kF16Dev) {
+                k_moments_f16pair<<<grid, 128, 0, stream>>>(P, static_cast<const __half*>(f), rho, ux, uy, theta);
+                return cudaGetLastError();
+            }
             PLBM_DISPATCH_DEV(prec, (k_moments_sym5<S, float2><<<grid, 128, 0, stream>>>(
                                         P, static_cast<const S*>(f), rho, ux, uy, theta, 0)));
         } else {

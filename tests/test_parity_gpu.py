@@ -835,6 +835,40 @@ def test_f64_rule_in_and_out_of_the_fixed_point_range(dim, iso, v):
     s.close()
 
 
+# Fields of FP16 pairs from exact 32-bit sums below 1/4 and in float-float from there on: as the 3D test of
+# the same; 25 roundings of 2^-53 of the sum of magnitudes.
+@pytest.mark.parametrize("v", [I.SET_013, I.SET_012])
+@pytest.mark.parametrize("extra", [None, 0.25, -0.25, 0.2498779296875, -0.2498779296875, 2.0**-24, 7.5, -300.0, np.inf, np.nan])
+def test_fp16_fields_from_exact_sums(extra, v):
+    nx, ny = 133, 8
+    rng = np.random.default_rng(19)
+    s = plbm.Solver(2, v, 1.1, nx, ny, theta0=0.7 if max(v) == 2 else 1.0, prec="f16dev")
+    one = np.ones((ny, nx))
+    s.init(one, 0 * one, 0 * one, (0.7 if max(v) == 2 else 1.0) * one)
+    f = s.get_populations()
+    g = (0.05 * rng.uniform(-1, 1, f.shape) * 10.0 ** rng.uniform(-5, 0, f.shape)).astype(np.float16).astype(np.float64)
+    if extra is not None:
+        g[7, 1, 5] = g[20, 6, 132] = extra
+    s.set_populations(f + g)
+    p = s.get_populations()
+    rho, ux, uy, th = s.moments()
+    s.close()
+    c = np.array([(v[k // 5], v[k % 5]) for k in range(25)], float)
+    ok = np.isfinite(p).all(axis=0)
+    assert ok.sum() == ok.size - (2 if extra is not None and not np.isfinite(extra) else 0)
+    p = np.where(ok, p, 1.0)
+    m, size = p.sum(0), np.abs(p).sum(0)
+    j = np.einsum("ka,kyx->ayx", c, p)
+    e = np.einsum("k,kyx->yx", (c ** 2).sum(1), p)
+    tol = 25 * 2.0**-53 * size / np.abs(m)
+    assert np.all((np.abs(rho - m) <= tol * np.abs(m))[ok])
+    for a, b in zip((ux, uy), j):
+        assert np.all((np.abs(a - b / m) <= 2 * 3 * tol * size / np.abs(m))[ok])
+    t = (e / m - ((j / m) ** 2).sum(0)) / 2
+    assert np.all((np.abs(th - t) <= 2 * 18 * tol * (size / m) ** 2)[ok])
+    assert not np.isfinite(rho[~ok]).any()
+
+
 # The final pass of the reductions (a cluster of blocks over one record per block of a step):
 # fewer records than blocks, one per thread, one more, several per thread.  The sums of the
 # populations themselves within 1e-13 of the sum of magnitudes, minima those of the fields.
