@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(kBlockX) k_reduce_state_dev(const __grid_const
 constexpr int kFinalBlocks = 8, kFinalThreads = 256;
 __device__ __forceinline__ long long min_key(double v) { return v == v ? dkey(v) : 0x7fffffffffffffffLL; }
 __global__ void __cluster_dims__(kFinalBlocks, 1, 1) __launch_bounds__(kFinalThreads)
-k_finalize(const double* __restrict__ partials, int nblocks, const unsigned* __restrict__ status, double* __restrict__ out) {
+k_finalize(const double* partials, int nblocks, const unsigned* status, double* __restrict__ out) {
     __shared__ double sum[4][kFinalThreads];
     __shared__ long long key[2][kFinalThreads];
     const int t = threadIdx.x;
@@ -793,7 +793,7 @@ k_finalize(const double* __restrict__ partials, int nblocks, const unsigned* __r
 #pragma unroll 4
     for (int b = blockIdx.x * kFinalThreads + t; b < nblocks; b += kFinalBlocks * kFinalThreads) {
         const double2* q = reinterpret_cast<const double2*>(partials + (long long)b * kPartialStride);
-        const double2 a = __ldcg(q), c = __ldcg(q + 1), d = __ldcg(q + 2);
+        const double2 a = load_state(q), c = load_state(q + 1), d = load_state(q + 2);
         r[0] += a.x;
         r[1] += a.y;
         r[2] += c.x;
@@ -836,7 +836,7 @@ k_finalize(const double* __restrict__ partials, int nblocks, const unsigned* __r
     }
     if (blockIdx.x == 0 && t == 32) {
         unsigned* o = reinterpret_cast<unsigned*>(out + 6);
-        o[0] = *reinterpret_cast<const volatile unsigned*>(status);
+        o[0] = load_state(status);
         o[1] = 0u;
     }
     // no block's shared memory goes before the first one has read it

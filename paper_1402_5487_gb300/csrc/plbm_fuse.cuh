@@ -67,7 +67,7 @@ struct FusePair {
     using E = typename PairStore<S>::V;
     using V = float2;
     static constexpr bool kPaired = true;
-    static __device__ __forceinline__ E load(const E* p) { return __ldg(p); }
+    static __device__ __forceinline__ E load(const E* p) { return load_state(p); }
     static __device__ __forceinline__ V cvt(E v) { return PairStore<S>::cvt(v); }
     static __device__ __forceinline__ V cvt_again(E v) { return PairStore<S>::cvt_again(v); }
     static __device__ __forceinline__ E pack(V v) {
@@ -87,7 +87,7 @@ template <typename S>
 struct FuseNode {
     using V = float;
     static constexpr bool kPaired = false;
-    static __device__ __forceinline__ S load(const S* p) { return __ldg(p); }
+    static __device__ __forceinline__ S load(const S* p) { return load_state(p); }
     static __device__ __forceinline__ V cvt_again(S v) { return cvt(v); }
     static __device__ __forceinline__ V cvt(S v) {
         if constexpr (std::is_same<S, __half>::value) return __half2float(v);
@@ -113,7 +113,7 @@ struct FuseElem<__nv_bfloat16> : FuseNode<__nv_bfloat16> {};
 // (V = E) or, in the plain layout, columns t and t + NT (E = float, V = float2).
 // rows >= 2w and nx >= 2w: no index wraps twice.  begin() is called before the first load.
 template <class E, class V, int NT, class Begin>
-__device__ __forceinline__ void two_steps(const PairParams& P, const E* __restrict__ src, E* __restrict__ dst, E* ring, int x0,
+__device__ __forceinline__ void two_steps(const PairParams& P, const E* src, E* __restrict__ dst, E* ring, int x0,
                                           int wn, int r0, int r1, Begin begin) {
     using X = FuseElem<E>;
     constexpr bool kPaired = X::kPaired, kTwo = sizeof(V) > sizeof(typename X::V);   // kTwo: E = float, V = float2
@@ -167,7 +167,7 @@ __device__ __forceinline__ void two_steps(const PairParams& P, const E* __restri
             for (int j = 0; j < 5; ++j) {
                 const E* q = src + (5 * i + j) * P.plane2;
                 if constexpr (kTwo)
-                    g[5 * i + j] = f2(__ldg(q + (row[j] + col[i])), __ldg(q + (row[j] + col1[i])));
+                    g[5 * i + j] = f2(X::load(q + (row[j] + col[i])), X::load(q + (row[j] + col1[i])));
                 else
                     g[5 * i + j] = X::load(q + (row[j] + col[i]));
             }
@@ -247,7 +247,7 @@ __device__ __forceinline__ void two_steps(const PairParams& P, const E* __restri
 // (pair) rows [rows s / segments, rows (s + 1) / segments).
 template <class E, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
-k_two_steps(const __grid_constant__ PairParams P, const E* __restrict__ src, E* __restrict__ dst) {
+k_two_steps(const __grid_constant__ PairParams P, const E* src, E* __restrict__ dst) {
     extern __shared__ __align__(16) unsigned char fuse_ring[];
     step_begin();
     const int rows = FuseElem<E>::kPaired ? P.half_ny : P.ny;
@@ -272,12 +272,13 @@ k_batch_two_steps(const PairParams* __restrict__ inst, const FusePiece* __restri
     for (int k = threadIdx.x; k < (int)(sizeof(PairParams) / sizeof(int)); k += NT)
         reinterpret_cast<int*>(&sp)[k] = reinterpret_cast<const int*>(&inst[p.inst])[k];
     __syncthreads();
+    const PairParams lp = sp;   // in registers: no store of the loop can change it (142.7 -> 139.5 us a step for 6.0 M nodes)
     if (sp.paired)
-        two_steps<float2, float2, NT>(sp, static_cast<const float2*>(sp.f[parity]), static_cast<float2*>(sp.f[parity ^ 1]),
+        two_steps<float2, float2, NT>(lp, static_cast<const float2*>(sp.f[parity]), static_cast<float2*>(sp.f[parity ^ 1]),
                                                      reinterpret_cast<float2*>(fuse_ring), p.x0, p.wn, p.r0, p.r1,
                                                      [] { step_wait(); });
     else
-        two_steps<float, float2, NT>(sp, static_cast<const float*>(sp.f[parity]), static_cast<float*>(sp.f[parity ^ 1]),
+        two_steps<float, float2, NT>(lp, static_cast<const float*>(sp.f[parity]), static_cast<float*>(sp.f[parity ^ 1]),
                                                     reinterpret_cast<float*>(fuse_ring), p.x0, p.wn, p.r0, p.r1,
                                                     [] { step_wait(); });
 }

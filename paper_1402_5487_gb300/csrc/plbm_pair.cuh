@@ -87,7 +87,7 @@ struct PairStore<float> {
     using V = float2;
     static constexpr bool kReconvert = false;
     static __device__ __forceinline__ void store(V* p, float2 v) { *p = v; }
-    static __device__ __forceinline__ V raw(const V* p) { return __ldg(p); }
+    static __device__ __forceinline__ V raw(const V* p) { return load_state(p); }
     static __device__ __forceinline__ V swap(V v) { return f2(v.y, v.x); }
     static __device__ __forceinline__ float2 cvt(V v) { return v; }
     static __device__ __forceinline__ float2 cvt_again(V v) { return v; }
@@ -105,7 +105,7 @@ struct PairStore<__half> {
     using V = __half2;
     static constexpr bool kReconvert = false;
     static __device__ __forceinline__ void store(V* p, float2 v) { *p = __float22half2_rn(v); }
-    static __device__ __forceinline__ V raw(const V* p) { return __ldg(p); }
+    static __device__ __forceinline__ V raw(const V* p) { return load_state(p); }
     static __device__ __forceinline__ V swap(V v) { return __lowhigh2highlow(v); }
     static __device__ __forceinline__ float2 cvt(V v) { return __half22float2(v); }
     static __device__ __forceinline__ float2 cvt_again(V v) { return cvt(v); }
@@ -116,7 +116,7 @@ struct PairStore<__nv_bfloat16> {
     using V = __nv_bfloat162;
     static constexpr bool kReconvert = true;
     static __device__ __forceinline__ void store(V* p, float2 v) { *p = __float22bfloat162_rn(v); }
-    static __device__ __forceinline__ V raw(const V* p) { return __ldg(p); }
+    static __device__ __forceinline__ V raw(const V* p) { return load_state(p); }
     static __device__ __forceinline__ V swap(V v) { return __lowhigh2highlow(v); }
     static __device__ __forceinline__ float2 cvt(V v) { return __bfloat1622float2(v); }
     static __device__ __forceinline__ float2 cvt_again(V v) {
@@ -243,7 +243,7 @@ __device__ __forceinline__ void flag_unhealthy(const PairParams& P, float rho, f
 // The 25 pulls of a node pair (lane order fixed up across the y wrap), each
 // passed through conv on its way into dst.
 template <typename PS, typename T, class Conv>
-__device__ __forceinline__ void pull25(const typename PS::V* __restrict__ src, long long plane2,
+__device__ __forceinline__ void pull25(const typename PS::V* src, long long plane2,
                                        const unsigned (&row)[5], const unsigned (&col)[5], const bool (&swp)[5],
                                        bool any_swap, T (&dst)[25], Conv conv) {
     if (!any_swap) {
@@ -324,7 +324,7 @@ __device__ __forceinline__ unsigned pair_pull_index(const PairParams& P, int x, 
 
 // One thread's work: nodes (x, r) and (x, r + ny/2) of one lattice, x < nx.
 template <typename S, bool REDUCE>
-__device__ __forceinline__ void pair_node(const PairParams& P, const typename PairStore<S>::V* __restrict__ src,
+__device__ __forceinline__ void pair_node(const PairParams& P, const typename PairStore<S>::V* src,
                                           typename PairStore<S>::V* __restrict__ dst, int x, int r,
                                           NodeDiagF& d) {
     using PS = PairStore<S>;
@@ -356,7 +356,7 @@ constexpr int kPair2Block = 64;
 
 template <typename S>
 __global__ void __launch_bounds__(kPair2Block)
-k_stream_collide_pair2(const __grid_constant__ PairParams P, const typename PairStore<S>::V* __restrict__ src,
+k_stream_collide_pair2(const __grid_constant__ PairParams P, const typename PairStore<S>::V* src,
                        typename PairStore<S>::V* __restrict__ dst, int tiles_x, int ntiles) {
     using PS = PairStore<S>;
     using V = typename PS::V;
@@ -409,23 +409,23 @@ template <typename S>
 struct Scalar16;
 template <>
 struct Scalar16<float> {
-    static __device__ __forceinline__ float load(const float* p) { return __ldg(p); }
+    static __device__ __forceinline__ float load(const float* p) { return load_state(p); }
     static __device__ __forceinline__ void store(float* p, float v) { *p = v; }
 };
 template <>
 struct Scalar16<__half> {
-    static __device__ __forceinline__ float load(const __half* p) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ float load(const __half* p) { return __half2float(load_state(p)); }
     static __device__ __forceinline__ void store(__half* p, float v) { *p = __float2half_rn(v); }
 };
 template <>
 struct Scalar16<__nv_bfloat16> {
-    static __device__ __forceinline__ float load(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+    static __device__ __forceinline__ float load(const __nv_bfloat16* p) { return __bfloat162float(load_state(p)); }
     static __device__ __forceinline__ void store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
 template <typename S, bool REDUCE>
-__device__ __forceinline__ void sym5_node(const PairParams& P, const S* __restrict__ src, S* __restrict__ dst,
-                                          int x, int y, NodeDiagF& d) {
+__device__ __forceinline__ void sym5_node(const PairParams& P, const S* src, S* __restrict__ dst, int x, int y,
+                                          NodeDiagF& d) {
     unsigned col[5], row[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
@@ -464,7 +464,7 @@ __device__ __forceinline__ void sym5_node(const PairParams& P, const S* __restri
 // grid = (ceil(nx / blockDim.x), ny), one node per thread (blockDim.x = kBlockX when REDUCE).
 template <typename S, bool REDUCE, bool LATE = false>
 __global__ void __launch_bounds__(kBlockX)
-k_stream_collide_sym5(const __grid_constant__ PairParams P, const S* __restrict__ src, S* __restrict__ dst) {
+k_stream_collide_sym5(const __grid_constant__ PairParams P, const S* src, S* __restrict__ dst) {
     if (!LATE) step_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     NodeDiagF d;
@@ -490,8 +490,7 @@ struct PairMinBlocks {
 // grid = (ceil(nx / blockDim.x), ny / 2), blockDim.x = kBlockX when REDUCE; thread (x, r) owns nodes (x, r) and (x, r + ny/2).
 template <typename S, bool REDUCE, bool LATE = false>
 __global__ void __launch_bounds__(kBlockX, REDUCE ? 0 : PairMinBlocks<S>::value)
-k_stream_collide_pair(const __grid_constant__ PairParams P,
-                      const typename PairStore<S>::V* __restrict__ src,
+k_stream_collide_pair(const __grid_constant__ PairParams P, const typename PairStore<S>::V* src,
                       typename PairStore<S>::V* __restrict__ dst) {
     if (!LATE) step_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;

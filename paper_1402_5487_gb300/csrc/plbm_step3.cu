@@ -87,8 +87,8 @@ __device__ __forceinline__ void axis_dev(const LatticeParams& P, float u, float 
 }
 
 template <typename S>
-__global__ void __launch_bounds__(kB3, 2) k_stream_collide3(const __grid_constant__ LatticeParams P,
-                                                           const S* __restrict__ src, S* __restrict__ dst) {
+__global__ void __launch_bounds__(kB3, 2) k_stream_collide3(const __grid_constant__ LatticeParams P, const S* src,
+                                                           S* __restrict__ dst) {
     step_begin();
     const int x = blockIdx.x * kB3 + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -186,8 +186,7 @@ constexpr int kSplitThreads = kSplitNodes * kQ1;   // 160
 
 template <typename S>
 __global__ void __launch_bounds__(kSplitThreads) k_stream_collide3_split(const __grid_constant__ LatticeParams P,
-                                                                         const S* __restrict__ src,
-                                                                         S* __restrict__ dst) {
+                                                                         const S* src, S* __restrict__ dst) {
     __shared__ float sS[kQ1][kSplitNodes];
     __shared__ float sT[kQ1][kQ1][kSplitNodes];   // [warp a][b][node]
     __shared__ float sU[kQ1][kQ1][kSplitNodes];   // [warp a][c][node]
@@ -371,8 +370,8 @@ __device__ __forceinline__ void axis_dev2(const LatticeParams& P, float2 u, floa
 // pair rows away from the wrap (all but 2 max|v| of them) take the WRAP = false
 // copy without the per-load lane test.
 template <typename S, bool WRAP>
-__device__ __forceinline__ void zpair_update(const LatticeParams& P, const unsigned* __restrict__ s32,
-                                             unsigned* __restrict__ d32, int x, int y, int r) {
+__device__ __forceinline__ void zpair_update(const LatticeParams& P, const unsigned* s32, unsigned* __restrict__ d32, int x,
+                                             int y, int r) {
     const int H = P.half_nz;
     int xs[kQ1], ys[kQ1], zr[kQ1];
     bool sw[kQ1];
@@ -395,7 +394,7 @@ __device__ __forceinline__ void zpair_update(const LatticeParams& P, const unsig
 #pragma unroll
             for (int a = 0; a < kQ1; ++a) {
                 const int p = (a * kQ1 + b) * kQ1 + c;
-                const unsigned v = __ldg(s32 + (p * plane + row + xs[a]));
+                const unsigned v = load_state(s32 + (p * plane + row + xs[a]));
                 g[p] = (WRAP && sw[c]) ? __byte_perm(v, 0u, 0x1032) : v;
             }
         }
@@ -471,8 +470,7 @@ constexpr int kZpairBlock = 64;
 
 template <typename S>
 __global__ void __launch_bounds__(kZpairBlock) k_stream_collide3_zpair(const __grid_constant__ LatticeParams P,
-                                                                      const S* __restrict__ src,
-                                                                      S* __restrict__ dst) {
+                                                                      const S* src, S* __restrict__ dst) {
     step_begin();
     const int x = blockIdx.x * kZpairBlock + threadIdx.x;
     const int y = blockIdx.y, r = blockIdx.z;   // pair row r: nodes z = r and z = r + nz/2
@@ -526,12 +524,6 @@ __device__ __forceinline__ double w0_3(const LatticeParams& P, int p) {
 // R_ab = sum_c f, S_a, T_b, U_c; the second loads them again (L1/L2 hits) and
 // writes f' = (1 - omega) f + (omega rho r^x_a r^y_b) r^z_c (moments and the
 // C mu rule of Eq. eq:rdr, with the sums factorised).
-__device__ __forceinline__ double ldg_again(const double* p) {
-    double v;
-    asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
-    return v;
-}
-
 template <int Q1>
 __device__ __forceinline__ void rule_q(const LatticeParams& P, double u, double th, double (&r)[Q1]) {
     double mu[Q1];
@@ -550,8 +542,7 @@ __device__ __forceinline__ void rule_q(const LatticeParams& P, double u, double 
 
 template <int Q1>
 __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_constant__ LatticeParams P,
-                                                              const double* __restrict__ src,
-                                                              double* __restrict__ dst) {
+                                                              const double* src, double* __restrict__ dst) {
     step_begin();
     const int x = blockIdx.x * kB3 + threadIdx.x;
     const int y = blockIdx.y, z = blockIdx.z;
@@ -576,7 +567,7 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
 #pragma unroll
             for (int c = 0; c < Q1; ++c) {
                 const int p = (a * Q1 + b) * Q1 + c;
-                const double v = __ldg(src + (long long)p * P.plane + (zr[c] + yr[b] + xs[a]));
+                const double v = load_state(src + (long long)p * P.plane + (zr[c] + yr[b] + xs[a]));
                 R += v;
                 Uc[c] += v;
             }
@@ -612,12 +603,12 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
 #pragma unroll
         for (int b = 0; b < Q1; ++b) {
             const double X = om * m0 * ra[a] * rb[b];
+            double f[Q1];   // loaded together: a load does not pass a store that it could alias
 #pragma unroll
-            for (int c = 0; c < Q1; ++c) {
-                const int p = (a * Q1 + b) * Q1 + c;
-                const double f = ldg_again(src + (long long)p * plane2 + (zr[c] + yr[b] + xs[a]));
-                dst[(long long)p * plane2 + here] = fma(keep, f, X * rc[c]);
-            }
+            for (int c = 0; c < Q1; ++c)
+                f[c] = load_state(src + (long long)((a * Q1 + b) * Q1 + c) * plane2 + (zr[c] + yr[b] + xs[a]));
+#pragma unroll
+            for (int c = 0; c < Q1; ++c) dst[(long long)((a * Q1 + b) * Q1 + c) * plane2 + here] = fma(keep, f[c], X * rc[c]);
         }
 }
 
