@@ -198,6 +198,10 @@ plbm_status plbm_init(plbm_handle h, const double *rho, const double *ux, const 
  * steps in one launch; the state is that of single steps. */
 plbm_status plbm_step(plbm_handle h, long n);
 
+/* Step kernels that plbm_step and plbm_step_diagnostics have launched for the handle so far (those of a
+ * graph replay included): fewer than steps where a launch takes several.  PLBM_E_ARG for NULL. */
+plbm_status plbm_step_launches(plbm_handle h, long long *launches);
+
 /* Read the device status word (synchronises the stream).  Returns
  * PLBM_E_DIVERGED if any PLBM_STATUS_* bit has been set. */
 plbm_status plbm_check(plbm_handle h);
@@ -315,6 +319,8 @@ plbm_status plbm_batch_create(const plbm_desc *descs, int n, void *stream, plbm_
  * (row-paired or plain layout), instances in the other groups, and persistent
  * launches per step (one per group). */
 plbm_status plbm_batch_groups(plbm_batch b, int *paired_instances, int *plain_instances, int *launches_per_step);
+/* Step kernels that plbm_batch_step has launched so far (as plbm_step_launches). */
+plbm_status plbm_batch_step_launches(plbm_batch b, long long *launches);
 
 /* Release the batch, its instances and its memory.  Accepts NULL. */
 plbm_status plbm_batch_destroy(plbm_batch b);

@@ -115,6 +115,13 @@ class Batch:
     def step(self, n=1, mode="persistent_graph"):
         self._ok(plbm.lib().plbm_batch_step(self.b, int(n), MODES[mode] if isinstance(mode, str) else int(mode)))
 
+    @property
+    def step_launches(self):
+        """Step kernels that step() has launched so far."""
+        n = ctypes.c_longlong()
+        self._ok(plbm.lib().plbm_batch_step_launches(self.b, ctypes.byref(n)))
+        return n.value
+
     def check(self):
         bad = ctypes.c_int()
         st = plbm.lib().plbm_batch_check(self.b, ctypes.byref(bad))

@@ -40,6 +40,7 @@ struct Handle {
     double* host_buf = nullptr; // pinned: 8 result doubles + status word
     cudaStream_t stream = nullptr;
     long long steps = 0;
+    long long launches = 0;    // step kernels launched (plbm_step_launches)
     plbm_status sticky = PLBM_OK;
     bool initialised = false;
     bool in_batch = false;     // owned by a plbm_batch: not destroyable on its own
@@ -683,6 +684,13 @@ plbm_status plbm_check(plbm_handle hh) {
     return PLBM_OK;
 }
 
+plbm_status plbm_step_launches(plbm_handle hh, long long* launches) {
+    Handle* h = reinterpret_cast<Handle*>(hh);
+    if (!h || !launches) return PLBM_E_ARG;
+    *launches = h->launches;
+    return PLBM_OK;
+}
+
 plbm_status plbm_step(plbm_handle hh, long n) {
     Handle* h = reinterpret_cast<Handle*>(hh);
     plbm_status st = usable(h);
@@ -723,6 +731,7 @@ plbm_status plbm_step(plbm_handle hh, long n) {
             }
             CK(cudaGraphLaunch(g, h->stream));
             h->steps += kGraphSteps;
+            h->launches += kGraphSteps / per;
         }
     }
     while (s < n) {
@@ -737,6 +746,7 @@ plbm_status plbm_step(plbm_handle hh, long n) {
             CK(launch(h->cur, (int)k, h->stream));
             h->cur ^= 1;
             h->steps += k;
+            ++h->launches;
             s += k;
             run -= k;
         }
@@ -827,6 +837,7 @@ plbm_status plbm_step_diagnostics(plbm_handle hh, long n, plbm_diag* out) {
     CK(plbm::launch_step(h->prec, h->P, h->f[h->cur], h->f[h->cur ^ 1], true, h->stream));
     h->cur ^= 1;
     ++h->steps;
+    ++h->launches;
     CK(plbm::launch_finalize(h->P, plbm::step_blocks(h->P), h->result, h->stream));
     CK(cudaMemcpyAsync(h->host_buf, h->result, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
@@ -1192,7 +1203,7 @@ struct Batch {
     int order = PLBM_BATCH_ORDER_INTERLEAVED;
     int block_x = 128, ctas_per_sm = 0, sms = 0;
     cudaGraphExec_t graph[3][2] = {};  // [persistent, per instance, runs of two-step launches][start parity]
-    long long steps = 0;
+    long long steps = 0, launches = 0;   // launches: of step kernels (plbm_batch_step_launches)
     char err[512] = "";
 };
 
@@ -1324,6 +1335,14 @@ plbm_status batch_launch4(Batch* b, int parity, int ctas) {
             BCK(plbm::launch_batch_node(g.prec, g.q1, g.d_params, g.d_span, g.total_tiles, g.ctas, parity ^ (k & 1),
                                         g.d_tile_inst, b->stream));
     return PLBM_OK;
+}
+
+// Step kernels that batch_launch4 (run = 4 where a group has pieces) or `run` calls of batch_launch launch.
+long long batch_launches(const Batch* b, int scheme, int run) {
+    if (scheme != 0) return (long long)b->inst.size() * run;
+    long long n = (long long)b->nodes.size() * run;
+    for (const PairGroup& g : b->pairs) n += run == 4 && !g.pieces.empty() ? 2 : run;
+    return n;
 }
 
 // The pieces of an FP32 group for k_batch_two_steps: strips of at most 96 (node pairs) or 192 columns
@@ -1633,6 +1652,7 @@ plbm_status plbm_batch_step(plbm_batch bb, long n, int mode) {
         for (; done + 4 <= n; done += 4) {
             const plbm_status st = batch_launch4(b, parity, ctas);
             if (st != PLBM_OK) return st;
+            b->launches += batch_launches(b, scheme, 4);
         }
     if (use_graph) {
         while (done + 2 <= n) {
@@ -1652,12 +1672,14 @@ plbm_status plbm_batch_step(plbm_batch bb, long n, int mode) {
                 BCK(ei);
             }
             BCK(cudaGraphLaunch(g, b->stream));
+            b->launches += batch_launches(b, scheme, run);
             done += run;
         }
     }
     for (; done < n; ++done) {
         plbm_status st = batch_launch(b, scheme, parity, ctas);
         if (st != PLBM_OK) return st;
+        b->launches += batch_launches(b, scheme, 1);
         parity ^= 1;
     }
     if (n % 2) parity = parity0 ^ 1; else parity = parity0;
@@ -1666,6 +1688,13 @@ plbm_status plbm_batch_step(plbm_batch bb, long n, int mode) {
         h->steps += n;
     }
     b->steps += n;
+    return PLBM_OK;
+}
+
+plbm_status plbm_batch_step_launches(plbm_batch bb, long long* launches) {
+    Batch* b = reinterpret_cast<Batch*>(bb);
+    if (!b || !launches) return PLBM_E_ARG;
+    *launches = b->launches;
     return PLBM_OK;
 }
 

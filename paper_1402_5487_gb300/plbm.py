@@ -102,12 +102,14 @@ SIGNATURES = {
     "plbm_batch_tune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(ctypes.c_int),
                                        ctypes.POINTER(ctypes.c_int), _D]),
     "plbm_batch_last_error": (ctypes.c_char_p, [ctypes.c_void_p]),
+    "plbm_batch_step_launches": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_longlong)]),
     "plbm_batch_groups": (ctypes.c_int, [ctypes.c_void_p] + [ctypes.POINTER(ctypes.c_int)] * 3),
     "plbm_create": (ctypes.c_int, [ctypes.POINTER(PlbmDesc), ctypes.POINTER(_H)]),
     "plbm_destroy": (ctypes.c_int, [_H]),
     "plbm_init": (ctypes.c_int, [_H, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                  ctypes.c_void_p, ctypes.c_int]),
     "plbm_step": (ctypes.c_int, [_H, ctypes.c_long]),
+    "plbm_step_launches": (ctypes.c_int, [_H, ctypes.POINTER(ctypes.c_longlong)]),
     "plbm_check": (ctypes.c_int, [_H]),
     "plbm_moments": (ctypes.c_int, [_H, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                     ctypes.c_void_p, ctypes.c_int]),
@@ -375,6 +377,13 @@ class Solver:
 
     def step(self, n: int = 1):
         _ok(lib().plbm_step(self.h, int(n)), self.h)
+
+    @property
+    def step_launches(self) -> int:
+        """Step kernels launched so far: fewer than steps where a launch takes several."""
+        n = ctypes.c_longlong()
+        _ok(lib().plbm_step_launches(self.h, ctypes.byref(n)), self.h)
+        return n.value
 
     def step_status(self, n: int = 1) -> int:
         """Like step() but returns the status code instead of raising."""

@@ -197,6 +197,50 @@ def test_two_steps_per_launch_of_a_batch_equal_single_steps():
         assert all(np.array_equal(x, y) for x, y in zip(got[0], g))
 
 
+# A group large enough for its pieces to be chosen (the test above stays below that): pieces of every width, both
+# layouts, thin lattices down to the fewest rows (2w), sets with w = 2 and 3 in either order, beside groups
+# that take single steps.  Against one launch per instance and step, bit for bit, and by the number of launches.
+def _beyond_the_cache(more=()):
+    v2, v3 = I.SET_012, I.SET_013
+    mem = [(1100, v3), (1001, v2), (1003, v3), (514, v3), (513, v2), (181, v3), (98, v3), (60, v2), (640, (0, 3, -3, 1, -1)),
+           (187, (0, 2, -2, 1, -1)), (12, v3), (9, v2), (7, v3), (8, v2), (5, v2), (97, v3), (90, v3), (91, v3), *more]
+    inst = [I.Instance(index=k, L=L, v=v, omega=1.1 + 0.01 * k, theta0=0.7 if max(v) == 2 else 1.0, kind="kh", seed=950 + k)
+            for k, (L, v) in enumerate(mem)]
+    n = len(inst)
+    return inst + [I.Instance(index=n, L=72, v=v3, omega=1.3, theta0=1.0, kind="kh", seed=7, prec="f64"),
+                   I.Instance(index=n + 1, L=66, v=v3, omega=1.2, theta0=1.0, kind="kh", seed=8, prec="f16dev")]
+
+
+def _runs_equal_single_launches(inst):
+    fields = [I.instance_fields(x) for x in inst]
+    ref = None
+    # parts of a run (negative: each instance stepped on its own), scheme, step kernels launched for the FP32 group
+    for parts, mode, launches in (((11,), "per_instance", None), ((11,), "persistent", 2 * 2 + 3), ((11,), "persistent_graph", 2 * 2 + 3),
+                                  ((4, 6, 1), "persistent_graph", 2 + (2 + 2) + 1), ((1, 10), "persistent", 1 + (2 * 2 + 2)),
+                                  ((5, -2, 4), "persistent_graph", (2 + 1) + 2)):
+        b = B.Batch(inst, prec="f32")
+        for s, f in zip(b.solvers, fields):
+            s.init(*f)
+        for k in parts:
+            if k > 0:
+                b.step(k, mode)
+            else:
+                for s in b.solvers:
+                    s.step(-k)
+        assert b.check()[0] == plbm.PLBM_OK
+        if launches is not None:   # the other two groups take one launch a step
+            assert b.step_launches == launches + 2 * sum(k for k in parts if k > 0)
+        got = [s.get_populations() for s in b.solvers]
+        b.close()
+        ref = ref or got
+        for x, a, c in zip(inst, ref, got):
+            assert np.array_equal(a, c), (x.L, x.v, parts, mode)
+
+
+def test_batches_beyond_the_cache_take_two_steps_per_launch():
+    _runs_equal_single_launches(_beyond_the_cache())
+
+
 def test_full_sweep_sampled_nodes():
     # The bench's sweep (256 instances drawn by the R8 gates, sides over every
     # integer of [64, 1024], 1.0e8 nodes) in its timed launch scheme: after k steps a

@@ -960,6 +960,53 @@ def test_two_steps_of_one_launch_equal_single_steps(prec, v, shape, plain):
         assert pop is None or np.array_equal(ref[1], pop)
 
 
+# The same where the library says that it launched once per two steps: shapes well inside the rule on any
+# number of SMs, and the flattest ones that it takes (15 and 8 rows of pairs for w = 3 and 2: nearly every
+# row pulls across the wrap; the strips fill the resident CTAs exactly).
+@pytest.mark.parametrize("prec,v,shape,plain", [
+    ("f32", I.SET_013, (2048, 1100), False), ("f32", I.SET_013, (2047, 1101), False), ("f32", I.SET_012, (1700, 1500), True),
+    ("f32", (0, 3, -3, 1, -1), (2048, 1100), False), ("f32", I.SET_013, (90 * 2, 32), False), ("f32", I.SET_012, (60 * 8, 16), False),
+    ("f16dev", I.SET_013, (2700, 2704), False), ("f16dev", I.SET_012, (2701, 2703), False), ("bf16dev", I.SET_013, (3000, 3002), False)])
+def test_lattices_that_take_two_steps_of_one_launch(prec, v, shape, plain):
+    import torch
+    from paper_1402_5487_gb300 import plbm
+    nx, ny = shape
+    if nx < 1000:
+        nx *= torch.cuda.get_device_properties(0).multi_processor_count
+    g = torch.Generator(device="cuda").manual_seed(5)
+    one = torch.ones(ny, nx, dtype=torch.float64, device="cuda")
+    u = [0.02 * (torch.rand(ny, nx, dtype=torch.float64, device="cuda", generator=g) - 0.5) for _ in range(2)]
+    th0 = 0.7 if max(v) == 2 else 1.0
+    out = []
+    for parts, launches in (((1,) * 8, 8), ((8,), 4), ((3, 5), 3 + 3)):   # as many launches as steps, modulo 2
+        s = plbm.Solver(2, v, 1.1, nx, ny, theta0=th0, prec=prec, plain_layout=plain)
+        s.init(one, u[0], u[1], th0 * one)
+        for k in parts:
+            s.step(k)
+        assert s.step_launches == launches, (parts, s.step_launches)
+        out.append([f.clone() for f in s.moments(on_device=True)])
+        s.close()
+    for o in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(out[0], o))
+
+
+def test_step_launches_counts_what_was_launched():
+    from paper_1402_5487_gb300 import plbm
+    one = np.ones((64, 64))
+    s = plbm.Solver(2, I.SET_013, 1.1, 64, 64, prec="f32")
+    s.init(one, 0 * one, 0 * one, one)
+    s.step(70)                # two replays of 32 and six single steps
+    s.step_diagnostics(3)
+    assert s.step_launches == 73
+    s.close()
+    t = plbm.Solver(1, I.SET_013, 1.1, 1000, 1, prec="f32")
+    t.init(np.ones(1000), np.zeros(1000), None, np.ones(1000))
+    t.step(64)
+    assert 0 < t.step_launches < 64
+    t.close()
+    assert plbm.lib().plbm_step_launches(None, None) == plbm.PLBM_E_ARG
+
+
 # Two lattices whose rings differ in size (w = 2 and 3), stepped by two threads on streams of their own.
 @pytest.mark.parametrize("prec", ["f32", "f16dev"])
 def test_two_steps_of_one_launch_from_two_threads(prec):
