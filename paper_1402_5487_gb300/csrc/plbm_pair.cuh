@@ -38,11 +38,28 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, f2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// A sum that stays apart from a product that is one of its terms.  The compiler may fuse the two when they are packed
+// (__fadd2_rn of __fmul2_rn becomes one FMA) and never does so with the single-lane forms below, and the layouts would
+// differ in the last bit wherever the product's factor is no power of two; where a fused one is wanted, it is written out.
+__device__ __forceinline__ unsigned long long bits2(float2 a) {
+    unsigned long long r;
+    memcpy(&r, &a, 8);
+    return r;
+}
+__device__ __forceinline__ float2 add2_apart(float2 a, float2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits2(a)), "l"(bits2(b)));
+    float2 v;
+    memcpy(&v, &r, 8);
+    return v;
+}
 // The same operations on one node (plain layout): each is the single-lane form of
-// the packed one above, correctly rounded and never contracted, so a node gets
-// bit for bit the same result whichever layout and kernel update it.
+// the packed one above, correctly rounded, and sym5_collide leaves the compiler no product to fuse into
+// a sum but exact ones (by 2 and 1/2), so a node gets bit for bit the same result whichever
+// layout and kernel update it.
 __device__ __forceinline__ float add2(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float sub2(float a, float b) { return __fadd_rn(a, -b); }
+__device__ __forceinline__ float add2_apart(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float mul2(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fma2(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 template <class V>
@@ -140,12 +157,12 @@ __device__ __forceinline__ void sym5_axis(const PairParams& P, V u, V th, V dth,
     const V Ob = mul2(fma2(splat<V>(-P.sa2), d1, d3), splat<V>(P.kOb));
     const V Oa = mul2(fma2(splat<V>(-2.0f * P.sb), Ob, d1), splat<V>(P.kOa));
     const V Eb = mul2(fma2(splat<V>(-P.sa2), d2, d4), splat<V>(P.kEb));
-    const V Ea = mul2(fma2(splat<V>(-2.0f * P.sb2), Eb, d2), splat<V>(P.kEa));
-    dr[0] = mul2(splat<V>(-2.0f), add2(Ea, Eb));
-    dr[1] = add2(Ea, Oa);
-    dr[2] = sub2(Ea, Oa);
-    dr[3] = add2(Eb, Ob);
-    dr[4] = sub2(Eb, Ob);
+    const V xa = fma2(splat<V>(-2.0f * P.sb2), Eb, d2), kEa = splat<V>(P.kEa);   // E_a = xa kEa
+    dr[0] = mul2(splat<V>(-2.0f), fma2(xa, kEa, Eb));
+    dr[1] = fma2(xa, kEa, Oa);
+    dr[2] = fma2(xa, kEa, neg2(Oa));
+    dr[3] = add2_apart(Eb, Ob);
+    dr[4] = add2_apart(Eb, neg2(Ob));
 }
 
 // sum(p), col(p): pulled deviation p of the node(s), read for the moment sums

@@ -204,7 +204,8 @@ def _beyond_the_cache(more=()):
     v2, v3 = I.SET_012, I.SET_013
     mem = [(1100, v3), (1001, v2), (1003, v3), (514, v3), (513, v2), (181, v3), (98, v3), (60, v2), (640, (0, 3, -3, 1, -1)),
            (187, (0, 2, -2, 1, -1)), (12, v3), (9, v2), (7, v3), (8, v2), (5, v2), (97, v3), (90, v3), (91, v3), *more]
-    inst = [I.Instance(index=k, L=L, v=v, omega=1.1 + 0.01 * k, theta0=0.7 if max(v) == 2 else 1.0, kind="kh", seed=950 + k)
+    inst = [I.Instance(index=k, L=L, v=v, omega=1.1 + 0.01 * k, theta0=1.6 if {2, 3} <= set(v) else 0.7 if max(v) == 2 else 1.0, kind="kh",
+                       seed=950 + k)
             for k, (L, v) in enumerate(mem)]
     n = len(inst)
     return inst + [I.Instance(index=n, L=72, v=v3, omega=1.3, theta0=1.0, kind="kh", seed=7, prec="f64"),
@@ -239,6 +240,13 @@ def _runs_equal_single_launches(inst):
 
 def test_batches_beyond_the_cache_take_two_steps_per_launch():
     _runs_equal_single_launches(_beyond_the_cache())
+
+
+# Odd sides (plain layout, packed arithmetic over two columns in the fused kernel) with sets whose factors 1/(2a)
+# and 1/(2a^2) are no powers of two.
+def test_batches_of_two_steps_per_launch_with_factors_that_are_no_powers_of_two():
+    _runs_equal_single_launches(_beyond_the_cache([(371, (0, 3, -3, 1, -1)), (229, (0, 3, -3, 2, -2)), (370, (0, 3, -3, 2, -2)),
+                                                   (13, (0, 3, -3, 1, -1))]))
 
 
 def test_full_sweep_sampled_nodes():

@@ -731,6 +731,26 @@ def test_plain_and_row_paired_layouts_give_the_same_state(prec, ny, nx):
             assert abs(out[0][1][k] - o[1][k]) <= 1e-12 * max(1.0, abs(out[0][1][k])), k
 
 
+# Sets whose factors 1/(2a) and 1/(2a^2) are no powers of two: a product fused into a sum would show.
+@pytest.mark.parametrize("prec", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("v", [(0, 3, -3, 1, -1), (0, 3, -3, 2, -2), (0, 5, -5, 1, -1)])
+def test_layouts_give_the_same_state_for_factors_that_are_no_powers_of_two(prec, v):
+    nx, ny = 131, 48
+    fields = I.kh_fields(nx, ny=ny)
+    out = []
+    for plain in (False, True):
+        s = plbm.Solver(2, v, 1.1, nx, ny, theta0=1.0, prec=prec, plain_layout=plain, skip_admissibility=True)
+        s.init(*fields)
+        pops = [s.get_populations()]
+        for _ in range(3):
+            s.step(1)
+            pops.append(s.get_populations())
+        out.append(pops)
+        s.close()
+    for k, (a, b) in enumerate(zip(*out)):
+        assert bool(np.isfinite(a).all()) and bool(np.array_equal(a, b)), (k, np.mean(a != b))
+
+
 # Steps queued back to back (large grids overlap one step's start with the end of the
 # step before; small ones do not) equal steps awaited one by one, bit for bit: every
 # step kernel, on both sides of the size from which its launches overlap.
