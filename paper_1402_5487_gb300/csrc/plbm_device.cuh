@@ -536,10 +536,11 @@ __device__ __forceinline__ bool few_threads() { return (long long)gridDim.x * gr
 // Sums of doubles on the integer pipe.  x = fixed_of(f, E) is f in units of 2^(E - 1080), E the largest
 // biased exponent among the terms: five bits below the last place of the largest, so that a sum of up to
 // 25 of them fits in 63 bits and is exact but for the rounding of each term, 2^-57 of the largest (the
-// last bit of a term that loses bits is set to 1, which errs to either side alike; an FP64 sum rounds
-// each addition to 2^-53 of itself).  f64_of_fixed rounds the sum to nearest even, by the conversion
-// instruction, which takes the FP64 pipe, where there are few warps (few: their latency counts;
-// 128^2 7.2 -> 6.7 us a step) and by integer ones otherwise (1024^2 175 -> 160 us).
+// last bit of a term that may lose bits is set to 1: away from zero where it loses none, to either side
+// alike otherwise, and the same for f and -f; an FP64 sum rounds each addition to 2^-53 of itself).
+// f64_of_fixed rounds the sum to nearest even, by the conversion instruction, which takes the FP64 pipe, where
+// there are few warps (few: their latency counts; 128^2 7.2 -> 6.7 us a step) and by integer ones otherwise
+// (1024^2 175 -> 160 us).
 __device__ __forceinline__ long long fixed_of(double f, int E) {
     const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
     const int e = (int)((hi >> 20) & 0x7ffu), d = min(E - e, 63);
@@ -565,21 +566,26 @@ __device__ __forceinline__ double f64_of_fixed(long long x, int E, bool few) {
 }
 
 // The product of two fixed-point numbers x / 2^m and y / 2^n as one over 2^(m + n - 63): the high
-// word of the product, whose lost bits are replaced by their mean (errs to either side alike).
-__device__ __forceinline__ long long fixed_mul(long long x, long long y) { return (__mul64hi(x, y) << 1) | 1; }
+// word of the product, whose lost bits are replaced by their mean (to either side alike, but for products
+// that have none, zero among them).
+__device__ __forceinline__ long long fixed_mul(long long x, long long y, long long mean = 1) {
+    return (__mul64hi(x, y) << 1) | mean;
+}
+// For x, y >= 0: without the signed product's corrections.
+__device__ __forceinline__ long long fixed_mul_pos(long long x, long long y, long long mean = 1) {
+    return (long long)(__umul64hi((unsigned long long)x, (unsigned long long)y) << 1) | mean;
+}
 // x times a small positive integer: two multiply instructions.
 __device__ __forceinline__ long long fixed_times(long long x, unsigned c) {
     const unsigned long long lo = (unsigned long long)(unsigned)x * c;
     return (long long)(((unsigned long long)((unsigned)(x >> 32) * c) << 32) + lo);
 }
-// x in units of 2^-n for |x| < 2^(63 - n); the last bit of one that loses bits is set to 1, as above.
-__device__ __forceinline__ long long fixed_n(double x, int n) {
+// |x| in units of 2^-n for |x| < 2^(63 - n); the last bit of one that may lose bits is set to 1, as above.
+__device__ __forceinline__ long long fixed_abs(double x, int n) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     const int e = (int)((hi >> 20) & 0x7ffu), d = min(1085 - n - e, 63);
     const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
-    const long long q = (long long)(((m << 10) >> d) | (d > 10 ? 1ull : 0ull));
-    const long long s = (long long)((int)hi >> 31);
-    return (q ^ s) - s;
+    return (long long)(((m << 10) >> d) | (e && d > 10 ? 1ull : 0ull));
 }
 
 // ---------------------------------------------------------------------------
@@ -629,7 +635,8 @@ struct Sym5Core {
     // fits): bits after the point in the names.  Nothing keeps fewer than 57 (an FP64 mu_4 has 50 to 52), and r
     // is 13 to 80 times nearer to the exact value before it is rounded to FP64.  O_a and E_a follow from the
     // rounded O_b and E_b, so that sum r = 1, sum v r = u and sum v^2 r = mu_2 hold without a
-    // systematic error in the last place, which the steps would add up.
+    // systematic error in the last place, which the steps would add up.  The odd parts are those of |u| with
+    // u's sign, and zero for u = 0: a mirrored flow stays the mirrored flow and a fluid at rest exactly at rest.
     struct Theta {
         long long t61, six57;   // theta, 6 theta^2
     };
@@ -639,19 +646,21 @@ struct Sym5Core {
     }
     static __device__ __forceinline__ Theta theta_fixed(double th) {
         Theta t;
-        t.t61 = fixed_n(th, 61);
-        t.six57 = (3 * fixed_mul(t.t61, t.t61)) >> 1;
+        t.t61 = fixed_abs(th, 61);
+        t.six57 = (3 * fixed_mul_pos(t.t61, t.t61)) >> 1;
         return t;
     }
     static __device__ __forceinline__ void axis_fixed(const LatticeParams& P, double ud, Theta th, bool few, double (&r)[5]) {
-        const long long u60 = fixed_n(ud, 60), u62 = u60 << 2;
-        const long long m61 = fixed_mul(u62, u62) + th.t61;          // mu_2
+        const long long u60 = fixed_abs(ud, 60), u62 = u60 << 2, some = u60 ? 1 : 0;   // of |u|
+        const long long m61 = fixed_mul_pos(u62, u62) + th.t61;      // mu_2
         const long long A60 = (m61 >> 1) + th.t61;                   // u^2 + 3 theta
-        const long long yb59 = fixed_mul(u62, A60) - fixed_times(u60 >> 1, P.ia2);
-        const long long zb57 = fixed_mul(A60, A60) - th.six57 - fixed_times(m61 >> 4, P.ia2);
-        const long long Ob = fixed_mul(yb59, P.ikOb65), Eb = fixed_mul(zb57 << 1, P.ikEb65) << 1;   // 61 bits from here
-        const long long w = 2 * (u60 - fixed_times(Ob, P.ib));                   // 2 a O_a, even
-        const long long Oa = P.ia2 == 1 ? w >> 1 : fixed_mul(w, P.ikOa63);
+        const long long yb59 = fixed_mul_pos(u62, A60, some) - fixed_times(u60 >> 1, P.ia2);
+        const long long zb57 = fixed_mul_pos(A60, A60) - th.six57 - fixed_times(m61 >> 4, P.ia2);
+        const long long Ob0 = fixed_mul(yb59, P.ikOb65, some), Eb = fixed_mul(zb57 << 1, P.ikEb65) << 1;   // 61 bits from here
+        const long long w = 2 * (u60 - fixed_times(Ob0, P.ib));   // 2 a O_a
+        const long long Oa0 = P.ia2 == 1 ? w >> 1 : fixed_mul(w, P.ikOa63, w ? 1 : 0);
+        const long long sign = (long long)(__double2hiint(ud) >> 31);
+        const long long Oa = (Oa0 ^ sign) - sign, Ob = (Ob0 ^ sign) - sign;
         const long long Ea = fixed_mul(m61 - fixed_times(Eb, P.ib2x2), P.ikEa63);
         r[0] = f64_of_fixed((1ll << 61) - 2 * (Ea + Eb), 1019, few);
         r[1] = f64_of_fixed(Ea + Oa, 1019, few);

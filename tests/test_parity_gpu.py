@@ -857,6 +857,50 @@ def test_f64_rule_in_and_out_of_the_fixed_point_range(dim, iso, v):
 
 # Fields of FP16 pairs from exact 32-bit sums below 1/4 and in float-float from there on: as the 3D test of
 # the same; 25 roundings of 2^-53 of the sum of magnitudes.
+# The FP64 rule of the symmetric sets in and out of the range of its fixed point: a fluid at rest stays exactly at
+# rest, and the mirrored flow is the flow, mirrored, bit for bit.  Sizes on both sides of the number of threads from
+# which the conversions are made by integer instructions.
+SETS_F64 = [I.SET_013, I.SET_012, (0, 3, -3, 1, -1), (0, 2, -2, 3, -3), (0, 1, -1, 4, -4)]
+
+
+@pytest.mark.parametrize("v", SETS_F64)
+@pytest.mark.parametrize("dim,nx,ny", [(1, 64, 1), (2, 40, 36), (2, 300, 260)])
+def test_f64_rest_is_exact(v, dim, nx, ny):
+    for th in np.random.default_rng(3).uniform(0.3, 1.6, 12 if nx < 100 else 3):
+        s = plbm.Solver(dim, v, 1.1, nx, ny, theta0=float(th), prec="f64", skip_admissibility=True)
+        one = np.ones((ny, nx))
+        s.init(one, 0 * one, 0 * one, th * one)
+        for _ in range(3):
+            _, ux, uy, _ = s.moments()
+            assert not ux.any() and not uy.any(), (th, np.abs(ux).max())
+            s.step(2)
+        s.close()
+
+
+@pytest.mark.parametrize("v", SETS_F64)
+@pytest.mark.parametrize("n,speed", [(48, 0.02), (48, 0.6), (264, 0.02)])
+def test_f64_steps_commute_with_mirrors(v, n, speed):
+    rng = np.random.default_rng(4)
+    rho, th = 1.0 + 0.01 * rng.uniform(-1, 1, (2, n, n))
+    ux, uy = speed * rng.uniform(-1, 1, (2, n, n))
+    ux[3, 5] = uy[7, 2] = 0.0
+
+    def run(f):
+        s = plbm.Solver(2, v, 1.0, n, n, theta0=1.0, prec="f64", skip_admissibility=True)
+        s.init(*[np.ascontiguousarray(a) for a in f])
+        s.step(3)
+        out = s.moments()
+        s.close()
+        return out
+
+    back = -np.arange(n) % n
+    ref = run((rho, ux, uy, th))
+    for index, sign in ((np.ix_(np.arange(n), back), (1, -1, 1, 1)), (np.ix_(back, np.arange(n)), (1, 1, -1, 1))):
+        got = run([g * a[index] for g, a in zip(sign, (rho, ux, uy, th))])
+        for g, a, b in zip(sign, got, ref):
+            assert bool(np.array_equal(a, g * b[index])), np.abs(a - g * b[index]).max()
+
+
 @pytest.mark.parametrize("v", [I.SET_013, I.SET_012])
 @pytest.mark.parametrize("extra", [None, 0.25, -0.25, 0.2498779296875, -0.2498779296875, 2.0**-24, 7.5, -300.0, np.inf, np.nan])
 def test_fp16_fields_from_exact_sums(extra, v):
