@@ -359,10 +359,12 @@ int plbm_batch_get_order(plbm_batch b);
 plbm_status plbm_batch_info(plbm_batch b, int *ninst, int *total_tiles, int *block_x, int *ctas,
                             int *max_ctas_per_sm);
 
-/* Autotuner: times steps_per_trial persistent steps for both orders, every
- * block_x and every ctas_per_sm up to the occupancy limit and keeps the
- * fastest (plbm_batch_get_order reads the order it chose).  It advances the
- * instances (initialise them again afterwards if the state matters). */
+/* Autotuner: times steps_per_trial persistent steps, one per launch, for both
+ * orders, every block_x and every ctas_per_sm up to the occupancy limit and keeps
+ * the fastest (plbm_batch_get_order reads the order it chose).  The shape and order
+ * are those of single steps: a group that takes two steps per launch in runs of four
+ * uses them for the remaining steps only.  It advances the instances (initialise
+ * them again afterwards if the state matters). */
 plbm_status plbm_batch_tune(plbm_batch b, int steps_per_trial, int *best_block_x, int *best_ctas_per_sm,
                             double *best_ms_per_step);
 

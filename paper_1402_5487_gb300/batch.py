@@ -151,7 +151,8 @@ class Batch:
                                                              paired, int(round(n / 1e6)))
 
     def autotune(self, steps_per_trial=6, cache_path=None):
-        """Pick the persistent-kernel shape (cached in JSON by precision, count and size)."""
+        """Pick the shape and order of the persistent single-step kernel (cached in JSON by precision, count and
+        size); ms_per_step is that of single steps."""
         key = self.cache_key()
         cache = {}
         if cache_path and os.path.exists(cache_path):

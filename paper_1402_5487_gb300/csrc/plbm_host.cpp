@@ -1398,6 +1398,75 @@ std::vector<plbm::FusePiece> batch_pieces(const Batch* b, const PairGroup& g) {
     return best;
 }
 
+// two: let groups with pieces take two steps per launch.
+plbm_status batch_step(Batch* b, long n, int mode, bool two) {
+    if (!b || n < 0 || mode < 0 || mode > 3) {
+        batch_err(b, "bad arguments");
+        return PLBM_E_ARG;
+    }
+    const int parity0 = b->inst[0]->cur;
+    for (size_t i = 0; i < b->inst.size(); ++i) {
+        Handle* h = b->inst[i];
+        if (h->sticky != PLBM_OK || !h->initialised) {
+            batch_err(b, "instance %zu is not initialised or in an error state", i);
+            return PLBM_E_STATE;
+        }
+        if (h->cur != parity0) {
+            batch_err(b, "instance %zu was stepped on its own; all instances must be in step", i);
+            return PLBM_E_STATE;
+        }
+    }
+    BCK(cudaSetDevice(b->device));
+    const int scheme = (mode == PLBM_BATCH_PERSISTENT || mode == PLBM_BATCH_PERSISTENT_GRAPH) ? 0 : 1;
+    const bool use_graph = (mode == PLBM_BATCH_PERSISTENT_GRAPH || mode == PLBM_BATCH_PER_INSTANCE_GRAPH);
+    int parity = parity0;
+    long done = 0;
+    const int ctas = batch_ctas(b);  // occupancy query outside any stream capture
+    bool fused = false;              // runs of four steps, two per launch where a group can
+    for (const PairGroup& g : b->pairs) fused |= two && scheme == 0 && !g.pieces.empty();
+    if (fused && !use_graph)
+        for (; done + 4 <= n; done += 4) {
+            const plbm_status st = batch_launch4(b, parity, ctas);
+            if (st != PLBM_OK) return st;
+            b->launches += batch_launches(b, scheme, 4);
+        }
+    if (use_graph) {
+        while (done + 2 <= n) {
+            const int run = fused && done + 4 <= n ? 4 : 2;
+            cudaGraphExec_t& g = b->graph[run == 4 ? 2 : scheme][parity];
+            if (!g) {
+                cudaGraph_t graph = nullptr;
+                BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+                plbm_status st = run == 4 ? batch_launch4(b, parity, ctas) : batch_launch(b, scheme, parity, ctas);
+                if (st == PLBM_OK && run == 2) st = batch_launch(b, scheme, parity ^ 1, ctas);
+                cudaError_t ec = cudaStreamEndCapture(b->stream, &graph);
+                cudaError_t ei = (st == PLBM_OK && ec == cudaSuccess) ? cudaGraphInstantiate(&g, graph, 0)
+                                                                       : cudaSuccess;
+                if (graph) cudaGraphDestroy(graph);
+                if (st != PLBM_OK) return st;
+                BCK(ec);
+                BCK(ei);
+            }
+            BCK(cudaGraphLaunch(g, b->stream));
+            b->launches += batch_launches(b, scheme, run);
+            done += run;
+        }
+    }
+    for (; done < n; ++done) {
+        plbm_status st = batch_launch(b, scheme, parity, ctas);
+        if (st != PLBM_OK) return st;
+        b->launches += batch_launches(b, scheme, 1);
+        parity ^= 1;
+    }
+    if (n % 2) parity = parity0 ^ 1; else parity = parity0;
+    for (Handle* h : b->inst) {
+        h->cur = parity;
+        h->steps += n;
+    }
+    b->steps += n;
+    return PLBM_OK;
+}
+
 // Groups the created instances and builds the groups' device tables.
 plbm_status batch_groups(Batch* b) {
     for (size_t i = 0; i < b->inst.size(); ++i) {
@@ -1623,72 +1692,7 @@ plbm_status plbm_batch_instance(plbm_batch bb, int i, plbm_handle* out) {
 }
 
 plbm_status plbm_batch_step(plbm_batch bb, long n, int mode) {
-    Batch* b = reinterpret_cast<Batch*>(bb);
-    if (!b || n < 0 || mode < 0 || mode > 3) {
-        batch_err(b, "bad arguments");
-        return PLBM_E_ARG;
-    }
-    const int parity0 = b->inst[0]->cur;
-    for (size_t i = 0; i < b->inst.size(); ++i) {
-        Handle* h = b->inst[i];
-        if (h->sticky != PLBM_OK || !h->initialised) {
-            batch_err(b, "instance %zu is not initialised or in an error state", i);
-            return PLBM_E_STATE;
-        }
-        if (h->cur != parity0) {
-            batch_err(b, "instance %zu was stepped on its own; all instances must be in step", i);
-            return PLBM_E_STATE;
-        }
-    }
-    BCK(cudaSetDevice(b->device));
-    const int scheme = (mode == PLBM_BATCH_PERSISTENT || mode == PLBM_BATCH_PERSISTENT_GRAPH) ? 0 : 1;
-    const bool use_graph = (mode == PLBM_BATCH_PERSISTENT_GRAPH || mode == PLBM_BATCH_PER_INSTANCE_GRAPH);
-    int parity = parity0;
-    long done = 0;
-    const int ctas = batch_ctas(b);  // occupancy query outside any stream capture
-    bool fused = false;              // runs of four steps, two per launch where a group can
-    for (const PairGroup& g : b->pairs) fused |= scheme == 0 && !g.pieces.empty();
-    if (fused && !use_graph)
-        for (; done + 4 <= n; done += 4) {
-            const plbm_status st = batch_launch4(b, parity, ctas);
-            if (st != PLBM_OK) return st;
-            b->launches += batch_launches(b, scheme, 4);
-        }
-    if (use_graph) {
-        while (done + 2 <= n) {
-            const int run = fused && done + 4 <= n ? 4 : 2;
-            cudaGraphExec_t& g = b->graph[run == 4 ? 2 : scheme][parity];
-            if (!g) {
-                cudaGraph_t graph = nullptr;
-                BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-                plbm_status st = run == 4 ? batch_launch4(b, parity, ctas) : batch_launch(b, scheme, parity, ctas);
-                if (st == PLBM_OK && run == 2) st = batch_launch(b, scheme, parity ^ 1, ctas);
-                cudaError_t ec = cudaStreamEndCapture(b->stream, &graph);
-                cudaError_t ei = (st == PLBM_OK && ec == cudaSuccess) ? cudaGraphInstantiate(&g, graph, 0)
-                                                                       : cudaSuccess;
-                if (graph) cudaGraphDestroy(graph);
-                if (st != PLBM_OK) return st;
-                BCK(ec);
-                BCK(ei);
-            }
-            BCK(cudaGraphLaunch(g, b->stream));
-            b->launches += batch_launches(b, scheme, run);
-            done += run;
-        }
-    }
-    for (; done < n; ++done) {
-        plbm_status st = batch_launch(b, scheme, parity, ctas);
-        if (st != PLBM_OK) return st;
-        b->launches += batch_launches(b, scheme, 1);
-        parity ^= 1;
-    }
-    if (n % 2) parity = parity0 ^ 1; else parity = parity0;
-    for (Handle* h : b->inst) {
-        h->cur = parity;
-        h->steps += n;
-    }
-    b->steps += n;
-    return PLBM_OK;
+    return batch_step(reinterpret_cast<Batch*>(bb), n, mode, true);
 }
 
 plbm_status plbm_batch_step_launches(plbm_batch bb, long long* launches) {
@@ -1795,10 +1799,10 @@ plbm_status plbm_batch_tune(plbm_batch bb, int steps_per_trial, int* best_block_
                 plbm_status st = plbm_batch_set_config(bb, bx, cps);
                 if (st == PLBM_OK) st = plbm_batch_set_order(bb, order);
                 if (st != PLBM_OK) return st;
-                st = plbm_batch_step(bb, 2, PLBM_BATCH_PERSISTENT);
+                st = batch_step(b, 2, PLBM_BATCH_PERSISTENT, false);
                 if (st != PLBM_OK) return st;
                 BCK(cudaEventRecord(e0, b->stream));
-                st = plbm_batch_step(bb, steps_per_trial, PLBM_BATCH_PERSISTENT);
+                st = batch_step(b, steps_per_trial, PLBM_BATCH_PERSISTENT, false);
                 if (st != PLBM_OK) return st;
                 BCK(cudaEventRecord(e1, b->stream));
                 BCK(cudaEventSynchronize(e1));

@@ -249,6 +249,25 @@ def test_batches_of_two_steps_per_launch_with_factors_that_are_no_powers_of_two(
                                                    (13, (0, 3, -3, 1, -1))]))
 
 
+def test_autotune_times_the_kernel_whose_shape_it_chooses():
+    # the shape and order are those of the single-step kernel; a group that takes two steps per launch in runs of four
+    # has to be timed by single steps all the same
+    b = B.Batch(_beyond_the_cache()[:-2], prec="f32")
+    b.init()
+    shapes = 0
+    for bx in (64, 128, 256):
+        b.set_config(bx, 0)
+        shapes += b.info()["max_ctas_per_sm"]
+    b.step(4, "persistent")
+    assert b.step_launches == 2
+    b.autotune(steps_per_trial=6)
+    assert b.step_launches == 2 + 2 * shapes * (2 + 6)   # two orders; two steps before each trial
+    b.step(4, "persistent")
+    assert b.step_launches == 4 + 2 * shapes * (2 + 6)
+    assert b.check()[0] == plbm.PLBM_OK
+    b.close()
+
+
 def test_full_sweep_sampled_nodes():
     # The bench's sweep (256 instances drawn by the R8 gates, sides over every
     # integer of [64, 1024], 1.0e8 nodes) in its timed launch scheme: after k steps a
