@@ -564,10 +564,10 @@ __global__ void __launch_bounds__(128) k_moments_f16pair(const __grid_constant__
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= P.nx) return;
     const __half2* at = reinterpret_cast<const __half2*>(f + elem_index(P, 0, x, y));
-    int2 S[5], T[5];
+    uint2 S[5], T[5];   // unsigned: sums modulo 2^32
     __half2 most = __float2half2_rn(0.0f);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) S[i] = T[i] = make_int2(0, 0);
+    for (int i = 0; i < 5; ++i) S[i] = T[i] = make_uint2(0u, 0u);
 #pragma unroll
     for (int i = 0; i < 5; ++i)
 #pragma unroll
@@ -575,10 +575,10 @@ __global__ void __launch_bounds__(128) k_moments_f16pair(const __grid_constant__
             const __half2 h = __ldg(at + (5 * i + j) * (P.plane / 2));
             most = __hmax2_nan(most, __habs2(h));
             const float2 g = add2(__half22float2(h), f2s(0.75f));
-            S[i].x += __float_as_int(g.x);
-            S[i].y += __float_as_int(g.y);
-            T[j].x += __float_as_int(g.x);
-            T[j].y += __float_as_int(g.y);
+            S[i].x += __float_as_uint(g.x);
+            S[i].y += __float_as_uint(g.y);
+            T[j].x += __float_as_uint(g.x);
+            T[j].y += __float_as_uint(g.y);
         }
     const float2 top = __half22float2(most);
     if (!(top.x < 0.25f && top.y < 0.25f)) {
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(128) k_moments_f16pair(const __grid_constant__
     const long long a = P.v[1], b = P.v[3];
 #pragma unroll
     for (int l = 0; l < 2; ++l) {
-        auto sum = [&](const int2& v) { return (long long)(int)((unsigned)(l ? v.y : v.x) - off); };
+        auto sum = [&](const uint2& v) { return (long long)(int)((l ? v.y : v.x) - off); };
         const long long sp = sum(S[1]) + sum(S[2]), sq = sum(S[3]) + sum(S[4]);
         const long long tp = sum(T[1]) + sum(T[2]), tq = sum(T[3]) + sum(T[4]);
         auto value = [](long long i) { return f64_of_fixed(i, 1056, false); };   // units of 2^-24

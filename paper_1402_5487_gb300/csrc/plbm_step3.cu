@@ -959,15 +959,15 @@ __global__ void __launch_bounds__(kB3) k_moments3_f16pair(const __grid_constant_
     if (x >= P.nx) return;
     const unsigned* at = reinterpret_cast<const unsigned*>(f + node3(P, x, y, z));
     const long long plane = P.plane / 2;
-    int2 S[kQ1], T[kQ1], U[kQ1];
+    uint2 S[kQ1], T[kQ1], U[kQ1];   // unsigned: sums modulo 2^32
     __half2 most = __float2half2_rn(0.0f);
 #pragma unroll
-    for (int i = 0; i < kQ1; ++i) S[i] = T[i] = U[i] = make_int2(0, 0);
+    for (int i = 0; i < kQ1; ++i) S[i] = T[i] = U[i] = make_uint2(0u, 0u);
 #pragma unroll
     for (int a = 0; a < kQ1; ++a)
 #pragma unroll
         for (int b = 0; b < kQ1; ++b) {
-            int2 R = make_int2(0, 0);
+            uint2 R = make_uint2(0u, 0u);
 #pragma unroll
             for (int c = 0; c < kQ1; ++c) {
                 const unsigned w = __ldg(at + ((a * kQ1 + b) * kQ1 + c) * plane);
@@ -975,7 +975,7 @@ __global__ void __launch_bounds__(kB3) k_moments3_f16pair(const __grid_constant_
                 memcpy(&h, &w, 4);
                 most = __hmax2_nan(most, __habs2(h));
                 const float2 g = add2(__half22float2(h), f2s(0.75f));
-                const int gx = __float_as_int(g.x), gy = __float_as_int(g.y);
+                const unsigned gx = __float_as_uint(g.x), gy = __float_as_uint(g.y);
                 R.x += gx;
                 R.y += gy;
                 U[c].x += gx;
@@ -995,9 +995,9 @@ __global__ void __launch_bounds__(kB3) k_moments3_f16pair(const __grid_constant_
     const long long va = P.v[1], vb = P.v[3];
 #pragma unroll
     for (int l = 0; l < 2; ++l) {
-        auto sum = [&](const int2& v) { return (long long)(int)((unsigned)(l ? v.y : v.x) - off); };
+        auto sum = [&](const uint2& v) { return (long long)(int)((l ? v.y : v.x) - off); };
         long long j[3], p = 0, q = 0, m = 0;
-        const int2* const axis[3] = {S, T, U};
+        const uint2* const axis[3] = {S, T, U};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const long long s1 = sum(axis[d][1]), s2 = sum(axis[d][2]), s3 = sum(axis[d][3]), s4 = sum(axis[d][4]);
