@@ -44,17 +44,20 @@ THETA0 = 1.0
 ELEM = {"f64": 8, "f32": 4, "f16dev": 2, "bf16dev": 2}
 
 
-KERNEL_NAME = {"f32": "k_two_steps<float2,96,2>", "f16dev": "k_two_steps<__half2,128,3>",
-               "bf16dev": "k_two_steps<__nv_bfloat162,128,3>", "f64": "k_stream_collide<double,5,2>"}
+#: step kernels of the (0, a, -a, 3, -3) lattices by (precision, even side): a step per launch and two
+KERNEL_NAME = {("f32", True): ("k_stream_collide_pair<float>", "k_two_steps<float2,96,2>"),
+               ("f16dev", True): ("k_stream_collide_pair2<__half>", "k_two_steps<__half2,128,3>"),
+               ("bf16dev", True): ("k_stream_collide_pair<__nv_bfloat16>", "k_two_steps<__nv_bfloat162,128,3>"),
+               ("f32", False): ("k_stream_collide_sym5<float>", "k_two_steps<float,128,3>"),
+               ("f16dev", False): ("k_stream_collide_sym5<__half>", "k_two_steps<__half,128,5>"),
+               ("bf16dev", False): ("k_stream_collide_sym5<__nv_bfloat16>", "k_two_steps<__nv_bfloat16,128,5>")}
 
 
-def launches(prec, L, steps):
-    """Step kernels that ``steps`` steps of the L x L lattice (even L) in one call launch: large
-    16/32-bit lattices take two steps a launch, in as many launches as steps modulo 2."""
-    if L < {"f32": 1024, "f16dev": 2048, "bf16dev": 2048}.get(prec, 1 << 30):
-        return steps
-    n = (steps + 1) // 2
-    return n + ((n ^ steps) & 1)
+def kernel_name(prec, L, launches, steps):
+    """The kernel that took ``steps`` steps of an L x L lattice in ``launches`` launches (the library's count)."""
+    if prec == "f64":
+        return "k_stream_collide<double,5,2>"
+    return KERNEL_NAME[prec, L % 2 == 0][launches < steps]
 
 
 def kernel_fingerprint(sources):
@@ -75,12 +78,14 @@ def kernel_fingerprint(sources):
     return h.hexdigest()
 
 
-def read_traffic(prec):
-    """DRAM bytes per launch from the committed ncu capture, or None when absent or
-    when the kernel's sources changed since the counters were taken."""
+def read_traffic(kernel, L):
+    """DRAM bytes per launch from the committed ncu capture of the L x L lattice, or None when
+    absent or when the kernel's sources changed since the counters were taken."""
     try:
         with open(os.path.join(ROOT, "profiles", "traffic.json")) as fh:
-            d = json.load(fh)[KERNEL_NAME[prec]]
+            d = json.load(fh)[kernel]
+        if not d["workload"].startswith("kh%d_" % L):
+            return None
         if kernel_fingerprint(d["kernel_sources"]) != d["kernel_sources_sha256"]:
             return None
         return float(d["bytes_per_launch"])
@@ -824,19 +829,21 @@ def main():
         e1 = torch.cuda.Event(enable_timing=True)
         torch.cuda.synchronize()
         barrier()
+        before = solver.step_launches
         e0.record(st)
         solver.step(args.steps)
         e1.record(st)
         e1.synchronize()
         torch.cuda.synchronize()
         barrier()
+        n_launches = solver.step_launches - before   # the same in every run
         runs.append(e0.elapsed_time(e1) * 1e-3)
     clock_info = clocks.stop()
     t = statistics.median(runs)
     healthy = solver.check() == 0
     solver.close()
     t_max, value = replica_throughput(torch, t, L * L * args.steps, dist)
-    n_launches = launches(args.prec, L, args.steps)
+    kernel = kernel_name(args.prec, L, n_launches, args.steps)
     per_launch = t / n_launches
     alg_bytes = 2 * q * ELEM[args.prec] * L * L
     peak, peak_kind = read_peaks()
@@ -891,11 +898,11 @@ def main():
                 "scaling": "weak", "vs_baseline": None, "dtype": args.prec, "data": "synthetic",
                 "config": config, "healthy": healthy,
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                             "frac": achieved / peak, "traffic": read_traffic(args.prec),
+                             "frac": achieved / peak, "traffic": read_traffic(kernel, L),
                              "peak_source": peak_kind + " (copy bandwidth, MEASURED_PEAKS.json hbm_gbs)",
                              "algorithmic_bytes_per_launch": alg_bytes,
                              "steps_per_launch": args.steps / n_launches,
-                             "kernel": KERNEL_NAME[args.prec]},
+                             "kernel": kernel},
                 "repeats": {"n": REPEATS, "reported": "median",
                             "ms_per_step_each": [r / args.steps * 1e3 for r in runs],
                             "spread": (max(runs) - min(runs)) / t},
