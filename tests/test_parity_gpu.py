@@ -786,6 +786,13 @@ def test_queued_steps_equal_awaited_steps(dim, v, shape, prec, kw):
     assert np.array_equal(got[0], got[1])
 
 
+# Small 16/32-bit lattices let the next grid start after their arithmetic (kernels of their own, in both layouts).
+@pytest.mark.parametrize("prec", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("shape", [(101, 97), (128, 128), (33, 5), (255, 255), (256, 254)])
+def test_queued_steps_of_small_lattices_equal_awaited_steps(prec, shape):
+    test_queued_steps_equal_awaited_steps(2, I.SET_013, shape, prec, {})
+
+
 # FP64 sums of five-velocity sets on the integer pipe: fields of given populations against exact
 # rational sums, over the exponent range and past both of its ends (there in FP64), with zeros,
 # negative values, a spread of 1e-9 and equal values.  A term is held to 2^-57 of the largest, a
@@ -857,6 +864,41 @@ def test_f64_rule_in_and_out_of_the_fixed_point_range(dim, iso, v):
 
 # Fields of FP16 pairs from exact 32-bit sums below 1/4 and in float-float from there on: as the 3D test of
 # the same; 25 roundings of 2^-53 of the sum of magnitudes.
+# The reciprocal of the FP64 steps and fields, through the velocity of nodes whose momentum is a power of two: within
+# half a unit of the last place and 2^-59 over the normal range, the division's value at and beyond its ends.
+def test_f64_reciprocal():
+    from fractions import Fraction
+    rng = np.random.default_rng(6)
+    rho = np.concatenate([rng.uniform(1, 2, 3000), -rng.uniform(1, 2, 200), 10.0 ** rng.uniform(-300, 300, 1000),
+                          [1.0, np.nextafter(1, 2), np.nextafter(1, 0), np.nextafter(2, 1), 1.5, 4 / 3],
+                          2.0 ** np.arange(-1021, -1015), 2.0 ** np.arange(1015, 1023),
+                          np.nextafter(2.0**-1021, 0) * np.ones(1), np.nextafter(2.0**1021, 0) * np.ones(1)])
+    odd = np.array([0.0, 5e-324, 2.0**-1030, -2.0**-1040, np.inf, -np.inf, np.nan, 1.7e308])
+    n = len(rho) + len(odd)
+    f = np.zeros((5, n))
+    with np.errstate(all="ignore"):
+        k = np.floor(np.log2(np.abs(rho))) - 20
+        f[1, :len(rho)] = 2.0 ** np.maximum(k, -1074)
+        f[0, :len(rho)] = rho - f[1, :len(rho)]
+        f[0, len(rho):] = odd
+        f[1, len(rho):] = 1.0 / 1024
+    s = plbm.Solver(1, I.SET_013, 1.1, n, 1, theta0=1.0, prec="f64")
+    s.init(np.ones((1, n)), np.zeros((1, n)), np.zeros((1, n)), np.ones((1, n)))
+    s.set_populations(f.reshape(5, 1, n))
+    m, u = (np.asarray(a).reshape(-1) for a in s.moments()[:2])
+    s.close()
+    with np.errstate(all="ignore"):
+        total = f[0] + f[1]
+        assert np.array_equal(m, total, equal_nan=True)
+        assert np.array_equal(u[len(rho):], f[1, len(rho):] * (1.0 / total[len(rho):]), equal_nan=True)
+    for r, j, v in zip(total[:len(rho)], f[1], u):
+        exact = Fraction(float(j)) / Fraction(float(r))
+        if abs(exact) < Fraction(2) ** -1000:
+            continue
+        err = abs(Fraction(float(v)) - exact)
+        assert err <= Fraction(float(np.spacing(abs(float(exact))))) / 2 + abs(exact) / 2**59, (r, j, v)
+
+
 # The FP64 rule of the symmetric sets in and out of the range of its fixed point: a fluid at rest stays exactly at
 # rest, and the mirrored flow is the flow, mirrored, bit for bit.  Sizes on both sides of the number of threads from
 # which the conversions are made by integer instructions.
