@@ -20,20 +20,15 @@
 // {0, +-1, +-2} 2048^2 120.9 and 78.6, 2047^2 123.4 and 83.2.
 // What bounds it: a warp's own latencies (1.5 warps a scheduler in pairs, 4.4 cycles from one
 // instruction to the next, a fifth of them waiting for loads); with all data in the second-level cache
-// 2048^2 takes 81 us a step, its traffic alone 65.  Measured slower there: a thread group for each of
-// the two phases (91-93), rows brought in by bulk copies (122 and more), loads two rows ahead
-// (91), bulk prefetches into the second-level cache (94), one node a thread in the paired
-// layout (93), both nodes of two columns a thread in the plain one (97).
+// 2048^2 takes 81 us a step, its traffic alone 65.
 //
 // 16-bit storage: the ring holds the rounded values that memory would, half the bytes, so that 12 warps
 // (pairs, 128 threads, three CTAs per SM) or 20 (plain) share an SM.  Their single steps are bound
 // by the SMs nearly as much as by memory; two at a time gain on large lattices: FP16 2048^2 67.7 and 63.7
-// (w = 2: 61.4), 4096^2 258 and 228, 4095^2 404 and 312, BF16 2048^2 67.7 and 65.9, 4096^2 261 and 236.  (At
-// 2048^2 FP16: 96 threads x 4 71, 64 x 6 65.5, 128 x 4 72.)
+// (w = 2: 61.4), 4096^2 258 and 228, 4095^2 404 and 312, BF16 2048^2 67.7 and 65.9, 4096^2 261 and 236.
 #pragma once
 
 #include <algorithm>
-#include <cstdlib>
 #include <type_traits>
 
 #include "plbm_pair.cuh"
@@ -261,8 +256,9 @@ k_two_steps(const __grid_constant__ PairParams P, const E* src, E* __restrict__ 
 // The lattices of a batch in one launch: CTA c takes piece c of the list, longest first (FusePiece,
 // plbm_internal.h).  Both layouts run on one shape of CTA, 96 threads and two resident: the plain one takes
 // two columns a thread (97 against 89 us a step at 2047^2, but no second launch with its own tail).
-// 16 lattices of 58 to 932 rows of pairs or nodes, 6.0 M nodes: 174 us a step by k_batch_pair, 120 here.
-template <int NT>
+// 16 lattices of 58 to 932 rows of pairs or nodes, 6.0 M nodes: 180 us a step by k_batch_pair, 139 here (122
+// with another batch's launches beside it to fill the tails).
+template <int NT>   // a template, as launch_batch_two_steps, to be compiled in the one unit that launches it
 __global__ void __launch_bounds__(NT, 2)
 k_batch_two_steps(const PairParams* __restrict__ inst, const FusePiece* __restrict__ pieces, int parity) {
     extern __shared__ __align__(16) unsigned char fuse_ring[];

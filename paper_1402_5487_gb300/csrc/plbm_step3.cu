@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
 // for 256 x 256 x 128 FP16 nodes.  Float-float pairs hi + lo (error-free sums and
 // products, ~2^-47 relative) on the deviations from the rest state, whose magnitude
 // is a hundredth of f's (so the absolute error stays at FP64's on f), take 404 / 236 us
-// and 1,234 / 754 us (388 by exact integer sums), bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
+// and 1,249 / 754 us (388 by exact integer sums), bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
 // the z-paired layout a thread takes both nodes of a pair (V = float2: packed FP32x2
 // arithmetic, one aligned 4-byte access for the two); otherwise one node (V = float).
 // ---------------------------------------------------------------------------
@@ -878,9 +878,6 @@ __device__ __forceinline__ double lane_f64(FFV<float2> v, int l) {
     return l ? ffv_f64(v.hi.y, v.lo.y) : ffv_f64(v.hi.x, v.lo.x);
 }
 
-// Row sums R_ab = sum_c g, S_a, T_b, U_c of the stored deviations, then
-// rho - 1 = sum S, j = sum v S (per axis), E - 3 theta0 = sum v^2 (S + T + U); the
-// fields of each node in FP64.
 // The fields of a node from rho - 1, j and E - 3 theta0.
 __device__ __forceinline__ void put_fields3(const LatticeParams& P, long long n, double dm, double jx, double jy, double jz, double de,
                                             double* rho, double* ux, double* uy, double* uz, double* theta) {
@@ -894,6 +891,9 @@ __device__ __forceinline__ void put_fields3(const LatticeParams& P, long long n,
     if (theta) theta[n] = ((3.0 * P.theta0 + de) * im - (a * a + b * b + c * c)) * (1.0 / 3.0);
 }
 
+// Row sums R_ab = sum_c g, S_a, T_b, U_c of the stored deviations, then
+// rho - 1 = sum S, j = sum v S (per axis), E - 3 theta0 = sum v^2 (S + T + U); the
+// fields of each node in FP64.
 template <typename S, class V>
 __device__ __forceinline__ void moments3_ff(const LatticeParams& P, const S* __restrict__ f, double* rho, double* ux, double* uy,
                                             double* uz, double* theta, int x, int y, int z) {
