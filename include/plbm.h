@@ -355,7 +355,7 @@ plbm_status plbm_batch_set_order(plbm_batch b, int order);
 /* Current order, or -1 for a NULL batch. */
 int plbm_batch_get_order(plbm_batch b);
 
-/* Current launch shape and the occupancy limit for it. */
+/* Current launch shape of the single-step kernel and the occupancy limit for it. */
 plbm_status plbm_batch_info(plbm_batch b, int *ninst, int *total_tiles, int *block_x, int *ctas,
                             int *max_ctas_per_sm);
 

@@ -602,7 +602,7 @@ __device__ __forceinline__ long long fixed_abs(double x, int n) {
 // 80-bit arithmetic, 200 steps of the 128^2 shear layer leave u_x 6e-15 and u_y 1.4e-13
 // off (DirectCore 1.3e-14, 2.3e-13), 40 of a 192^2 one 1.5e-15 and 2.8e-14 (3.8e-15, 6.1e-14).
 // Per step: 1024^2 D2Q25 414 us with DirectCore, 301 with all of this core in FP64, 206 with the
-// sums on the integer pipe, 154 now (127 of FP64 issue); 128^2 10.2, 7.95, 7.0, 6.7;
+// sums on the integer pipe, 152 now (the FP64 pipe busy for 0.79 of it, the integer one for 0.48); 128^2 10.2, 7.95, 7.0, 6.7;
 // the 1000-node D1Q5 tube 4.05 -> 3.2 us.  The identities sum r = 1, sum v^2 r = mu_2
 // hold by construction, so the global sums drift less: mean density of 1024^2 after
 // 40 steps 2e-16 off against 7e-15 (rounded C mu sums), energy 4e-16 against 5e-15.

@@ -544,7 +544,7 @@ cudaError_t launch_step_sym5_t(const LatticeParams& L, const void* src, void* ds
 }
 
 // Threads of a block without the reduction.  FP32: 64, whose slots refill in smaller pieces in the last wave (512^2,
-// 1.35 waves: 6.21 -> 5.96 us a step; 128, 96 and 32: 6.21, 6.05, 6.09), or 32 where that leaves
+// 1.35 waves: 6.21 -> 5.96 us a step, 5.70 since load_state; 128, 96 and 32: 6.21, 6.05, 6.09), or 32 where that leaves
 // an SM fewer than five blocks (256^2 3.03 -> 2.83 us).  BF16: 128, the seven CTAs of PairMinBlocks.
 template <typename S>
 int pair_block(const PairParams& P) {
