@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kB3) k_stream_collide3_f64q(const __grid_const
 // for 256 x 256 x 128 FP16 nodes.  Float-float pairs hi + lo (error-free sums and
 // products, ~2^-47 relative) on the deviations from the rest state, whose magnitude
 // is a hundredth of f's (so the absolute error stays at FP64's on f), take 404 / 236 us
-// and 1,249 / 754 us (388 by exact integer sums), bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
+// and 1,254 / 754 us (388 by exact integer sums), bounded by the FP32 pipe (the bytes alone: 167 and 358 us).  On
 // the z-paired layout a thread takes both nodes of a pair (V = float2: packed FP32x2
 // arithmetic, one aligned 4-byte access for the two); otherwise one node (V = float).
 // ---------------------------------------------------------------------------
@@ -661,6 +661,7 @@ __device__ __forceinline__ FFV<V> ffv_const(float2 c) { return {splat<V>(c.x), s
 struct Rule5FF {
     float2 w[kQ1], w2[kQ1 * kQ1];   // rest weights w_i and w_i w_j
     float2 th0, kOa, kOb, kEa, kEb;
+    double wab[kQ1 * kQ1];          // w_a w_b
 };
 float2 split_ff(double v) {
     const float hi = (float)v;
@@ -670,7 +671,10 @@ Rule5FF rule5_ff(const LatticeParams& P) {
     Rule5FF R;
     for (int i = 0; i < kQ1; ++i) {
         R.w[i] = split_ff(P.w1[i]);
-        for (int j = 0; j < kQ1; ++j) R.w2[i * kQ1 + j] = split_ff(P.w1[i] * P.w1[j]);
+        for (int j = 0; j < kQ1; ++j) {
+            R.wab[i * kQ1 + j] = P.w1[i] * P.w1[j];
+            R.w2[i * kQ1 + j] = split_ff(R.wab[i * kQ1 + j]);
+        }
     }
     const double a = P.v[1], b = P.v[3];
     R.th0 = split_ff(P.theta0);
@@ -725,10 +729,13 @@ __device__ __forceinline__ float round_ff(float hi, float lo, float d, bool& nea
 }
 
 // The populations of one node whose rounding the float-float arithmetic left open
-// (bit 5 b + c of open[a * stride]): f^eq_abc = rho r^x_a r^y_b r^z_c by the C mu rule in FP64.
+// (bit 5 b + c of open[a * stride]): f^eq_abc = rho r^x_a r^y_b r^z_c by the C mu rule in FP64.  Few in a flow,
+// all 125 in a fluid at rest, whose deviations are FP64's own rounding: w_a w_b comes from the host and rows without
+// any are passed over (128^3 FP32 at rest 2,775 -> 1,973 us, 256 x 256 x 128 FP16 12,300 -> 7,770, FP32
+// with |u| = 1e-3 1,603 -> 1,015).
 template <typename S>
-__device__ __noinline__ void init3_open(const LatticeParams& P, const unsigned* open, int stride, double rho, double ux,
-                                        double uy, double uz, double th, S* at) {
+__device__ __noinline__ void init3_open(const LatticeParams& P, const Rule5FF& R, const unsigned* open, int stride, double rho,
+                                        double ux, double uy, double uz, double th, S* at) {
     double ra[kQ1], rb[kQ1], rc[kQ1];
     rule_q<kQ1>(P, ux, th, ra);
     rule_q<kQ1>(P, uy, th, rb);
@@ -740,12 +747,14 @@ __device__ __noinline__ void init3_open(const LatticeParams& P, const unsigned* 
         const double ra1 = rho * ra[a];
 #pragma unroll
         for (int b = 0; b < kQ1; ++b) {
+            if (!((m >> (kQ1 * b)) & 31u)) continue;
             const double X = ra1 * rb[b];
 #pragma unroll
             for (int c = 0; c < kQ1; ++c)
                 if ((m >> (kQ1 * b + c)) & 1u) {
                     const int p = (a * kQ1 + b) * kQ1 + c;
-                    at[(long long)p * P.plane] = Storage<S>::from_f64(__dmul_rn(X, rc[c]), w0_3(P, p));   // f^eq rounded before the difference
+                    // f^eq rounded before the difference, w_a w_b w_c not
+                    at[(long long)p * P.plane] = Storage<S>::from_f64(fma(-R.wab[kQ1 * a + b], P.w1[c], __dmul_rn(X, rc[c])), 0.0);
                 }
         }
     }
@@ -867,7 +876,7 @@ __global__ void __launch_bounds__(kB3) k_init3_dev(const __grid_constant__ Latti
     for (int l = 0; l < kLanes; ++l) {
         if (!(l ? any[1] : any[0])) continue;
         const long long n = ((long long)(z + l * P.half_nz) * P.ny + y) * P.nx + x;
-        init3_open<S>(P, &sOpen[l][0][t], kB3, rho[n], ux[n], uy[n], uz[n], theta[n], f + node3(P, x, y, z) + l);
+        init3_open<S>(P, R, &sOpen[l][0][t], kB3, rho[n], ux[n], uy[n], uz[n], theta[n], f + node3(P, x, y, z) + l);
     }
 }
 

@@ -259,6 +259,34 @@ def test_d3q125_initial_state_and_fields_to_the_last_bit_of_storage(prec, shape,
         assert np.max(np.abs(a - b)) <= 3e-14
 
 
+# At and near rest the float-float arithmetic leaves most roundings, or all, to the FP64 rule (a row of five
+# populations at a time): a fluid at rest, one with a jump in density, weak noise, and rest beside a flow.
+@pytest.mark.parametrize("prec,nz", [("f32", 5), ("f16dev", 6), ("f16dev", 5), ("bf16dev", 6)])
+@pytest.mark.parametrize("kind", ["rest", "jump", "1e-6", "1e-3", "beside"])
+def test_d3q125_initial_state_at_and_near_rest(prec, nz, kind):
+    from paper_1402_5487_gb300 import plbm
+    nx, ny = 131, 3
+    rng = np.random.default_rng(12)
+    one = np.ones((nz, ny, nx))
+    rho, th, u = one.copy(), one.copy(), [0 * one for _ in range(3)]
+    if kind == "jump":
+        rho[:, :, :nx // 2] = 1.125
+    elif kind == "beside":
+        u = [0.1 * rng.uniform(-1, 1, one.shape) * (rng.uniform(0, 1, one.shape) < 0.3) for _ in range(3)]
+    elif kind != "rest":
+        u = [float(kind) * rng.uniform(-1, 1, one.shape) for _ in range(3)]
+    lat = O.Lattice3(V5, 1.2, nx, ny, nz, theta0=1.0)
+    want = lat.init(rho, *u, th).reshape(125, nz, ny, nx)
+    w0 = lat.init(one, 0 * one, 0 * one, 0 * one, one).reshape(125, nz, ny, nx)
+    s = plbm.Solver(3, V5, 1.2, nx, ny, nz=nz, theta0=1.0, prec=prec)
+    s.init(rho, u[0], u[1], th, uz=u[2])
+    got = s.get_populations().reshape(125, nz, ny, nx)
+    s.close()
+    bits, low = {"f32": (24, -149), "f16dev": (11, -24), "bf16dev": (8, -133)}[prec]
+    ulp = np.exp2(np.maximum(np.frexp(np.maximum(np.abs(want - w0), 1e-300))[1] - bits, low))
+    assert np.all(np.abs(got - want) <= 0.5 * ulp * (1 + 1e-6) + 4e-16)
+
+
 # Fields of FP16 pairs from exact 32-bit sums below 1/4 and in float-float from there on (and beside
 # non-finite values): random deviations with none, one at either edge, and large ones; sums of the
 # stored populations, 125 roundings of 2^-53 of the sum of magnitudes.
