@@ -27,6 +27,11 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <map>
+#include <mutex>
+#include <type_traits>
+#include <utility>
+
 #include "plbm_internal.h"
 
 namespace plbm {
@@ -41,11 +46,20 @@ namespace plbm {
 // waits for the grid before to be complete and flushed (step_wait) first.  A
 // kernel launched without the attribute passes both at once.  Per step: 2048^2 FP32
 // 123.2 -> 120.6 us, FP16 69.7 -> 67.3 us, 512^2 FP32 (graph) 6.56 -> 6.29 us.
-// Grids of fewer than kDependentThreads threads leave slots free for several
-// waiting grids at once, which then crowd the running one (128^2 FP64: 10.2 ->
-// 16.4 us a step): FP64 kernels (step_end; 128^2 8.35 -> 7.95 us a step, tube launches of
-// four steps 8.1 -> 7.6 us) and 16/32-bit ones of five-velocity sets (LATE, plbm_pair.cuh) then
-// say so only after their arithmetic, others are launched plainly.  The persistent batch
+// The same trigger does harm where the chip holds the whole grid: the slots it leaves free
+// then fill with waiting blocks of the next grids, which crowd it and leave their own
+// work unevenly spread over the SMs.  Measured against plain launches over 700 drawn 16/32-bit and 500 drawn
+// FP64 lattices (time as a dependent over time launched plainly, median and range; "waves": blocks over resident blocks):
+//   16/32-bit 2D   below 0.1 waves 0.86-0.91; 0.1-0.83 1.2 (0.84-1.51); above 0.87 (0.69-1.05)
+//     the trigger after the arithmetic (LATE, plbm_pair.cuh): below 0.4 0.93 (0.89-1.03), 0.4-1.5 1.02 (0.94-1.12)
+//   16/32-bit 3D   0.83 (0.63-1.03), whatever the waves
+//   FP64 2D        0.1-0.8 waves 1.45 (0.97-2.25), 0.8-3 1.00 (0.94-1.27), above 0.99 (0.95-1.01); after the arithmetic
+//     with blocks of 32 threads and up to five velocities 0.98 (0.95-0.99), otherwise 1.00 (0.95-1.28)
+//   FP64 3D        0.15-3 waves 1.24 (0.85-2.76), above 0.99 (0.97-1.00)
+// Hence: the trigger at the start from 5/6 of a wave on (FP64: three waves), after the arithmetic where that gains
+// always, plainly otherwise; 3D 16/32-bit grids from kDependentThreads threads on.  Of 530 lattices drawn between 2.5e4
+// and 9e5 nodes 5 are then more than 2 % slower than plainly, 1.12 at worst and 0.93 on average (with the trigger at
+// the start from 65,536 threads on: 87, 1.46, 0.96).  The persistent batch
 // kernels, which leave no slot free, are launched plainly (174 us a step either way).
 // ---------------------------------------------------------------------------
 constexpr long long kDependentThreads = 1 << 16;
@@ -80,17 +94,44 @@ __device__ __forceinline__ T load_state(const T* p) {
     }
     return v;
 }
-// FP64 kernels: the trigger at the start of a grid of more than one wave whatever the
-// registers (2^18 threads and up), after the arithmetic of a smaller one.
-__device__ __forceinline__ bool step_large() {
-    return (long long)gridDim.x * gridDim.y * gridDim.z * blockDim.x >= 1 << 18;
+// FP64 kernels of 1D lattices and of blocks of 32 threads: the trigger after the arithmetic.
+template <int DIM>
+__device__ __forceinline__ bool step_late() {
+    return DIM == 1 ? (long long)gridDim.x * blockDim.x < 1 << 18 : blockDim.x == 32;
 }
-__device__ __forceinline__ void step_end() {
-    if (!step_large()) step_begin();
+
+inline int device_sm_count() {
+    static int n = 0;
+    if (!n) {
+        int d = 0;
+        cudaGetDevice(&d);
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d) != cudaSuccess || n < 1) n = 1;
+    }
+    return n;
+}
+
+// Whether `threads` threads with work fill the resident blocks of `kernel` num / den times at least (the occupancy is
+// asked for once per kernel and block size).  Idle threads of a row's last block do not count: 38 x 2152 BF16
+// (1.01 waves of blocks, 0.3 of threads) takes 4.3 us a step as a dependent and 3.7 plainly.
+inline bool grid_waves(const void* kernel, long long threads, int block, int num, int den) {
+    static std::mutex lock;
+    static std::map<std::pair<const void*, int>, int> known;   // resident blocks per SM
+    int per_sm;
+    {
+        std::lock_guard<std::mutex> g(lock);
+        auto it = known.find({kernel, block});
+        if (it == known.end()) {
+            int n = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, 0) != cudaSuccess || n < 1) n = 1;
+            it = known.emplace(std::make_pair(kernel, block), n).first;
+        }
+        per_sm = it->second;
+    }
+    return threads * den >= (long long)per_sm * block * device_sm_count() * num;
 }
 
 template <class... P, class... A>
-cudaError_t launch_dependent_smem(bool small_too, size_t smem, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream,
+cudaError_t launch_dependent_smem(bool dependent, size_t smem, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream,
                                   A... args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -101,12 +142,19 @@ cudaError_t launch_dependent_smem(bool small_too, size_t smem, void (*kernel)(P.
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = &attr;
-    cfg.numAttrs = small_too || (long long)grid.x * grid.y * grid.z * block.x >= kDependentThreads ? 1 : 0;
+    cfg.numAttrs = dependent ? 1 : 0;   // otherwise plainly
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 template <class... P, class... A>
-cudaError_t launch_dependent(bool small_too, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
-    return launch_dependent_smem(small_too, 0, kernel, grid, block, stream, args...);
+cudaError_t launch_dependent(bool dependent, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args) {
+    return launch_dependent_smem(dependent, 0, kernel, grid, block, stream, args...);
+}
+// A kernel that triggers at its start: as a dependent from num / den waves on.
+template <class... P, class... A>
+cudaError_t launch_by_waves(long long threads, int num, int den, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream,
+                            A... args) {
+    return launch_dependent(grid_waves(reinterpret_cast<const void*>(kernel), threads, block.x, num, den), kernel, grid, block,
+                            stream, args...);
 }
 
 // ---------------------------------------------------------------------------
@@ -931,7 +979,7 @@ __device__ __forceinline__ void node_update(const LatticeParams& P, const S* src
         }
         if (!sym5) DirectCore<Q1, DIM>::collide(f, P, rho, th, jx, jy, e);
         flag_status_f64(P, rho, th);
-        step_end();
+        if (step_late<DIM>()) step_begin();
         if (REDUCE) {
             d.mass = rho;
             d.jx = jx;
@@ -986,7 +1034,7 @@ __device__ __forceinline__ void node_update(const LatticeParams& P, const S* src
 template <typename S, int Q1, int DIM, bool REDUCE>
 __global__ void __launch_bounds__(kBlockX)
 k_stream_collide(const __grid_constant__ LatticeParams P, const S* src, S* __restrict__ dst) {
-    if (sizeof(S) < 8 || step_large()) step_begin();
+    if (sizeof(S) < 8 || !step_late<DIM>()) step_begin();
     const int x = blockIdx.x * (REDUCE ? kBlockX : (int)blockDim.x) + threadIdx.x;
     const int y = blockIdx.y;
     step_wait();
@@ -1086,7 +1134,7 @@ __global__ void __launch_bounds__(32 * kWarps1) k_steps1(const __grid_constant__
             for (int i = 0; i < Q1; ++i) f[i] = Node1<S>::stored(g[i]);
         }
     }
-    step_begin();   // after the arithmetic, as in step_end
+    step_begin();   // after the arithmetic
     if (inside && lane >= w * steps && lane < w * steps + m) {
 #pragma unroll
         for (int i = 0; i < Q1; ++i) Storage<S>::store(dst + i * P.plane + x, f[i]);
@@ -1152,16 +1200,6 @@ k_batch_node(const LatticeParams* __restrict__ inst, const NodeSpan* __restrict_
     }
 }
 
-inline int device_sm_count() {
-    static int n = 0;
-    if (!n) {
-        int d = 0;
-        cudaGetDevice(&d);
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, d) != cudaSuccess || n < 1) n = 1;
-    }
-    return n;
-}
-
 template <typename S>
 cudaError_t launch_step_t(const LatticeParams& P, const void* src, void* dst, bool reduce,
                           cudaStream_t stream) {
@@ -1177,8 +1215,10 @@ cudaError_t launch_step_t(const LatticeParams& P, const void* src, void* dst, bo
     S* t = static_cast<S*>(dst);
 #define PLBM_LAUNCH(Q1v, DIMv)                                                              \
     if (P.q1 == Q1v && P.dim == DIMv) {                                                     \
-        return reduce ? launch_dependent(f64, k_stream_collide<S, Q1v, DIMv, true>, grid, block, stream, P, s, t)    \
-                      : launch_dependent(f64, k_stream_collide<S, Q1v, DIMv, false>, grid, block, stream, P, s, t);  \
+        const auto kernel = reduce ? k_stream_collide<S, Q1v, DIMv, true> : k_stream_collide<S, Q1v, DIMv, false>;  \
+        if (f64 && (DIMv == 1 || bx == 32))                                                                        \
+            return launch_dependent(DIMv == 1 || Q1v <= 5, kernel, grid, block, stream, P, s, t);                  \
+        return launch_by_waves((long long)P.nx * P.ny, f64 ? 3 : 5, f64 ? 1 : 6, kernel, grid, block, stream, P, s, t); \
     }
     PLBM_LAUNCH(3, 1)
     PLBM_LAUNCH(4, 1)

@@ -522,10 +522,13 @@ k_stream_collide_pair(const __grid_constant__ PairParams P, const typename PairS
     }
 }
 
-// LATE: grids of fewer than kDependentThreads threads let the next one start after their
-// arithmetic (as FP64 grids do): 128^2 FP32 2.19 -> 1.99 us a step, 256^2 2.83 -> 2.76.  A kernel of its own, as a
+// LATE: grids of fewer than 0.4 waves let the next one start after their arithmetic (as FP64 blocks of 32
+// threads do): 128^2 FP32 2.19 -> 1.99 us a step, 256^2 2.83 -> 2.69.  A kernel of its own, as a
 // test at the start of the others costs 512^2 1 and 511^2 7 %.
-inline bool step_few(dim3 grid, int bx) { return (long long)grid.x * grid.y * bx < kDependentThreads; }
+template <class K>
+bool step_few(K* late, long long threads, int bx) {
+    return !grid_waves(reinterpret_cast<const void*>(late), threads, bx, 2, 5);
+}
 
 // Plain-layout symmetric five-velocity lattices (odd ny, or PLBM_FLAG_PLAIN_LAYOUT):
 // one node per thread; small lattices take 32-thread blocks (more SMs busy).
@@ -538,9 +541,11 @@ cudaError_t launch_step_sym5_t(const LatticeParams& L, const void* src, void* ds
     dim3 grid((P.nx + bx - 1) / bx, P.ny);
     const S* s = static_cast<const S*>(src);
     S* t = static_cast<S*>(dst);
-    if (!reduce && step_few(grid, bx)) return launch_dependent(true, k_stream_collide_sym5<S, false, true>, grid, bx, stream, P, s, t);
-    return reduce ? launch_dependent(false, k_stream_collide_sym5<S, true>, grid, kBlockX, stream, P, s, t)
-                  : launch_dependent(false, k_stream_collide_sym5<S, false>, grid, bx, stream, P, s, t);
+    const auto late = k_stream_collide_sym5<S, false, true>;
+    const long long threads = (long long)P.nx * P.ny;
+    if (!reduce && step_few(late, threads, bx)) return launch_dependent(true, late, grid, bx, stream, P, s, t);
+    return launch_by_waves(threads, 5, 6, reduce ? k_stream_collide_sym5<S, true> : k_stream_collide_sym5<S, false>, grid, bx, stream,
+                           P, s, t);
 }
 
 // Threads of a block without the reduction.  FP32: 64, whose slots refill in smaller pieces in the last wave (512^2,
@@ -559,19 +564,21 @@ cudaError_t launch_step_pair_t(const LatticeParams& L, const void* src, void* ds
     const PairParams P = pair_params(L);
     const int bx = reduce ? kBlockX : pair_block<S>(P);
     dim3 grid((P.nx + bx - 1) / bx, P.half_ny);
+    const long long threads = (long long)P.nx * P.half_ny;
     const V* s = static_cast<const V*>(src);
     V* t = static_cast<V*>(dst);
     if constexpr (std::is_same<S, __half>::value) {
         if (!reduce) {
             const int tiles_x = (P.nx + kPair2Block - 1) / kPair2Block;
             const int ntiles = tiles_x * P.half_ny;
-            return launch_dependent(false, k_stream_collide_pair2<S>, (ntiles + 1) / 2, kPair2Block, stream, P, s, t, tiles_x,
+            return launch_by_waves(threads / 2, 5, 6, k_stream_collide_pair2<S>, (ntiles + 1) / 2, kPair2Block, stream, P, s, t, tiles_x,
                                     ntiles);
         }
     }
-    if (!reduce && step_few(grid, bx)) return launch_dependent(true, k_stream_collide_pair<S, false, true>, grid, bx, stream, P, s, t);
-    return reduce ? launch_dependent(false, k_stream_collide_pair<S, true>, grid, kBlockX, stream, P, s, t)
-                  : launch_dependent(false, k_stream_collide_pair<S, false>, grid, bx, stream, P, s, t);
+    const auto late = k_stream_collide_pair<S, false, true>;
+    if (!reduce && step_few(late, threads, bx)) return launch_dependent(true, late, grid, bx, stream, P, s, t);
+    return launch_by_waves(threads, 5, 6, reduce ? k_stream_collide_pair<S, true> : k_stream_collide_pair<S, false>, grid, bx, stream,
+                           P, s, t);
 }
 
 // ---------------------------------------------------------------------------

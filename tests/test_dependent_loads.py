@@ -45,8 +45,9 @@ def test_every_dependent_kernel_is_found():
              for _, s, _ in dependent_kernels()}
     launched = set()
     for f in CSRC.glob("*.cu*"):
-        launched |= set(re.findall(r"launch_dependent(?:_smem)?\([^,]+?,(?:\s*[\w.]+,)?\s*(k_\w+)", code(f.name)))
-    assert len(names) >= 10 and launched <= names, launched - names
+        for call in re.findall(r"launch_(?:dependent|dependent_smem|by_waves|large)\([^;]*;", code(f.name)):
+            launched |= set(re.findall(r"\bk_\w+", call))
+    assert len(names) >= 10 and len(launched) >= 8 and launched <= names, launched - names
 
 
 @pytest.mark.parametrize("name", ["plbm_device.cuh", "plbm_pair.cuh", "plbm_fuse.cuh"])

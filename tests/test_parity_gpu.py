@@ -793,6 +793,17 @@ def test_queued_steps_of_small_lattices_equal_awaited_steps(prec, shape):
     test_queued_steps_equal_awaited_steps(2, I.SET_013, shape, prec, {})
 
 
+# Lattices between the sizes at which one step's start overlaps the step before: launched plainly, with a row's
+# last block nearly empty, and FP64 grids of one and three waves.
+@pytest.mark.parametrize("dim,v,shape,prec,kw", [
+    (2, I.SET_013, (360, 360), "f32", {}), (2, I.SET_013, (360, 360), "f16dev", {}), (2, I.SET_013, (360, 360), "bf16dev", {}),
+    (2, I.SET_013, (430, 377), "bf16dev", {}), (2, I.SET_013, (38, 2152), "bf16dev", {}), (2, I.SET_013, (300, 301), "f32", {}),
+    (2, I.SET_D1Q3, (405, 134), "f16dev", {"theta0": 1 / 3, "isothermal": True}), (2, I.SET_013, (119, 456), "f64", {}),
+    (2, (0, 1, -1, 2, -2, 3, -3), (60, 50), "f64", {"theta0": 0.8}), (3, I.SET_013, (32, 32, 32), "f64", {}), (3, I.SET_013, (64, 64, 64), "f64", {})])
+def test_queued_steps_between_the_launch_rules_equal_awaited_steps(dim, v, shape, prec, kw):
+    test_queued_steps_equal_awaited_steps(dim, v, shape, prec, kw)
+
+
 # FP64 sums of five-velocity sets on the integer pipe: fields of given populations against exact
 # rational sums, over the exponent range and past both of its ends (there in FP64), with zeros,
 # negative values, a spread of 1e-9 and equal values.  A term is held to 2^-57 of the largest, a
