@@ -101,22 +101,27 @@ cudaError_t launch_step(int prec, const LatticeParams& P, const void* src, void*
 // constants are fitted to D1Q5 {0, +-1, +-3}, periodic, us per step with one step per
 // launch (graph replays) and with the k this rule takes: FP64 1000 nodes 4.04 (3.2
 // before the symmetric core alone) -> 1.87, 20,000 nodes 5.46 -> 3.54, 100,000 nodes
-// 18.95 -> 14.70 (k = 1); FP32 1.74 -> 0.53, 1.87 -> 0.91, 2.32 -> 1.55.
+// 18.95 -> 14.70 (k = 1); FP32 1.74 -> 0.53, 1.87 -> 0.91, 2.32 -> 1.55.  Of 420 drawn lattices (16 to 4 * 10^6 nodes,
+// three to eight velocities of up to 7) none is then more than 7 % slower than by single steps and the mean is 0.57 of them
+// (with one pair of constants for all numbers of velocities 1.33 at worst: eight velocities, 2.8 * 10^6 nodes).
 int steps_per_launch(int prec, const LatticeParams& P) {
     if (P.dim != 1)   // plbm_fuse.cuh
         return (prec == kF32 && two_steps_f32(P)) || (prec == kF16Dev && two_steps_f16(P)) || (prec == kBF16Dev && two_steps_bf16(P)) ? 2 : 1;
     const int w = halo1(P), sms = device_sm_count();
     const double launch = 1.5, latency = prec == kF64 ? 1.5 : 0.25;
+    // a round of FP32 arithmetic by the number of velocities, in k_stream_collide and in k_steps1 (80 rounds and more)
+    static const double single[6] = {0.173, 0.183, 0.207, 0.269, 0.316, 0.364}, several[6] = {0.093, 0.109, 0.129, 0.153, 0.186, 0.214};
     auto time = [&](int k) {   // per step
         const int m = k == 1 ? 32 : 32 - 2 * w * k;
         const long long warps = (P.nx + m - 1) / m, rounds = (warps + 4LL * sms - 1) / (4LL * sms);
-        const double work = rounds * (prec == kF64 ? 1.5 : k > 1 ? 0.09 : 0.19);   // k = 1: k_stream_collide
+        const double round = prec == kF64 ? 1.5 : k == 1 ? single[P.q1 - 3] : several[P.q1 - 3] * (rounds < 80 ? 0.75 + rounds / 320.0 : 1.0);
+        const double work = rounds * round;
         const double step = work > latency ? work : latency;
         return (launch + k * step) / k;
     };
     int best = 1;
     for (int k = 2; k <= 16 && 32 - 2 * w * k >= 2; k *= 2)   // divisors of half a captured run of 32 steps
-        if (time(k) < time(best)) best = k;
+        if (time(k) < (best == 1 ? 0.95 : 1.0) * time(best)) best = k;
     return best;
 }
 

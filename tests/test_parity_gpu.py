@@ -1124,6 +1124,21 @@ def test_step_launches_counts_what_was_launched():
     assert plbm.lib().plbm_step_launches(None, None) == plbm.PLBM_E_ARG
 
 
+# Several steps per launch of a 1D lattice cost more arithmetic, the more the wider the velocities: long lattices with
+# |v| = 4 and more take single steps, short ones never do.
+@pytest.mark.parametrize("prec", ["f32", "bf16dev"])
+@pytest.mark.parametrize("v,n,single", [((0, 1, -1, 2, -4), 2000000, True), ((1, -1, 2, -2, 3, -3, 4, -4), 2000000, True),
+                                        ((0, 1, -1), 2000000, False), ((1, -1, 2, -2, 3, -3, 4, -4), 1000, False), (I.SET_013, 1000, False)])
+def test_1d_steps_per_launch_by_velocities(prec, v, n, single):
+    from paper_1402_5487_gb300 import plbm
+    one = np.ones((1, n))
+    s = plbm.Solver(1, v, 1.1, n, 1, theta0=1.0, prec=prec, skip_admissibility=True)
+    s.init(one, 0 * one, 0 * one, one)
+    s.step(16)
+    assert (s.step_launches == 16) == single
+    s.close()
+
+
 # Two lattices whose rings differ in size (w = 2 and 3), stepped by two threads on streams of their own.
 @pytest.mark.parametrize("prec", ["f32", "f16dev"])
 def test_two_steps_of_one_launch_from_two_threads(prec):
