@@ -751,6 +751,22 @@ def test_layouts_give_the_same_state_for_factors_that_are_no_powers_of_two(prec,
         assert bool(np.isfinite(a).all()) and bool(np.array_equal(a, b)), (k, np.mean(a != b))
 
 
+# Blocks of 64 and 128 threads of the plain layout, by the columns of a row's last block, against the paired layout.
+@pytest.mark.parametrize("prec", ["f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("nx", [20, 32, 33, 64, 65, 128, 130, 192, 193])
+def test_plain_layout_blocks_give_the_paired_state(prec, nx):
+    ny = 512
+    fields = I.kh_fields(nx, ny=ny)
+    out = []
+    for plain in (False, True):
+        s = plbm.Solver(2, V5, 1.3, nx, ny, theta0=1.0, prec=prec, plain_layout=plain)
+        s.init(*fields)
+        s.step(5)
+        out.append(s.get_populations())
+        s.close()
+    assert bool(np.array_equal(out[0], out[1]))
+
+
 # Steps queued back to back (large grids overlap one step's start with the end of the
 # step before; small ones do not) equal steps awaited one by one, bit for bit: every
 # step kernel, on both sides of the size from which its launches overlap.
