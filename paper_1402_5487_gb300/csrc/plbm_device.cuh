@@ -112,7 +112,8 @@ inline int device_sm_count() {
 
 // Whether `threads` threads with work fill the resident blocks of `kernel` num / den times at least (the occupancy is
 // asked for once per kernel and block size).  Idle threads of a row's last block do not count: 38 x 2152 BF16
-// (1.01 waves of blocks, 0.3 of threads) takes 4.3 us a step as a dependent and 3.7 plainly.
+// (1.01 waves of blocks, 0.3 of threads) takes 4.3 us a step as a dependent and 3.7 plainly.  (FP64 grids, whose rule asks
+// for three waves, count them.)
 inline bool grid_waves(const void* kernel, long long threads, int block, int num, int den) {
     static std::mutex lock;
     static std::map<std::pair<const void*, int>, int> known;   // resident blocks per SM
@@ -1218,7 +1219,8 @@ cudaError_t launch_step_t(const LatticeParams& P, const void* src, void* dst, bo
         const auto kernel = reduce ? k_stream_collide<S, Q1v, DIMv, true> : k_stream_collide<S, Q1v, DIMv, false>;  \
         if (f64 && (DIMv == 1 || bx == 32))                                                                        \
             return launch_dependent(DIMv == 1 || Q1v <= 5, kernel, grid, block, stream, P, s, t);                  \
-        return launch_by_waves((long long)P.nx * P.ny, f64 ? 3 : 5, f64 ? 1 : 6, kernel, grid, block, stream, P, s, t); \
+        return launch_by_waves(f64 ? (long long)grid.x * grid.y * bx : (long long)P.nx * P.ny, f64 ? 3 : 5, f64 ? 1 : 6, kernel,  \
+                               grid, block, stream, P, s, t);                                                      \
     }
     PLBM_LAUNCH(3, 1)
     PLBM_LAUNCH(4, 1)

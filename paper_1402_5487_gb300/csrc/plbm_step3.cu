@@ -1320,11 +1320,12 @@ cudaError_t launch_step3(int prec, const LatticeParams& P, const void* src, void
     if (prec == kF64) {
         const double* a = static_cast<const double*>(src);
         double* b = static_cast<double*>(dst);
-        const long long nodes = (long long)P.nx * P.ny * P.nz;
+        const dim3 g = grid3(P);
+        const long long threads = (long long)g.x * g.y * g.z * kB3;
         switch (P.q1) {   // 32^3 D3Q125: 53 us a step plainly, 132 as a dependent
-            case 5: return launch_by_waves(nodes, 3, 1, k_stream_collide3_f64q<5>, grid3(P), kB3, s, P, a, b);
-            case 4: return launch_by_waves(nodes, 3, 1, k_stream_collide3_f64q<4>, grid3(P), kB3, s, P, a, b);
-            case 3: return launch_by_waves(nodes, 3, 1, k_stream_collide3_f64q<3>, grid3(P), kB3, s, P, a, b);
+            case 5: return launch_by_waves(threads, 3, 1, k_stream_collide3_f64q<5>, g, kB3, s, P, a, b);
+            case 4: return launch_by_waves(threads, 3, 1, k_stream_collide3_f64q<4>, g, kB3, s, P, a, b);
+            case 3: return launch_by_waves(threads, 3, 1, k_stream_collide3_f64q<3>, g, kB3, s, P, a, b);
         }
         return cudaErrorInvalidValue;
     }
